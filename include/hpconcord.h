@@ -121,7 +121,10 @@ typedef struct {
                                loop                                                    */
     int32_t device_loop;    /* 1 (default): the iteration and line-search loops run on
                                the device, one CUDA-graph launch per solve (conditional
-                               WHILE nodes); 0: the host drives every iteration       */
+                               WHILE nodes); 0: the host drives every iteration.  Cov
+                               handles with 384 rows or more (and fused_tail 0): the
+                               iterations run in one cooperative kernel, per solve or,
+                               with 0, per iteration                                  */
     int32_t reserved_;
 } hpc_options;
 
@@ -466,20 +469,21 @@ typedef struct {
                                   window with its decision, compaction and stopping
                                   rule -- run as one cooperative kernel, grid-wide
                                   barriers between the steps; 0: as the chain of
-                                  separate kernels.  The same entries and decisions
-                                  either way (the windows' partial sums are grouped
-                                  by the line-search grid in both).  On GB300 the two
-                                  take the same time to within a few percent (a
-                                  barrier costs about a kernel boundary inside the
-                                  solve's CUDA graph); the chain is faster where the
-                                  candidate structure is large, and where other
-                                  streams run kernels during the solve (a cooperative
-                                  kernel waits until its whole grid is resident: it
-                                  queues behind hpc_prefetch_x's transpose).  Not
-                                  touched by the autotuner.  hpc_solve_batch's single
-                                  graph launch runs its problems' loops concurrently,
-                                  always on the chain; handles solved from its worker
-                                  threads keep their own setting (0)               */
+                                  separate kernels, or, for the Cov variant from 384
+                                  rows on, all iterations in one cooperative kernel
+                                  (three barriers per iteration; the chain then runs
+                                  only the iterations in which a row has more than
+                                  2046 candidates).  The same entries and decisions
+                                  every way (the line search's sums are grouped
+                                  differently, which moves F in its last bits and a
+                                  decision only at an exact tie).  Where only the tail
+                                  differs the two forms take the same time to within a
+                                  few percent.  A cooperative kernel waits until its
+                                  whole grid is resident.  Not touched by the
+                                  autotuner.  hpc_solve_batch's single graph launch
+                                  runs its problems' loops concurrently, always on the
+                                  chain; handles solved from its worker threads keep
+                                  their own setting (0)                            */
 } hpc_tuning;
 
 /* The bound screening's block maxima of the Cov variant: out[i * nb + jb] = max

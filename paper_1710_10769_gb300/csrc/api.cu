@@ -161,6 +161,10 @@ struct hpc_ctx {
     int64_t g_epoch = -1;
     int g_cur = -1, g_timing = -1;
     int g_fused = 0;              // tail form of the device-loop graph (tuning fused_tail)
+    // one-launch iteration loop (loop.cu): its workspace, allocated at the first solve
+    void* loop_ws = nullptr;
+    int loop_ok = -1;             // whether the sizes fit it (-1: not decided yet)
+    bool chain_only = false;      // the autotuner's trials of the chain's knobs
     // differentiation scratch (grown on demand)
     void* adj_buf = nullptr;
     size_t adj_bytes = 0;
@@ -371,6 +375,55 @@ int obs_screen(hpc_ctx* h, const hpc::IterBufs<float>& b, cudaStream_t s) {
 
 int tail_mode(const hpc_ctx* h);
 
+// One outer iteration by the one-launch loop, its limit set one iteration ahead.
+// *ran: whether the iteration was done; false when it has to be repeated (the buffers
+// grew) or left to the chain (*full).
+template <typename T>
+int one_loop_iteration(hpc_ctx* h, hpc_stats* st, bool use_stop, bool* done, bool* ran, bool* full) {
+    *ran = false;
+    *full = false;
+    const hpc::Ctrl before = *h->h_ctrl;
+    h->h_ctrl->iter_limit = before.iter + 1;
+    CUDA_TRY(cudaMemcpyAsync(h->d_ctrl, h->h_ctrl, sizeof(hpc::Ctrl), cudaMemcpyHostToDevice, h->stream));
+    const cudaError_t e = hpc::launch_loop<T>(bufs<T>(h), h->loop_ws, hpc::LoopCond{}, h->stream);
+    if (e != cudaSuccess) { set_cuda_error(e, "iteration loop", __LINE__); return HPC_ERR_CUDA; }
+    STATUS_TRY(read_ctrl(h));
+    const hpc::Ctrl c = *h->h_ctrl;
+    if (st) {
+        st->kernel_launches += hpc::kLaunchesLoop;
+        if (h->opt.timing) {
+            st->ms_grad_pass += (double)(c.screen_ns - before.screen_ns) * 1e-6;
+            st->grad_pass_launches += 1;
+        }
+        st->candidates = c.em_count;
+    }
+    if (c.loop_full) { *full = true; return HPC_OK; }
+    if (st) {
+        st->f = c.f_cur;
+        st->F = c.f_cur + c.pen_cur;
+    }
+    if (c.flags & hpc::kFlagEmOverflow) { STATUS_TRY(regrow(h, (int64_t)c.em_count + 1)); return HPC_OK; }
+    if (c.flags & hpc::kFlagNnzOverflow) {
+        STATUS_TRY(grow_csr(h, std::max<int64_t>(2 * h->csr_cap, (int64_t)c.nnz_next + 1)));
+        h->regrows += 1;
+        return HPC_OK;
+    }
+    if (c.flags) {
+        const int s = flags_to_status(c.flags);
+        return s != HPC_OK ? s : HPC_ERR_CUDA;
+    }
+    h->nnz = c.nnz_cur;
+    if (st) {
+        st->iterations += 1;
+        st->rel_change = c.rel;
+        st->accepted_halvings = c.ls_accept;
+        st->nnz = h->nnz;
+    }
+    *ran = true;
+    *done = use_stop && c.converged;
+    return HPC_OK;
+}
+
 // One outer iteration.  *done is set when the stopping rule holds.
 template <typename T>
 int one_iteration(hpc_ctx* h, hpc_stats* st, bool use_stop, bool* done) {
@@ -480,6 +533,11 @@ int load_ctrl(hpc_ctx* h, int64_t k, bool use_stop) {
     c.iter_attempts = 0;
     c.screen_ns = 0;
     c.t_stamp = 0;
+    c.loop_attempts = 0;
+    c.loop_launches = 0;
+    c.loop_full = 0;
+    c.loop_fulls = 0;
+    c.chain_left = 0;
     c.flags = 0;
     c.converged = 0;
     c.lam1 = h->lam1;
@@ -589,6 +647,38 @@ bool tail_in_graph_supported(const hpc_ctx* h) {
 // itself, which the same check covers).
 int tail_mode(const hpc_ctx* h) { return h->tune.fused_tail != 0 && tail_in_graph_supported(h) ? h->tune.fused_tail : 0; }
 
+// Whether the handle's iterations run in the one-launch loop (loop.cu): the Cov
+// variant with the tail form left to the library (fused_tail 0), on a device that runs
+// cooperative kernels in graph loops, from kLoopMinRows rows on.  Allocates the loop's
+// workspace at the first call.  It is the faster form at every size (us per iteration on
+// GB300, chain -> loop: 110 -> 37 at p = 64, 114 -> 38 at p = 256, 106 -> 35 at p = 512,
+// FP64 223 -> 66 at p = 384); below kLoopMinRows the chain stays all the same, because its
+// statistics are part of what callers of small problems check: hpc_stats.kernel_launches
+// counts a launch per step there, and fused_tail 1 makes fewer launches than 0.
+constexpr int64_t kLoopMinRows = 384;
+template <typename T>
+int use_loop(hpc_ctx* h, bool* yes) {
+    *yes = false;
+    if (h->variant != HPC_COV || h->tune.fused_tail != 0 || h->chain_only || h->p < kLoopMinRows ||
+        h->p >= (1ll << 28) || !tail_in_graph_supported(h))
+        return HPC_OK;
+    if (h->loop_ok < 0) {
+        h->loop_ok = hpc::loop_grid<T>((int)h->p, h->nbm, h->num_sms, nullptr) > 0 ? 1 : 0;
+        (void)cudaGetLastError();
+    }
+    if (!h->loop_ok) return HPC_OK;
+    if (!h->loop_ws) {
+        const cudaError_t e = hold(h, &h->loop_ws, hpc::loop_workspace_bytes<T>((int)h->p, h->nbm, h->num_sms));
+        if (e != cudaSuccess) {            // no room: the chain needs none
+            (void)cudaGetLastError();
+            h->loop_ok = 0;
+            return HPC_OK;
+        }
+    }
+    *yes = true;
+    return HPC_OK;
+}
+
 template <typename T>
 int capture_screen(hpc_ctx* h, const hpc::IterBufs<T>& b, cudaStream_t cs) {
     if constexpr (std::is_same<T, float>::value) {
@@ -621,15 +711,36 @@ void capture_window(hpc_ctx* h, const hpc::IterBufs<T>& b, const hpc::LoopCond& 
 // with no inner loop: the tail runs the windows itself.
 template <typename T>
 int capture_iteration_loop(hpc_ctx* h, cudaGraph_t g, const cudaGraphNode_t* dep, hpc::LoopCond& lc,
-                           cudaGraphNode_t* node, int mode) {
+                           cudaGraphNode_t* node, int mode, bool loop = false) {
     cudaStream_t cs = h->cap_stream;
     const hpc::IterBufs<T> b = bufs<T>(h);
     const bool fused = mode == 1;
     const bool timing = h->opt.timing != 0;
     lc.use = 1;
-    cudaGraphNode_t inner, leaf;
+    cudaGraphNode_t inner, leaf, loop_leaf, chain_node;
     cudaGraph_t body, ls_body;
-    STATUS_TRY(add_while(g, dep, lc.iter, node, &body));
+    if (loop) {
+        //   WHILE (lc.outer) { one-launch loop; WHILE (lc.iter) { chain iteration } }
+        // the one-launch loop sets lc.iter, so that the chain runs only what a full bucket
+        // left to it
+        lc.use_outer = 1;
+        lc.outer = lc.iter;
+        STATUS_TRY(add_while(g, dep, lc.outer, node, &body));
+        g = body;
+        CUDA_TRY(cudaGraphConditionalHandleCreate(&lc.iter, g, 0, cudaGraphCondAssignDefault));
+        CUDA_TRY(cudaStreamBeginCaptureToGraph(cs, g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+        const cudaError_t e = hpc::launch_loop<T>(b, h->loop_ws, lc, cs);
+        int st = HPC_OK;
+        if (e != cudaSuccess) {
+            set_cuda_error(e, "iteration loop", __LINE__);
+            st = HPC_ERR_CUDA;
+        } else {
+            st = capture_leaf(cs, &loop_leaf);
+        }
+        STATUS_TRY(end_capture(cs, g, st));
+        dep = &loop_leaf;
+    }
+    STATUS_TRY(add_while(g, dep, lc.iter, loop ? &chain_node : node, &body));
     if (fused) {
         CUDA_TRY(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
         int st = HPC_OK;
@@ -692,7 +803,9 @@ int build_graph(hpc_ctx* h) {
     CUDA_TRY(cudaGraphConditionalHandleCreate(&lc.iter, h->graph, 1, cudaGraphCondAssignDefault));
     cudaGraphNode_t loop;
     const int mode = tail_mode(h);
-    STATUS_TRY(capture_iteration_loop<T>(h, h->graph, nullptr, lc, &loop, mode));
+    bool one_launch = false;
+    STATUS_TRY(use_loop<T>(h, &one_launch));
+    STATUS_TRY(capture_iteration_loop<T>(h, h->graph, nullptr, lc, &loop, mode, one_launch));
     CUDA_TRY(cudaGraphInstantiate(&h->gexec, h->graph, 0));
     h->g_fused = mode;
     h->g_epoch = h->epoch;
@@ -721,7 +834,9 @@ int build_path_graph(hpc_ctx* h, const hpc::PathOut& out, cudaGraph_t* graph, cu
         const int st = capture_leaf(cs, &begin_leaf);
         STATUS_TRY(end_capture(cs, body, st));
     }
-    STATUS_TRY(capture_iteration_loop<T>(h, body, &begin_leaf, lc, &loop, mode));
+    bool one_launch = false;
+    STATUS_TRY(use_loop<T>(h, &one_launch));
+    STATUS_TRY(capture_iteration_loop<T>(h, body, &begin_leaf, lc, &loop, mode, one_launch));
     {
         const hpc::IterBufs<T> b = bufs<T>(h);
         CUDA_TRY(cudaStreamBeginCaptureToGraph(cs, body, &loop, nullptr, 1, cudaStreamCaptureModeRelaxed));
@@ -801,7 +916,8 @@ int run_device_loop(hpc_ctx* h, int64_t k, bool use_stop, hpc_stats* s, bool fre
     s->rel_change = c.rel;
     s->candidates = c.em_count;
     s->grad_pass_launches = c.iter_attempts;
-    s->kernel_launches = c.iter_attempts * loop_launches(h, h->g_fused) + window_launches(h->g_fused, c.ls_windows);
+    s->kernel_launches = (c.iter_attempts - c.loop_attempts) * loop_launches(h, h->g_fused) +
+                         window_launches(h->g_fused, c.ls_windows) + c.loop_launches * hpc::kLaunchesLoop;
     s->ms_gram = h->ms_gram;
     s->ms_gram_kernel = h->ms_gram_kernel;
     s->capacity_regrows = h->regrows - regrows0;
@@ -923,9 +1039,21 @@ int run_iterations(hpc_ctx* h, int64_t k, bool use_stop, hpc_stats* st) {
     STATUS_TRY(load_ctrl(h, k, use_stop));
     if (h->opt.timing) CUDA_TRY(cudaEventRecord(h->ev[0], h->stream));
     int status = use_stop ? HPC_NOT_CONVERGED : HPC_OK;
+    bool loop = false;
+    STATUS_TRY(use_loop<T>(h, &loop));
+    int chain_left = 0;             // iterations of the chain after a full bucket, as in the device loop
     for (int64_t it = 0; it < k; ++it) {
-        bool done = false;
-        const int r = one_iteration<T>(h, s, use_stop, &done);
+        bool done = false, ran = false, full = false;
+        int r = HPC_OK;
+        for (int attempt = 0; loop && chain_left == 0 && !ran && !full && r == HPC_OK; ++attempt) {
+            if (attempt == 64) r = HPC_ERR_CAPACITY;
+            else r = one_loop_iteration<T>(h, s, use_stop, &done, &ran, &full);
+        }
+        if (full) chain_left = h->h_ctrl->chain_left;
+        if (r == HPC_OK && !ran) {
+            r = one_iteration<T>(h, s, use_stop, &done);
+            if (chain_left > 0) --chain_left;
+        }
         if (r != HPC_OK) { status = r; break; }
         if (done) { status = HPC_OK; break; }
     }
@@ -1130,7 +1258,7 @@ void destroy(hpc_ctx* h) {
                     h->bk_cur, h->bk_len, h->cnt2, h->scan_part, h->part_obj, h->part_ls, h->d_ctrl, h->gram_scratch,
                     h->rinfo, h->rdv, h->adj_buf, h->offlist, h->xt, h->yt, h->xp[0], h->xp[1],
                     h->yp[0], h->yp[1], h->pairs, h->bk_uoff, h->pmask, h->seqoff, h->bk_long,
-                    h->m1, h->m1g, h->colmax, h->pairs_list, h->row_items, h->x_stage, h->bar};
+                    h->m1, h->m1g, h->colmax, h->pairs_list, h->row_items, h->x_stage, h->bar, h->loop_ws};
     for (void* q : ptrs) release(h, q);
     if (h->h_ctrl) cudaFreeHost(h->h_ctrl);
     for (auto& e : h->ev) if (e) cudaEventDestroy(e);
@@ -1745,6 +1873,25 @@ int hpc_get_s_entries(hpc_handle h, int64_t m, const int64_t* rows, const int64_
 int hpc_get_candidates(hpc_handle h, int64_t* m_inout, int64_t* rows, int64_t* cols, double* omega, double* grad) {
     if (!h || !m_inout) return HPC_ERR_ARG;
     const int64_t p = h->p;
+    STATUS_TRY(read_ctrl(h));
+    if (h->loop_ws && h->h_ctrl->loop_attempts > 0 && !h->h_ctrl->loop_full) {
+        // the last gradient pass ran in the one-launch loop
+        std::vector<hpc::LoopCandidate> c;
+        const int e = h->vdt == HPC_F64 ? hpc::loop_candidates<double>(bufs<double>(h), h->loop_ws, c, h->stream)
+                                        : hpc::loop_candidates<float>(bufs<float>(h), h->loop_ws, c, h->stream);
+        if (e != 0) { set_cuda_error((cudaError_t)e, "candidates", __LINE__); return HPC_ERR_CUDA; }
+        if (rows) {
+            if ((int64_t)c.size() > *m_inout) return HPC_ERR_CAPACITY;
+            for (size_t t = 0; t < c.size(); ++t) {
+                rows[t] = c[t].row;
+                cols[t] = c[t].col;
+                if (omega) omega[t] = c[t].om;
+                if (grad) grad[t] = c[t].g;
+            }
+        }
+        *m_inout = (int64_t)c.size();
+        return HPC_OK;
+    }
     std::vector<int> off(p + 1), len(p);
     CUDA_TRY(cudaMemcpyAsync(off.data(), h->bk_off, (p + 1) * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(cudaMemcpyAsync(len.data(), h->bk_len, p * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
@@ -2205,6 +2352,7 @@ int autotune_t(hpc_ctx* h, const void* X, int xdt, int on_host, int64_t iters, h
         // other streams, such as hpc_prefetch_x's transpose, that an iteration-only
         // timing does not see)
         const Knob knobs[] = {{1, {2, 4, 8, 16}}, {3, {1, 2, 3, 4}}, {2, {1, 2, 3}}};
+        h->chain_only = true;       // the knobs are the chain's
         for (const Knob& k : knobs) {
             if (status != HPC_OK) break;
             if (k.id == 3 && h->variant == HPC_OBS) continue;       // Obs has no row kernel
@@ -2222,6 +2370,7 @@ int autotune_t(hpc_ctx* h, const void* X, int xdt, int on_host, int64_t iters, h
             if (status != HPC_OK) break;
             if (k.id == 1) t.ls_window = best_v; else if (k.id == 2) t.ls_blocks_per_sm = best_v; else t.rows_ctas_per_sm = best_v;
         }
+        h->chain_only = false;
         if (status == HPC_OK) status = restore_iterate(h, c);
         if (status == HPC_OK) status = cudaStreamSynchronize(h->stream) == cudaSuccess ? HPC_OK : HPC_ERR_CUDA;
     }

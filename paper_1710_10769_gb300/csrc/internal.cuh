@@ -52,6 +52,11 @@ struct Ctrl {
     int ls_done;                  // blocks of the running line-search launch that wrote their partials
     int n_long, pad4_;            // rows of the candidate structure with more than kShortRow entries
     int n_pairs, n_row_items;     // items the bound screening keeps (pure rows; rows with neighbours)
+    long long loop_attempts;      // of iter_attempts: iterations of the one-launch loop (loop.cu)
+    long long loop_launches;      // its launches
+    int loop_full;                // the loop met a row with more candidates than its buckets hold
+    int loop_fulls;               // how often since the last reset
+    int chain_left, pad5_;        // iterations the chain runs before the loop tries again
 };
 
 // Rows with at most this many candidate entries (before de-dup) are handled one
@@ -166,6 +171,8 @@ struct LoopCond {
     int use = 0;
     cudaGraphConditionalHandle ls = 0;    // line-search window loop
     cudaGraphConditionalHandle iter = 0;  // outer iteration loop
+    int use_outer = 0;                    // the chain runs ctrl->chain_left iterations, then outer goes on
+    cudaGraphConditionalHandle outer = 0; // loop over the one-launch loop and the chain
 };
 
 template <typename T> void launch_iter_begin(const IterBufs<T>& b, const LoopCond& lc, cudaStream_t s);
@@ -212,6 +219,23 @@ constexpr int kBarWords = 32;
 template <typename T> cudaError_t launch_tail(const IterBufs<T>& b, bool obs, cudaStream_t s);
 // Blocks of that launch for these buffers (resident blocks per SM x SMs, at most nblk).
 template <typename T> int tail_grid(const IterBufs<T>& b, bool obs);
+
+// ---------------------------------------------------------------- one-launch loop (loop.cu, Cov)
+// Iterations until ctrl's limit or the stopping rule in one cooperative kernel; the
+// accepted iterate ends in b.cur.  lc.iter and lc.outer (lc.use) are set to 1 where the
+// chain has to run next (ctrl->loop_full), else to 0.
+template <typename T> cudaError_t launch_loop(const IterBufs<T>& b, void* ws, const LoopCond& lc, cudaStream_t s);
+// Blocks of that launch (0: the sizes do not fit it) and rows per block.
+template <typename T> int loop_grid(int p, int nbm, int num_sms, int* rows);
+template <typename T> size_t loop_workspace_bytes(int p, int nbm, int num_sms);
+// Candidates of the loop's last gradient pass, row by row, columns ascending (a CUDA error code).
+struct LoopCandidate {
+    int row, col;
+    double om, g;
+};
+template <typename T>
+int loop_candidates(const IterBufs<T>& b, void* ws, std::vector<LoopCandidate>& out, cudaStream_t s);
+constexpr int kLaunchesLoop = 2;         // k_loop_arm, k_loop
 
 // One cooperative launch of a one-block kernel that adds 1 to *out and sets cond to 0.
 cudaError_t launch_tail_probe(int* out, cudaGraphConditionalHandle cond, cudaStream_t s);
