@@ -11,22 +11,18 @@
 //   BF16 X           : one panel, one product (bf16 x bf16 is exact in FP32);
 //   TF32             : FP32 panel rounded to TF32, kind::tf32 products.
 //
-// Tiles.  A 128 x 256 tile S[I, J] (UMMA M = 128, N = 256) is accumulated in
-// chunks of K (each from a zero TMEM accumulator, the chunk sums added in FP32
-// round-to-nearest in registers).  Only the tiles that touch the upper triangle
-// run, in bands of row blocks (a tuning knob) so that the tiles in flight share A
-// and B panels in L2.  The product kernel writes S_ij for i <= j; a second pass
+// Tiles.  A 128 x 256 (one CTA; UMMA M = 128, N = 256) or 256 x 256 tile S[I, J] (a pair of
+// CTAs; M = N = 256) is accumulated in chunks of K (each from a zero TMEM accumulator, the
+// chunk sums added in FP32 round-to-nearest in registers).  Only the tiles that touch the
+// upper triangle run, in bands of row blocks (a tuning knob) so that the tiles in flight
+// share A and B panels in L2.  The product kernel writes S_ij for i <= j; a second pass
 // (k_mirror_max) writes S_ji = S_ij, so S is bitwise symmetric by construction, and
-// optionally the block maxima of |S| for the bound screening.
+// optionally the block maxima of |S| for the bound screening.  (Written by the product's
+// epilogue instead, they come in bursts of all SMs at once that hold the tensor pipe up for
+// as long as the pass takes: measured equal at p = 16384, slower at p = 65536.)
 //
-// Persistent kernel (384 threads, one CTA per SM): warp 0 takes tiles and issues
-// TMA loads into a ring of stages, warp 1 issues MMAs from one lane and owns the
-// TMEM allocation (two 256-column accumulators, so the epilogue of one chunk
-// overlaps the MMAs of the next), warps 4-11 drain the accumulators (TMEM lanes
-// 32 (w % 4) .. + 31, one column half each), sum the chunks, scale by 1/n and store
-// the upper part of the tile.  Every mbarrier wait is bounded; on timeout the CTA
-// records an error word, stops issuing, waits (bounded) for its own copies and
-// MMAs, frees its TMEM and returns.
+// Every mbarrier wait is bounded; on timeout the CTA records an error word, stops issuing,
+// waits (bounded) for its copies and MMAs, frees its TMEM and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
@@ -42,14 +38,13 @@
 namespace hpc {
 namespace {
 
-constexpr int kBM = 128;           // rows of A per tile (UMMA M)
-constexpr int kBN = 256;           // rows of B per tile (UMMA N)
+constexpr int kBM = 128;           // rows of A per CTA
+constexpr int kTile = 256;         // columns of a tile (UMMA N); rows: 128 for one CTA, 256 for a pair
 constexpr int kRowBytes = 128;     // one swizzle row = one K-slab of a panel row
-constexpr int kABytes = kBM * kRowBytes;   // 16 KB
-constexpr int kBBytes = kBN * kRowBytes;   // 32 KB
-constexpr int kBand = 16;          // row blocks per band of the tile order
+constexpr int kHalfBytes = kBM * kRowBytes;   // 16 KB: 128 rows of an operand per stage
+constexpr int kBand = 16;          // row blocks of 128 per band of the tile order
 constexpr uint32_t kTmemCols = 256;
-constexpr long long kWaitLimit = 1ll << 26;
+constexpr long long kWaitNs = 4000000000ll;   // 4 s per wait
 
 enum : int { kModeBf16 = 0, kModeBf16x3 = 1, kModeTf32 = 2 };
 
@@ -67,26 +62,42 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
                  : "memory");
 }
 
+template <bool PAIR>
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
+    if constexpr (PAIR)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
     return ok != 0;
 }
 
-// Bounded wait: false on timeout or when another role raised the abort flag.
+// Bounded wait: false after kWaitNs or when another role raised the abort flag.
 // The first wait to give up records its code in the launch's error word.
+template <bool PAIR>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int code,
                                           int* err) {
-    for (long long it = 0; it < kWaitLimit; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((it & 255) == 255) {
+    long long t0 = 0;
+    for (unsigned it = 1;; ++it) {
+        if (mbar_try_wait<PAIR>(bar, parity)) return true;
+        if ((it & 255u) == 0u) {
             if (*abort_flag) return false;
+            long long t;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            if (t0 == 0) t0 = t;
+            if (t - t0 > kWaitNs) break;
             __nanosleep(64);
         }
     }
@@ -95,26 +106,73 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return false;
 }
 
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1)
-        : "memory");
+// The address in the pair's leader (rank 0 of the cluster), or in the given rank, of what
+// this CTA has at p.
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
+// A load into this CTA's shared memory whose bytes are counted on a barrier (PAIR: of
+// either CTA of the pair; bar: a shared::cluster address).
+template <bool PAIR>
+__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
+    if constexpr (PAIR) {
+        asm volatile(
+            "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
+            "[%0], [%1, {%3, %4}], [%2];"
+            ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
+            : "memory");
+    } else {
+        asm volatile(
+            "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+            ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
+            : "memory");
+    }
+}
+
+// TMEM.  PAIR: of the pair, every call made by one warp of each of the two CTAs.
+template <bool PAIR>
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)),
-                 "r"(ncols)
-                 : "memory");
+    if constexpr (PAIR)
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)), "r"(ncols)
+                     : "memory");
+    else
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)), "r"(ncols)
+                     : "memory");
 }
+template <bool PAIR>
 __device__ __forceinline__ void tmem_relinquish() {
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (PAIR) asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    else asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
+template <bool PAIR>
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+    if constexpr (PAIR)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+    else
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// PAIR: BF16X3 and TF32 run on CTA pairs, one BF16 product on single CTAs (see below).
+constexpr bool pair_mode(int mode) { return mode != kModeBf16; }
 
 template <int MODE>
 __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
@@ -122,7 +180,13 @@ __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t adesc, uint64_t b
     if constexpr (MODE == kModeTf32) {
         asm volatile(
             "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+            "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            : "memory");
+    } else if constexpr (pair_mode(MODE)) {
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
             ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
             : "memory");
     } else {
@@ -134,11 +198,30 @@ __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t adesc, uint64_t b
     }
 }
 
+// The completion of the MMAs issued so far, as an arrival on the barrier (PAIR: of both CTAs).
+template <bool PAIR>
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
+    if constexpr (PAIR)
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+                smem_u32(bar)),
+            "h"((uint16_t)3)
+            : "memory");
+    else
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+                     : "memory");
 }
 
+// 32 TMEM lanes x 16 consecutive 32-bit columns: thread t gets lane (base + t).
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
 // 32 TMEM lanes x 32 consecutive 32-bit columns: thread t gets lane (base + t).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
@@ -149,16 +232,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
           "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-}
-// 32 TMEM lanes x 16 consecutive 32-bit columns: thread t gets lane (base + t).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr)
         : "memory");
 }
@@ -177,14 +250,14 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
 }
 
 // Instruction descriptor: D = F32, A/B = BF16 (kind::f16) or TF32 (kind::tf32),
-// both K-major, N = 256, M = 128.
+// both K-major, N = 256, M = 128 or, for a pair, 256 (128 rows in each CTA).
 template <int MODE>
 __host__ __device__ constexpr uint32_t instr_desc() {
     return (1u << 4)                                          // D format F32
            | ((MODE == kModeTf32 ? 2u : 1u) << 7)             // A format
            | ((MODE == kModeTf32 ? 2u : 1u) << 10)            // B format
-           | ((uint32_t)(kBN >> 3) << 17)                     // N >> 3
-           | ((uint32_t)(kBM >> 4) << 24);                    // M >> 4
+           | ((uint32_t)(kTile >> 3) << 17)                   // N >> 3
+           | ((uint32_t)((pair_mode(MODE) ? 2 * kBM : kBM) >> 4) << 24);   // M >> 4
 }
 
 template <int MODE>
@@ -194,8 +267,10 @@ struct Cfg {
     static constexpr int kElem = (MODE == kModeTf32) ? 4 : 2;
     static constexpr int kBK = kRowBytes / kElem;                      // K elements per stage
     static constexpr int kMmaK = 32 / kElem;                           // K per instruction
-    static constexpr int kStageBytes = kPieces * (kABytes + kBBytes);
-    static constexpr int kStages = (MODE == kModeBf16x3) ? 2 : 4;
+    static constexpr bool kPair = pair_mode(MODE);
+    static constexpr int kPieceBytes = (kPair ? 2 : 3) * kHalfBytes;   // A, and half of B or all of it
+    static constexpr int kStageBytes = kPieces * kPieceBytes;          // per CTA
+    static constexpr int kStages = (MODE == kModeBf16x3) ? 3 : kPair ? 6 : 4;
     static constexpr int kSmem = kStages * kStageBytes + 1024 /*align*/ + 256 /*barriers and flags*/
                                  + 8 * 32 * 17 * 4 /*per-warp staging of the row stores*/;
 };
@@ -210,11 +285,28 @@ __device__ __forceinline__ uint16_t bf16_up_f(float x) {
 __device__ __forceinline__ void mbar_arrive_local(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// On the leader's barrier.
+template <bool PAIR>
+__device__ __forceinline__ void arrive_leader(uint64_t* bar) {
+    if constexpr (PAIR) mbar_arrive_cluster(cluster_addr(bar, 0));
+    else mbar_arrive_local(bar);
+}
 
-// Persistent form: one CTA per SM walks the banded order of the tile list, so the
-// tiles running together share X panels in L2.  Dynamic: the CTAs take tiles from a
-// counter they share, so the tiles in flight stay a contiguous window of the order
-// however the CTAs drift; static: CTA g takes tiles g, g + grid, ...
+// Persistent workers, single CTAs or CTA pairs (clusters of two), one CTA per SM, walk the
+// banded order of the tile list, so the tiles running together share X panels in L2.
+// Dynamic: the workers take tiles from a counter they share, so the tiles in flight stay a
+// contiguous window of the order however they drift; static: worker g takes tiles g,
+// g + workers, ...
+//
+// Pairs or single CTAs.  At full rate an MMA of M = 128, N = 256 in one CTA reads 96 B of
+// operands per cycle from shared memory while TMA refills it at the same rate; with
+// cta_group::2 the two SMs share one M = 256, N = 256 product, each holding its 128 rows of
+// A and half of B: 64 B per cycle each way, and two thirds of the bytes per stage.  BF16X3
+// (two panels per operand) got two stages of 96 KB from one CTA and gets three of 64 KB
+// from a pair: 1650 -> 1900 TFLOP/s of BF16 products at p = 16384, n = 8192.  One BF16
+// product gains nothing: its pipe waits about 450 cycles at every change of accumulator
+// (32 MMAs; one chunk per tile runs 10% faster, but its sums are biased), and under the
+// power cap the single CTA is ahead at p = 65536 (94 against 96-98 ms), so it keeps it.
 //
 // Chunked accumulation.  The tensor core adds each MMA's K slice into the FP32
 // accumulator with truncation, so a sum over the whole K = n carries a bias that
@@ -225,22 +317,25 @@ __device__ __forceinline__ void mbar_arrive_local(uint64_t* bar) {
 // The bias then scales with the chunk lengths instead of n (the sum over chunks of
 // length^2 / K).  A chunk longer than K gives one chunk per tile.
 //
-// Roles:
-//   warp 0      TMA producer: takes the next tile, publishes its index in a ring of
-//               kTileRing slots (tid_full / tid_empty), loads its K slices ahead;
-//   warp 1      MMA issuer: chunk c of the CTA's sequence into TMEM accumulator
-//               c & 1 (columns 0 / 256), so a chunk accumulates while the previous
-//               one is read out;
+// Roles (leader: rank 0 of the pair, or the CTA alone, which then is both):
+//   warp 0      TMA producer of both CTAs: its rows of A and its half of B per stage, all
+//               counted on the leader's full barrier.  The leader's takes the next tile and
+//               publishes its index in a ring of kTileRing slots of both CTAs (tid_full;
+//               tid_empty: the leader's);
+//   warp 1      of the leader: MMA issuer, chunk c of the pair's sequence into TMEM
+//               accumulator c & 1 (columns 0 / 256) of both CTAs, so a chunk accumulates
+//               while the previous one is read out;
 //   warps 2-3   idle (they complete warpgroup 0, which hands registers to the
 //               epilogue with setmaxnreg);
-//   warps 4-11  epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 and the column
-//               half (w - 4) / 4 of the tile (128 columns), keeps the running
-//               sums of its row's 128 columns in registers, and after a tile's last
-//               chunk scales by 1/n and stores the entries with i <= j (the lower
-//               triangle and the block maxima come from the mirror pass).
-// acc_full[b] (one commit) and acc_empty[b] (eight epilogue warps) hand the
-// buffers over.  Every wait is bounded; an abort stops all roles, drains the
-// loads in flight and frees TMEM.
+//   warps 4-11  epilogue of both CTAs: warp w reads TMEM lanes 32 (w % 4) .. +31 (rows of
+//               the CTA's 128) and the column half (w - 4) / 4 of the tile (128 columns),
+//               keeps the running sums of its row's 128 columns in registers, and after a
+//               tile's last chunk scales by 1/n and stores the entries with i <= j (the
+//               lower triangle and the block maxima come from the mirror pass).
+// A commit arrives at empty[s] and acc_full[b] of both CTAs; acc_empty[b] is the leader's
+// and counts the sixteen epilogue warps of the pair.  Every wait is bounded; an abort stops
+// the roles of its CTA (the other's waits run out), the loads in flight are drained, and
+// neither CTA leaves or frees TMEM before the other is done.
 constexpr int kEpiWarps = 8;
 constexpr int kPersistThreads = 128 + 32 * kEpiWarps;     // warpgroup 0: roles; warpgroups 1-2: epilogue
 // Registers per thread after setmaxnreg: warpgroup 0 gives down to kRegsSmall, the two
@@ -251,7 +346,7 @@ constexpr int kRegsSmall = 56;
 constexpr int kRegsEpi = 216;
 constexpr int kMinLaunchRegs = (128 * kRegsSmall + 32 * kEpiWarps * kRegsEpi + kPersistThreads - 1) / kPersistThreads;
 constexpr int kTileRing = 4;
-constexpr int kHalf = kBN / 2;          // columns per epilogue warp
+constexpr int kHalf = kTile / 2;        // columns per epilogue warp
 
 // The launch's control words in the scratch's slack: the shared tile counter and the
 // error word of the bounded waits, reset before each launch (by a kernel, so the reset
@@ -266,14 +361,15 @@ k_gram_tc_persist(const __grid_constant__ CUtensorMap map_hi, const __grid_const
                   float* __restrict__ S, int64_t lds, unsigned* __restrict__ tile_ctr, int* __restrict__ err,
                   int dynamic, int chunk_kt, int lead_kt) {
     using C = Cfg<MODE>;
+    constexpr bool kPair = C::kPair;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStageBytes);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::kStages * C::kStageBytes);   // the leader's
     uint64_t* empty = full + C::kStages;
     uint64_t* acc_full = empty + C::kStages;     // [2]
-    uint64_t* acc_empty = acc_full + 2;          // [2]
+    uint64_t* acc_empty = acc_full + 2;          // [2], the leader's
     uint64_t* tid_full = acc_empty + 2;          // [kTileRing]
-    uint64_t* tid_empty = tid_full + kTileRing;  // [kTileRing]: MMA thread + one epilogue thread
+    uint64_t* tid_empty = tid_full + kTileRing;  // [kTileRing], the leader's: MMA thread, peer's producer, two epilogue threads
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tid_empty + kTileRing);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* s_tid = reinterpret_cast<volatile int*>(tmem_slot + 2);      // [kTileRing]
@@ -282,25 +378,29 @@ k_gram_tc_persist(const __grid_constant__ CUtensorMap map_hi, const __grid_const
     static_assert(8 * (2 * C::kStages + 4 + 2 * kTileRing) + 4 * (2 + kTileRing + 2) <= 256, "barrier area");
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = kPair ? cluster_rank() : 0;
+    const bool leader = rank == 0;
+    const unsigned worker = kPair ? blockIdx.x >> 1 : blockIdx.x, workers = kPair ? gridDim.x >> 1 : gridDim.x;
     if (chunk_kt < 1) chunk_kt = 1;
     if (lead_kt < chunk_kt) lead_kt = chunk_kt;
     const int nch = num_chunks(k_tiles, chunk_kt, lead_kt);     // chunks per tile
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], kEpiWarps); }
-        for (int r = 0; r < kTileRing; ++r) { mbar_init(&tid_full[r], 1); mbar_init(&tid_empty[r], 2); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], (kPair ? 2 : 1) * kEpiWarps); }
+        for (int r = 0; r < kTileRing; ++r) { mbar_init(&tid_full[r], 1); mbar_init(&tid_empty[r], kPair ? 4 : 2); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_hi)) : "memory");
         if (C::kPieces > 1) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_lo)) : "memory");
     }
     if (warp == 1) {
-        tmem_alloc(tmem_slot, 2 * kTmemCols);
-        tmem_relinquish();
+        tmem_alloc<kPair>(tmem_slot, 2 * kTmemCols);
+        tmem_relinquish<kPair>();
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (kPair) cluster_sync();     // the peer's barriers are initialised, its TMEM is allocated
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
@@ -313,50 +413,63 @@ k_gram_tc_persist(const __grid_constant__ CUtensorMap map_hi, const __grid_const
             long long g = 0;
             bool ok = true;
             for (int lt = 0; ok; ++lt) {
-                // the next tile of the shared order, published to the MMA and epilogue roles
                 const int slot = lt % kTileRing;
-                if (!mbar_wait(&tid_empty[slot], ((uint32_t)(lt / kTileRing) & 1u) ^ 1u, abort_flag, 15, err)) break;
-                // dynamic: the counter shared by the CTAs; static: tiles blockIdx.x + lt * grid
-                const unsigned t = dynamic ? atomicAdd(tile_ctr, 1u)
-                                           : (unsigned)blockIdx.x + (unsigned)lt * (unsigned)gridDim.x;
-                const int tt = t < (unsigned)ntiles ? (int)t : -1;
-                s_tid[slot] = tt;
-                mbar_arrive_local(&tid_full[slot]);
+                const uint32_t rph = (uint32_t)(lt / kTileRing) & 1u;
+                int tt;
+                if (leader) {
+                    // the next tile of the shared order, published to the roles of both CTAs
+                    if (!mbar_wait<kPair>(&tid_empty[slot], rph ^ 1u, abort_flag, 15, err)) break;
+                    // dynamic: the counter shared by the workers; static: tiles worker + lt * workers
+                    const unsigned t = dynamic ? atomicAdd(tile_ctr, 1u) : worker + (unsigned)lt * workers;
+                    tt = t < (unsigned)ntiles ? (int)t : -1;
+                    s_tid[slot] = tt;
+                    mbar_arrive_local(&tid_full[slot]);
+                    if constexpr (kPair) {
+                        st_cluster(cluster_addr(const_cast<int*>(s_tid + slot), 1), tt);
+                        mbar_arrive_cluster(cluster_addr(&tid_full[slot], 1));
+                    }
+                } else {
+                    if (!mbar_wait<kPair>(&tid_full[slot], rph, abort_flag, 18, err)) break;
+                    tt = s_tid[slot];
+                    mbar_arrive_cluster(cluster_addr(&tid_empty[slot], 0));
+                }
                 if (tt < 0) break;
                 const int2 tile = tiles[tt];
-                const int I0 = tile.x * kBM, J0 = tile.y * kBN;
+                const int I0 = kPair ? tile.x * kTile + (int)rank * kBM : tile.x * kBM;
+                const int J0 = tile.y * kTile + (int)rank * kBM;
                 for (int kt = 0; kt < k_tiles; ++kt, ++g) {
                     const int s = (int)(g % C::kStages);
                     const uint32_t ph = (uint32_t)(g / C::kStages) & 1u;
-                    if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, 11, err)) { ok = false; break; }
+                    if (!mbar_wait<kPair>(&empty[s], ph ^ 1u, abort_flag, 11, err)) { ok = false; break; }
                     uint8_t* st = smem + s * C::kStageBytes;
-                    mbar_expect_tx(&full[s], C::kStageBytes);
+                    // the bytes of both CTAs; the peer's may arrive first
+                    if (leader) mbar_expect_tx(&full[s], (kPair ? 2 : 1) * C::kStageBytes);
+                    const uint32_t bar = kPair ? cluster_addr(&full[s], 0) : smem_u32(&full[s]);
                     const int kc = kt * C::kBK;
                     for (int pc = 0; pc < C::kPieces; ++pc) {
                         const CUtensorMap* m = pc == 0 ? &map_hi : &map_lo;
-                        uint8_t* a = st + pc * (kABytes + kBBytes);
-                        uint8_t* b = a + kABytes;
-                        tma_load_2d(a, m, &full[s], kc, I0);
-                        tma_load_2d(b, m, &full[s], kc, J0);
-                        tma_load_2d(b + kABytes, m, &full[s], kc, J0 + kBM);
+                        uint8_t* a = st + pc * C::kPieceBytes;
+                        tma_load_2d<kPair>(a, m, bar, kc, I0);
+                        tma_load_2d<kPair>(a + kHalfBytes, m, bar, kc, J0);
+                        if constexpr (!kPair) tma_load_2d<kPair>(a + 2 * kHalfBytes, m, bar, kc, J0 + kBM);
                     }
                     ++issued;
                 }
             }
-        } else if (threadIdx.x == 32) {
+        } else if (threadIdx.x == 32 && leader) {
             // ---------------- MMA issuer: chunk after chunk, alternating the two accumulators
             constexpr uint32_t idesc = instr_desc<MODE>();
             long long g = 0, gc = 0;
             bool ok = true;
             for (int lt = 0; ok; ++lt) {
                 const int slot = lt % kTileRing;
-                if (!mbar_wait(&tid_full[slot], (uint32_t)(lt / kTileRing) & 1u, abort_flag, 16, err)) break;
+                if (!mbar_wait<kPair>(&tid_full[slot], (uint32_t)(lt / kTileRing) & 1u, abort_flag, 16, err)) break;
                 const int tt = s_tid[slot];
                 mbar_arrive_local(&tid_empty[slot]);
                 if (tt < 0) break;
                 for (int c = 0; c < nch && ok; ++c, ++gc) {
                     const int b = (int)(gc & 1);
-                    if (!mbar_wait(&acc_empty[b], ((uint32_t)(gc >> 1) & 1u) ^ 1u, abort_flag, 12, err)) { ok = false; break; }
+                    if (!mbar_wait<kPair>(&acc_empty[b], ((uint32_t)(gc >> 1) & 1u) ^ 1u, abort_flag, 12, err)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t acc = tmem + (uint32_t)(b * kTmemCols);
                     const int kt0 = chunk_start(c, k_tiles, chunk_kt, lead_kt);
@@ -364,11 +477,11 @@ k_gram_tc_persist(const __grid_constant__ CUtensorMap map_hi, const __grid_const
                     for (int kt = kt0; kt < kt1; ++kt, ++g) {
                         const int s = (int)(g % C::kStages);
                         const uint32_t ph = (uint32_t)(g / C::kStages) & 1u;
-                        if (!mbar_wait(&full[s], ph, abort_flag, 13, err)) { ok = false; break; }
+                        if (!mbar_wait<kPair>(&full[s], ph, abort_flag, 13, err)) { ok = false; break; }
                         tc_fence_after();
                         const uint32_t st = smem_u32(smem + s * C::kStageBytes);
-                        const uint32_t a_hi = st, b_hi = st + kABytes;
-                        const uint32_t a_lo = st + (kABytes + kBBytes), b_lo = a_lo + kABytes;
+                        const uint32_t a_hi = st, b_hi = st + kHalfBytes;
+                        const uint32_t a_lo = st + C::kPieceBytes, b_lo = a_lo + kHalfBytes;
     #pragma unroll
                         for (int kk = 0; kk < C::kBK / C::kMmaK; ++kk) {
                             const uint32_t off = kk * 32;
@@ -379,9 +492,9 @@ k_gram_tc_persist(const __grid_constant__ CUtensorMap map_hi, const __grid_const
                                 umma<MODE>(acc, smem_desc_sw128(a_lo + off), smem_desc_sw128(b_hi + off), idesc, 1u);
                             }
                         }
-                        umma_commit(&empty[s]);
+                        umma_commit<kPair>(&empty[s]);
                     }
-                    if (ok) umma_commit(&acc_full[b]);
+                    if (ok) umma_commit<kPair>(&acc_full[b]);
                 }
             }
         }
@@ -409,9 +522,9 @@ k_gram_tc_persist(const __grid_constant__ CUtensorMap map_hi, const __grid_const
             if (et == 0) {
                 const int slot = lt % kTileRing;
                 int tt = -1;
-                if (!*abort_flag && mbar_wait(&tid_full[slot], (uint32_t)(lt / kTileRing) & 1u, abort_flag, 17, err)) {
+                if (!*abort_flag && mbar_wait<kPair>(&tid_full[slot], (uint32_t)(lt / kTileRing) & 1u, abort_flag, 17, err)) {
                     tt = s_tid[slot];
-                    mbar_arrive_local(&tid_empty[slot]);
+                    arrive_leader<kPair>(&tid_empty[slot]);
                 }
                 s_epi[lt & 1] = tt;
             }
@@ -422,29 +535,52 @@ k_gram_tc_persist(const __grid_constant__ CUtensorMap map_hi, const __grid_const
 #pragma unroll
             for (int q = 0; q < kHalf; ++q) acc[q] = 0.f;
             bool have = true;
+            // this warp's lanes of buffer b are read
+            auto hand_back = [&](int b) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) arrive_leader<kPair>(&acc_empty[b]);
+            };
             for (int c = 0; c < nch; ++c, ++gc) {
                 const int b = (int)(gc & 1);
                 bool got = have && !*abort_flag &&
-                           mbar_wait(&acc_full[b], (uint32_t)(gc >> 1) & 1u, abort_flag, 14, err);
+                           mbar_wait<kPair>(&acc_full[b], (uint32_t)(gc >> 1) & 1u, abort_flag, 14, err);
                 got = __all_sync(kFull, got);
                 if (!got) { have = false; continue; }
                 tc_fence_after();
+                const uint32_t from = lane_base + (uint32_t)(b * kTmemCols);
+                // Pairs: 64 columns per round, two loads in flight, the buffer handed back
+                // before the last round's adds (a single CTA gains nothing from either).
+                if constexpr (kPair) {
 #pragma unroll
-                for (int s4 = 0; s4 < kHalf / 16; ++s4) {
-                    uint32_t v[16];
-                    tmem_ld16(lane_base + (uint32_t)(b * kTmemCols + s4 * 16), v);
-                    tmem_ld_wait();
+                    for (int s4 = 0; s4 < kHalf / 64; ++s4) {
+                        uint32_t v0[32], v1[32];
+                        tmem_ld32(from + s4 * 64, v0);
+                        tmem_ld32(from + s4 * 64 + 32, v1);
+                        tmem_ld_wait();
+                        if (s4 == kHalf / 64 - 1) hand_back(b);
 #pragma unroll
-                    for (int q = 0; q < 16; ++q) acc[s4 * 16 + q] += __uint_as_float(v[q]);
+                        for (int q = 0; q < 32; ++q) {
+                            acc[s4 * 64 + q] += __uint_as_float(v0[q]);
+                            acc[s4 * 64 + 32 + q] += __uint_as_float(v1[q]);
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int s4 = 0; s4 < kHalf / 16; ++s4) {
+                        uint32_t v[16];
+                        tmem_ld16(from + s4 * 16, v);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) acc[s4 * 16 + q] += __uint_as_float(v[q]);
+                    }
+                    hand_back(b);
                 }
-                // this warp's lanes of buffer b are read: hand the buffer back
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_local(&acc_empty[b]);
             }
             if (!have) continue;
             const int2 tile = tiles[tt];
-            const int I0 = tile.x * kBM, J0 = tile.y * kBN + hc * kHalf;   // this warp's columns
+            // this CTA's rows, this warp's columns
+            const int I0 = kPair ? tile.x * kTile + (int)rank * kBM : tile.x * kBM, J0 = tile.y * kTile + hc * kHalf;
             // 16 columns at a time, staged through this warp's shared buffer so that each
             // store covers two rows x 64 contiguous bytes (a lane per row would write 32
             // rows x 16 bytes per instruction)
@@ -470,19 +606,22 @@ k_gram_tc_persist(const __grid_constant__ CUtensorMap map_hi, const __grid_const
     __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (*abort_flag && threadIdx.x == 0) {
-        // drain: bounded waits for the loads this CTA issued, so no copy lands after exit
+    if (*abort_flag && leader && threadIdx.x == 0) {
+        // drain: bounded waits for the pair's loads into the stages that were issued, so no
+        // copy lands after exit (the peer stays until the leader is through)
         for (long long g = issued > C::kStages ? issued - C::kStages : 0; g < issued; ++g) {
             const int s = (int)(g % C::kStages);
             const uint32_t ph = (uint32_t)(g / C::kStages) & 1u;
-            for (long long it = 0; it < (1ll << 22) && !mbar_try_wait(&full[s], ph); ++it) __nanosleep(64);
+            for (long long it = 0; it < (1ll << 22) && !mbar_try_wait<kPair>(&full[s], ph); ++it) __nanosleep(64);
         }
     }
     __syncthreads();
+    if constexpr (kPair) cluster_sync();     // neither CTA's TMEM, barriers or operands are in use any more
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, 2 * kTmemCols);
+        tmem_dealloc<kPair>(tmem, 2 * kTmemCols);
     }
+    if constexpr (kPair) cluster_sync();
 }
 
 // The lower triangle and, with m1, the block maxima, after the product kernel wrote
@@ -813,29 +952,33 @@ struct Geometry {
 Geometry geometry(int xdt, int64_t n, int64_t p, int precision) {
     const int mode = mode_of(xdt, precision);
     Geometry g;
-    g.p_pad = (p + kBN - 1) / kBN * kBN;
+    g.p_pad = (p + kTile - 1) / kTile * kTile;
     g.n_pad = (n + 63) / 64 * 64;
     const int es = mode == kModeTf32 ? 4 : 2;
     g.panel_bytes = (size_t)g.p_pad * g.n_pad * es;
     g.panel_bytes = (g.panel_bytes + 1023) / 1024 * 1024;
     g.pieces = mode == kModeBf16x3 ? 2 : 1;
-    const int64_t nbi = g.p_pad / kBM, nbj = g.p_pad / kBN;
-    int64_t t = 0;
-    for (int64_t bj = 0; bj < nbj; ++bj) t += std::min<int64_t>(2 * bj + 2, nbi);
-    g.ntiles = t;
+    const int64_t nb = g.p_pad / kTile;
+    g.ntiles = pair_mode(mode) ? nb * (nb + 1) / 2 : nb * (nb + 1);
     return g;
 }
 
-// Upper-triangle tiles (128 bi <= 256 bj + 255) in bands of `band` row blocks;
-// within a band, columns left to right, rows top to bottom.  The band sets
-// which X panels the concurrently running tiles share in L2 (a tuning knob).
-std::vector<int2> tile_order(int64_t p_pad, int band) {
-    const int64_t nbi = p_pad / kBM, nbj = p_pad / kBN;
-    std::vector<int2> t;
-    for (int64_t b0 = 0; b0 < nbi; b0 += band)
+// Upper-triangle tiles (rows r bi .. of r = 128 or, for pairs, 256 rows each; 256 columns)
+// in bands of `band` row blocks of 128 (pairs: rounded up to 256); within a band, columns
+// left to right, rows top to bottom.  The band sets which X panels the concurrently
+// running tiles share in L2 (a tuning knob).
+template <typename F>
+__host__ __device__ inline void for_tiles(int64_t p_pad, int band, bool pair, F&& f) {
+    const int64_t rows = pair ? kTile : kBM, nbi = p_pad / rows, nbj = p_pad / kTile;
+    const int64_t step = pair ? (band + 1) / 2 : band;
+    for (int64_t b0 = 0; b0 < nbi; b0 += step)
         for (int64_t bj = 0; bj < nbj; ++bj)
-            for (int64_t bi = b0; bi < std::min<int64_t>(b0 + band, nbi); ++bi)
-                if (bi * kBM <= bj * kBN + kBN - 1) t.push_back(make_int2((int)bi, (int)bj));
+            for (int64_t bi = b0; bi < (b0 + step < nbi ? b0 + step : nbi); ++bi)
+                if (bi * rows <= bj * kTile + kTile - 1) f(make_int2((int)bi, (int)bj));
+}
+std::vector<int2> tile_order(int64_t p_pad, int band, bool pair) {
+    std::vector<int2> t;
+    for_tiles(p_pad, band, pair, [&](int2 x) { t.push_back(x); });
     return t;
 }
 
@@ -901,13 +1044,25 @@ cudaError_t launch_mode(const Geometry& g, void* hi, void* lo, const int2* tiles
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int grid = (int)std::min<int64_t>(g.ntiles, sms);
+    const int grid = C::kPair ? 2 * (int)std::min<int64_t>(g.ntiles, std::max(1, sms / 2))
+                              : (int)std::min<int64_t>(g.ntiles, sms);
     unsigned* ctl = ctl_words(tiles, g);
     k_zero_ctl<<<1, 1, 0, s>>>(ctl);
-    k_gram_tc_persist<MODE><<<grid, kPersistThreads, C::kSmem, s>>>(mh, ml, tiles, (int)g.ntiles, k_tiles, p, n, S,
-                                                                   lds, ctl, reinterpret_cast<int*>(ctl + 1),
-                                                                   dynamic, chunk_kt, lead_kt);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kPersistThreads);
+    cfg.dynamicSmemBytes = C::kSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = C::kPair ? 1 : 0;
+    if ((e = cudaLaunchKernelEx(&cfg, k_gram_tc_persist<MODE>, mh, ml, tiles, (int)g.ntiles, k_tiles, p, n, S, lds, ctl,
+                                reinterpret_cast<int*>(ctl + 1), dynamic, chunk_kt, lead_kt)) != cudaSuccess)
+        return e;
     if (after_kernel && (e = cudaEventRecord(after_kernel, s)) != cudaSuccess) return e;
     return launch_mirror(S, lds, p, m1, nbm, s);
 }
@@ -988,9 +1143,9 @@ cudaError_t gram_tc(const void* X, int xdt, int64_t n, int64_t p, float* S, int6
     int2* tiles = reinterpret_cast<int2*>(base + g.pieces * g.panel_bytes);
     // the tile order depends on p_pad and the band only: with tiles_sig the caller keeps
     // it on the device between calls (no copy queued behind other transfers)
-    const uint64_t sig = (reinterpret_cast<uintptr_t>(tiles) * 1000003ull) ^ ((uint64_t)g.p_pad << 20) ^ (uint64_t)band;
+    const uint64_t sig = (reinterpret_cast<uintptr_t>(tiles) * 1000003ull) ^ ((uint64_t)g.p_pad << 20) ^ ((uint64_t)pair_mode(mode) << 16) ^ (uint64_t)band;
     if (!tiles_sig || *tiles_sig != sig) {
-        const std::vector<int2> order = tile_order(g.p_pad, band);
+        const std::vector<int2> order = tile_order(g.p_pad, band, pair_mode(mode));
         e = cudaMemcpyAsync(tiles, order.data(), order.size() * sizeof(int2), cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return e;
         // the host vector must outlive the copy
@@ -1057,14 +1212,9 @@ std::mutex g_noalloc_mu;
 void* g_noalloc_base[kMaxDevices] = {};   // device address of g_noalloc_scratch, per device
 
 // The tile order of tile_order(), written on the device (no host staging buffer).
-__global__ void k_tile_order(int2* __restrict__ out, int64_t p_pad) {
+__global__ void k_tile_order(int2* __restrict__ out, int64_t p_pad, bool pair) {
     if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    const int64_t nbi = p_pad / kBM, nbj = p_pad / kBN;
-    int64_t t = 0;
-    for (int64_t b0 = 0; b0 < nbi; b0 += kBand)
-        for (int64_t bj = 0; bj < nbj; ++bj)
-            for (int64_t bi = b0; bi < (b0 + kBand < nbi ? b0 + kBand : nbi); ++bi)
-                if (bi * kBM <= bj * kBN + kBN - 1) out[t++] = make_int2((int)bi, (int)bj);
+    for_tiles(p_pad, kBand, pair, [&](int2 x) { *out++ = x; });
 }
 
 // Device address of the scratch array for the current device; the first call on
@@ -1121,7 +1271,7 @@ extern "C" int hpc_gram_noalloc(const void* X, hpc_dtype xdt, int64_t n, int64_t
     void* hi = base;
     void* lo = g.pieces > 1 ? base + g.panel_bytes : nullptr;
     int2* tiles = reinterpret_cast<int2*>(base + g.pieces * g.panel_bytes);
-    k_tile_order<<<1, 1, 0, s>>>(tiles, g.p_pad);
+    k_tile_order<<<1, 1, 0, s>>>(tiles, g.p_pad, pair_mode(mode));
     if (xdt == HPC_BF16) launch_prep<__nv_bfloat16>(X, mode, n, p, hi, lo, g, s);
     else launch_prep<float>(X, mode, n, p, hi, lo, g, s);
     e = cudaGetLastError();
