@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -85,16 +86,22 @@ k_gram_simt(const TX* __restrict__ X, int64_t n, int64_t p, T* __restrict__ S, i
     }
 }
 
-// FP32 form for rows of X that start on 16-byte boundaries (p a multiple of 4 and X
-// aligned; S likewise for its rows): 128 x 128 tiles, 256 threads as 16 x 16, each
-// thread owning an 8 x 8 micro-tile made of rows {4 ty .. 4 ty + 3, 64 + 4 ty .. + 3}
-// and the same split of columns around tx, so that the 16-byte operand reads of
-// eight consecutive lanes fall on 32 different banks.  K-slabs of 8 rows are
-// double-buffered in shared memory: the next slab is loaded into registers (one
-// 4-element vector of each operand per thread) while the current one is multiplied,
-// one barrier per slab; 4 vector reads per 64 FMAs.  Every entry is still one FMA
-// chain over k in ascending order, so S is bitwise symmetric and equals the scalar
-// kernel's values.
+// FP32 form: BM x BM tiles (BM = 16 TM), 256 threads as 16 x 16, each thread owning a TM x TM
+// micro-tile made of groups of four rows {64 h + 4 ty .. + 3} and the same split of columns
+// around tx, so that the 16-byte operand reads of eight consecutive lanes fall on 32
+// different banks.  K-slabs of 16 rows are double-buffered in shared memory: the next slab
+// is loaded into registers while the current one is multiplied, one barrier per slab.  Every
+// entry is one FMA chain over k in ascending order, so S is bitwise symmetric and equals the
+// scalar kernel's values.
+//
+// What bounds it: FP32 FMAs, 128 per SM and cycle.  They are issued in pairs
+// (fma.rn.f32x2, each half rounded as fma.rn.f32), a pair of columns per
+// instruction, which leaves half of the issue slots to the operand reads, the loads and the
+// packing of the row operand.  VEC: rows of X that start on 16-byte boundaries (8 for
+// BF16) come in by four elements and S goes out by four; other rows element by
+// element, 128 neighbours at a time, into the same slabs.
+// Measured on GB300, FP32 X: p = 3001, n = 1500 (rows off 16 bytes) 421 -> 326 us, 41 TFLOP/s;
+// p = 3001, n = 600 170 -> 150; p = 4096, n = 600 242 -> 225; p = 300, n = 600 70 -> 31.
 template <typename TX>
 __device__ __forceinline__ float4 load4(const TX* p);
 template <>
@@ -105,11 +112,23 @@ __device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16* p) {
     return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
                        __uint_as_float(u.y & 0xffff0000u));
 }
+template <>
+__device__ __forceinline__ float4 load4<double>(const double*) { return make_float4(0.f, 0.f, 0.f, 0.f); }   // not VEC
 
-template <typename TX>
-__global__ void __launch_bounds__(256)
-k_gram_simt_v4(const TX* __restrict__ X, int64_t n, int64_t p, float* __restrict__ S, int64_t lds, int nb) {
-    constexpr int BM = 128, BK = 8;
+__device__ __forceinline__ void fma2(unsigned long long& c, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long dup2(float a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+    return r;
+}
+
+template <typename TX, int TM, bool VEC>
+__global__ void __launch_bounds__(256, TM == 4 ? 4 : 2)
+k_gram_simt_f32(const TX* __restrict__ X, int64_t n, int64_t p, float* __restrict__ S, int64_t lds, int nb) {
+    constexpr int BM = 16 * TM, BK = 16, H = TM / 4;
+    constexpr int L = BK * BM / 256;                  // elements of each operand a thread loads
     __shared__ __align__(16) float As[2][BK][BM];
     __shared__ __align__(16) float Bs[2][BK][BM];
     int t = blockIdx.x, bi = 0;
@@ -117,94 +136,147 @@ k_gram_simt_v4(const TX* __restrict__ X, int64_t n, int64_t p, float* __restrict
     const int bj = bi + t;
     const int64_t i0 = (int64_t)bi * BM, j0 = (int64_t)bj * BM;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    // slab loader: thread -> (row kk = tid / 32, columns 4 (tid % 32) .. + 3) of each operand
-    const int lk = threadIdx.x >> 5, lc = 4 * (threadIdx.x & 31);
-    const bool ai = i0 + lc < p, bj_ok = j0 + lc < p;          // p % 4 == 0: a vector is all in or all out
-    float acc[8][8];
+    // slab loader: VEC: vector u of thread t is row t / (BM / 4) + u 1024 / BM, columns
+    // 4 (t % (BM / 4)) .. + 3; else element u is row t / BM + u 256 / BM, column t % BM
+    constexpr int PR = VEC ? BM / 4 : BM, RS = 256 / PR;
+    const int lk = threadIdx.x / PR, lc = (threadIdx.x % PR) * (VEC ? 4 : 1);
+    const bool ai = i0 + lc < p, bj_ok = j0 + lc < p;          // VEC: p % 4 == 0, a vector is all in or all out
+    float ra[L], rb[L];
+    auto load = [&](int64_t k0) {
+        if constexpr (VEC) {
 #pragma unroll
-    for (int a = 0; a < 8; ++a)
+            for (int u = 0; u < L / 4; ++u) {
+                const int64_t k = k0 + lk + RS * u;
+                const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4 va = k < n && ai ? load4<TX>(X + k * p + i0 + lc) : z;
+                const float4 vb = k < n && bj_ok ? load4<TX>(X + k * p + j0 + lc) : z;
+                ra[4 * u] = va.x; ra[4 * u + 1] = va.y; ra[4 * u + 2] = va.z; ra[4 * u + 3] = va.w;
+                rb[4 * u] = vb.x; rb[4 * u + 1] = vb.y; rb[4 * u + 2] = vb.z; rb[4 * u + 3] = vb.w;
+            }
+        } else {
 #pragma unroll
-        for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
-    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 ra = z4, rb = z4;
-    if (lk < n) {
-        if (ai) ra = load4<TX>(X + (int64_t)lk * p + i0 + lc);
-        if (bj_ok) rb = load4<TX>(X + (int64_t)lk * p + j0 + lc);
-    }
-    *reinterpret_cast<float4*>(&As[0][lk][lc]) = ra;
-    *reinterpret_cast<float4*>(&Bs[0][lk][lc]) = rb;
+            for (int u = 0; u < L; ++u) {
+                const int64_t k = k0 + lk + RS * u;
+                ra[u] = k < n && ai ? load_as<TX, float>(X + k * p + i0 + lc) : 0.f;
+                rb[u] = k < n && bj_ok ? load_as<TX, float>(X + k * p + j0 + lc) : 0.f;
+            }
+        }
+    };
+    auto store = [&](int b) {
+        if constexpr (VEC) {
+#pragma unroll
+            for (int u = 0; u < L / 4; ++u) {
+                *reinterpret_cast<float4*>(&As[b][lk + RS * u][lc]) =
+                    make_float4(ra[4 * u], ra[4 * u + 1], ra[4 * u + 2], ra[4 * u + 3]);
+                *reinterpret_cast<float4*>(&Bs[b][lk + RS * u][lc]) =
+                    make_float4(rb[4 * u], rb[4 * u + 1], rb[4 * u + 2], rb[4 * u + 3]);
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < L; ++u) {
+                As[b][lk + RS * u][lc] = ra[u];
+                Bs[b][lk + RS * u][lc] = rb[u];
+            }
+        }
+    };
+    unsigned long long acc[TM][TM / 2];
+#pragma unroll
+    for (int q = 0; q < TM; ++q)
+#pragma unroll
+        for (int r = 0; r < TM / 2; ++r) acc[q][r] = 0ull;
+    load(0);
+    store(0);
     __syncthreads();
     int buf = 0;
     for (int64_t k0 = 0; k0 < n; k0 += BK) {
-        const int64_t kn = k0 + BK + lk;
         const bool more = k0 + BK < n;
-        ra = z4;
-        rb = z4;
-        if (more && kn < n) {
-            if (ai) ra = load4<TX>(X + kn * p + i0 + lc);
-            if (bj_ok) rb = load4<TX>(X + kn * p + j0 + lc);
-        }
+        if (more) load(k0 + BK);
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][4 * ty]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][64 + 4 * ty]);
-            const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][4 * tx]);
-            const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][kk][64 + 4 * tx]);
-            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+            float a[TM];
+            unsigned long long b[TM / 2];
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
+            for (int h = 0; h < H; ++h) {
+                const float4 v = *reinterpret_cast<const float4*>(&As[buf][kk][64 * h + 4 * ty]);
+                a[4 * h] = v.x; a[4 * h + 1] = v.y; a[4 * h + 2] = v.z; a[4 * h + 3] = v.w;
+                const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][64 * h + 4 * tx]);
+                b[2 * h] = w.x; b[2 * h + 1] = w.y;
+            }
 #pragma unroll
-                for (int r = 0; r < 8; ++r) acc[q][r] = __fmaf_rn(a[q], b[r], acc[q][r]);
+            for (int q = 0; q < TM; ++q) {
+                const unsigned long long aa = dup2(a[q]);
+#pragma unroll
+                for (int r = 0; r < TM / 2; ++r) fma2(acc[q][r], aa, b[r]);
+            }
         }
-        if (more) {
-            *reinterpret_cast<float4*>(&As[buf ^ 1][lk][lc]) = ra;
-            *reinterpret_cast<float4*>(&Bs[buf ^ 1][lk][lc]) = rb;
-        }
+        if (more) store(buf ^ 1);
         __syncthreads();
         buf ^= 1;
     }
     const float dn = (float)n;
-    // rows (columns) q < 4 at 4 ty + q, q >= 4 at 64 + 4 ty + q - 4; p % 4 == 0, so each
-    // group of four is all inside or all outside
-    const int64_t ia[2] = {i0 + 4 * ty, i0 + 64 + 4 * ty};
-    const int64_t ja[2] = {j0 + 4 * tx, j0 + 64 + 4 * tx};
+    float v[TM][TM];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int64_t i = ia[q >> 2] + (q & 3);
-        if (i >= p) continue;
+    for (int q = 0; q < TM; ++q)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (ja[h] < p)
-                *reinterpret_cast<float4*>(S + i * lds + ja[h]) =
-                    make_float4(acc[q][4 * h] / dn, acc[q][4 * h + 1] / dn, acc[q][4 * h + 2] / dn,
-                                acc[q][4 * h + 3] / dn);
+        for (int r = 0; r < TM / 2; ++r) {
+            v[q][2 * r] = __uint_as_float((unsigned)acc[q][r]) / dn;
+            v[q][2 * r + 1] = __uint_as_float((unsigned)(acc[q][r] >> 32)) / dn;
         }
-    }
-    if (bi != bj) {
-        // the mirror S[j, i] = S[i, j]: row j of the lower tile gets this thread's column r
+    // row (column) q of the thread is 64 (q / 4) + 4 ty (tx) + q % 4 of the tile
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            const int64_t j = ja[r >> 2] + (r & 3);
-            if (j >= p) continue;
+    for (int q = 0; q < TM; ++q) {
+        const int64_t i = i0 + 64 * (q >> 2) + 4 * ty + (q & 3), j = j0 + 64 * (q >> 2) + 4 * tx + (q & 3);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (ia[h] < p)
-                    *reinterpret_cast<float4*>(S + j * lds + ia[h]) =
-                        make_float4(acc[4 * h][r] / dn, acc[4 * h + 1][r] / dn, acc[4 * h + 2][r] / dn,
-                                    acc[4 * h + 3][r] / dn);
+        for (int h = 0; h < H; ++h) {
+            const int64_t jc = j0 + 64 * h + 4 * tx, ic = i0 + 64 * h + 4 * ty;
+            if constexpr (VEC) {         // a group of four is all inside or all outside
+                if (i < p && jc < p)
+                    *reinterpret_cast<float4*>(S + i * lds + jc) =
+                        make_float4(v[q][4 * h], v[q][4 * h + 1], v[q][4 * h + 2], v[q][4 * h + 3]);
+                // the mirror: row j of the lower tile gets this thread's column q
+                if (bi != bj && j < p && ic < p)
+                    *reinterpret_cast<float4*>(S + j * lds + ic) =
+                        make_float4(v[4 * h][q], v[4 * h + 1][q], v[4 * h + 2][q], v[4 * h + 3][q]);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (i < p && jc + u < p) S[i * lds + jc + u] = v[q][4 * h + u];
+                    if (bi != bj && j < p && ic + u < p) S[j * lds + ic + u] = v[4 * h + u][q];
+                }
             }
         }
     }
 }
 
-template <typename TX>
-cudaError_t run_v4(const void* X, int64_t n, int64_t p, void* S, int64_t lds, cudaStream_t s) {
-    const int nb = (int)((p + 127) / 128);
-    const long long tiles = (long long)nb * (nb + 1) / 2;
-    k_gram_simt_v4<TX><<<(unsigned)tiles, 256, 0, s>>>(static_cast<const TX*>(X), n, p, static_cast<float*>(S), lds,
-                                                        nb);
+template <typename TX, int TM>
+cudaError_t run_f32_t(const void* X, int64_t n, int64_t p, float* S, int64_t lds, bool vec, cudaStream_t s) {
+    const int64_t nb = (p + 16 * TM - 1) / (16 * TM);
+    const unsigned tiles = (unsigned)(nb * (nb + 1) / 2);
+    if constexpr (!std::is_same<TX, double>::value) {
+        if (vec) {
+            k_gram_simt_f32<TX, TM, true><<<tiles, 256, 0, s>>>(static_cast<const TX*>(X), n, p, S, lds, (int)nb);
+            return cudaGetLastError();
+        }
+    }
+    k_gram_simt_f32<TX, TM, false><<<tiles, 256, 0, s>>>(static_cast<const TX*>(X), n, p, S, lds, (int)nb);
     return cudaGetLastError();
+}
+
+template <typename TX>
+cudaError_t run_f32(const void* X, int64_t n, int64_t p, void* S, int64_t lds, cudaStream_t s) {
+    const bool vec = p % 4 == 0 && lds % 4 == 0 && reinterpret_cast<uintptr_t>(S) % 16 == 0 &&
+                     reinterpret_cast<uintptr_t>(X) % (4 * sizeof(TX)) == 0;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // 64 x 64 tiles where 128 x 128 ones would leave a third of the SMs without one, or give a few
+    // of them a second one (n = 600, us, 64 against 128: p = 1001 35, 84; p = 1500 45, 70; p = 2000
+    // 86, 70; p = 2200 107, 121; p = 3001 above 150, 150)
+    const int64_t nb = (p + 127) / 128, t = nb * (nb + 1) / 2;
+    const bool small = 3 * t < 2 * sms || (t > sms && 7 * t < 8 * sms);
+    return small ? run_f32_t<TX, 4>(X, n, p, static_cast<float*>(S), lds, vec, s)
+                 : run_f32_t<TX, 8>(X, n, p, static_cast<float*>(S), lds, vec, s);
 }
 
 template <typename TX, typename T, int TM>
@@ -227,12 +299,9 @@ cudaError_t gram_simt(const void* X, int xdt, int64_t n, int64_t p, void* S, int
         if (xdt == HPC_F32) return run<float, double, 4>(X, n, p, S, lds, s);
         return run<__nv_bfloat16, double, 4>(X, n, p, S, lds, s);
     }
-    if (xdt == HPC_F64) return run<double, float, 8>(X, n, p, S, lds, s);
-    // the vector form needs 16-byte (8-byte for BF16) aligned rows of X and S
-    const bool vec = p % 4 == 0 && lds % 4 == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0 &&
-                     (reinterpret_cast<uintptr_t>(X) & (xdt == HPC_F32 ? 15 : 7)) == 0;
-    if (xdt == HPC_F32) return vec ? run_v4<float>(X, n, p, S, lds, s) : run<float, float, 8>(X, n, p, S, lds, s);
-    return vec ? run_v4<__nv_bfloat16>(X, n, p, S, lds, s) : run<__nv_bfloat16, float, 8>(X, n, p, S, lds, s);
+    if (xdt == HPC_F64) return run_f32<double>(X, n, p, S, lds, s);
+    if (xdt == HPC_F32) return run_f32<float>(X, n, p, S, lds, s);
+    return run_f32<__nv_bfloat16>(X, n, p, S, lds, s);
 }
 
 }  // namespace hpc
