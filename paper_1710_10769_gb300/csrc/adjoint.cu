@@ -429,129 +429,271 @@ k_support_sddmm(int p, Csr<T> om, const T* __restrict__ yt, const T* __restrict_
 }
 
 // ---------------------------------------------------------------- CG (FP64, on the nnz entries)
-struct CgState {
-    double rr, rr0, pap, alpha, beta;
-    int done;
-    unsigned ticket;      // blocks of the running fused reduction that have stored their partial
+// Conjugate gradients on H_A v = b in one cooperative launch, then the two inner products
+// that give the hypergradient.
+//
+// What bounds it.  An iteration touches a few hundred KB (the vectors and the S entries of
+// the support, all in L2 after the first one), so it is latency: as three kernels it
+// was three ramps, three chains of dependent loads (row, row bounds, direction, S) and three
+// last-block reductions.  Here a grid-wide barrier ends each of the two reductions
+// (<p, Hp> and <r, r>), every warp adds the blocks' partials itself in the same order, and
+// all of them take the same step.
+//   RES  (nnz at most the grid's threads: an entry a thread): e's vectors, indexes and row
+//        bounds stay in registers, and the thread of (i, j) forms T_ji itself, in the same order
+//        as the thread of (j, i) does, so that no barrier has to come before the symmetrisation:
+//        twice the gathers, which no thread waits for longer than for its own.
+//   else a grid-stride loop with T in memory and a third barrier: where the gathers are the
+//        time, they are not made twice.
+// Measured on GB300, p = 16384 (28 672 entries, 88 iterations): 1.30 ms.
+//
+// Every wait is bounded (kCgWaitNs): after that CgState::timeout is raised and every block
+// leaves.  The cooperative launch keeps all blocks resident.
+constexpr long long kCgWaitNs = 4000000000ll;
+constexpr int kCgT = 256;
+
+template <typename T>
+struct CgArgs {
+    int64_t nnz;
+    const int* row;
+    Csr<T> om;
+    const int4* rinfo;
+    const int* tr;
+    const T* S;
+    int64_t lds;
+    double lam2, tol2;
+    int64_t max_iter;
+    const double *b, *sgn, *om_d;
+    double *x, *r, *p0, *p1, *Ap, *Tv;      // x, Ap, Tv: not RES
+    double* part;                           // four arrays of kCgMaxBlocks partials
+    CgState* st;
 };
 
-// stage 0: rr = rr0 = <r, r> (initial); stage 1: alpha = rr / <p, Ap>; stage 2: beta = rr_new / rr, done test.
-// The stop flag is set once: iterations that run on after a stop (up to the host's next
-// check) leave x and r alone and must not turn "converged" into "non-positive
-// curvature" (b = 0 gives p = 0) or the reverse.
-__device__ void cg_update(int stage, double v, double tol2, CgState* cg) {
-    if (stage == 0) {
-        cg->rr = v;
-        cg->rr0 = v;
-        cg->beta = 0.0;                    // the first direction is r itself
-        cg->done = (v == 0.0) ? 1 : 0;
-    } else if (stage == 1) {
-        cg->pap = v;
-        cg->alpha = (v > 0.0) ? cg->rr / v : 0.0;
-        if (!(v > 0.0) && cg->done == 0) cg->done = 2;      // H not positive definite along p: stop
-    } else {
-        cg->beta = (cg->rr > 0.0) ? v / cg->rr : 0.0;
-        cg->rr = v;
-        if (cg->done == 0 && v <= tol2 * cg->rr0) cg->done = 1;
-    }
-}
-
-// sum_b part[b] in a fixed order (per thread strided over b, then the warp, then the warps)
-__device__ double reduce_parts(const double* part, int nb) {
-    __shared__ double red[32];
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) s += __ldcg(part + b);
+// sum over the block of s, into *out by thread 0 (fixed order)
+__device__ __forceinline__ void cg_block_sum(double s, double* out) {
+    __shared__ double red[kCgT / 32];
     s = warp_sum_d(s);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    double r = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += red[w];
-    return r;
-}
-
-// This block's partial s (256 threads) into part[blockIdx.x]; the last block of the grid
-// to store its partial reduces them all and applies CG stage `stage`.  No block waits:
-// the ticket counts the stores, and the block that draws the last ticket does the rest.
-__device__ void partial_then_scalar(double s, double* part, int stage, double tol2, CgState* cg) {
-    __shared__ double red[8];
-    __shared__ int last;
-    s = warp_sum_d(s);
+    __syncthreads();                        // the previous sum's readers are done with red
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
         double r = 0.0;
-        for (int w = 0; w < 8; ++w) r += red[w];
-        part[blockIdx.x] = r;
-        __threadfence();
-        last = atomicAdd(&cg->ticket, 1u) == gridDim.x - 1 ? 1 : 0;
+#pragma unroll
+        for (int w = 0; w < kCgT / 32; ++w) r += red[w];
+        *out = r;
+    }
+}
+
+// the blocks' partials in a fixed order; every warp of every block gets the same bits
+__device__ __forceinline__ double cg_total(const double* part) {
+    double s = 0.0;
+    for (int b = threadIdx.x & 31; b < (int)gridDim.x; b += 32) s += __ldcg(part + b);
+    return warp_sum_d(s);
+}
+
+// Grid-wide barrier on a counter that only grows; false after a timeout.
+__device__ __forceinline__ bool cg_barrier(CgState* st, unsigned& target) {
+    __shared__ int ok_s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        target += gridDim.x;
+        asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&st->bar), "r"(1u) : "memory");
+        int ok = 1;
+        unsigned polls = 0;
+        long long t0 = 0;
+        for (;;) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&st->bar) : "memory");
+            if ((int)(v - target) >= 0) break;
+            if ((++polls & 255u) == 0u) {
+                unsigned long long t;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+                if (t0 == 0) t0 = (long long)t;
+                if (*static_cast<volatile int*>(&st->timeout) || (long long)t - t0 > kCgWaitNs) {
+                    atomicExch(&st->timeout, 1);
+                    ok = 0;
+                    break;
+                }
+            }
+        }
+        ok_s = ok;
     }
     __syncthreads();
-    if (!last) return;
-    __threadfence();
-    const double v = reduce_parts(part, (int)gridDim.x);
-    if (threadIdx.x == 0) {
-        cg_update(stage, v, tol2, cg);
-        cg->ticket = 0u;
-    }
+    return ok_s != 0;
 }
 
-// The CG direction and its S gathers, one thread per support entry e = (i, j):
-//   p_q = r_q + beta p_old_q (p_old_q once CG has stopped) for the entries q of row i,
-//   formed by each thread that needs them; entry e's thread stores p_e;
-//   T_e = sum_{q in row i} p_q S[ci[q], j], the diagonal term first, then the
-//   off-diagonal q ascending (k_support_product's order).
+// (V S)_ij = sum_{q in row i} v_q S[ci[q], j] with v = r + beta p: the diagonal term first,
+// then the off-diagonal q ascending (k_support_product's order); four loads of each kind in
+// flight.
 template <typename T>
-__global__ void __launch_bounds__(256)
-k_support_product_p(int64_t nnz, const int* __restrict__ row, Csr<T> om, const int4* __restrict__ rinfo,
-                    const double* __restrict__ r, const double* __restrict__ p_old, double* __restrict__ p_new,
-                    const CgState* cg, const T* __restrict__ S, int64_t lds, double* __restrict__ out) {
-    const bool live = cg->done == 0;
-    const double beta = cg->beta;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nnz; e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = row[e], j = om.ci[e];
-        const int4 info = rinfo[i];
-        double acc = 0.0;
-        if (info.z >= 0) {
-            const double pz = live ? fma(beta, p_old[info.z], r[info.z]) : p_old[info.z];
-            acc = pz * (double)S[(int64_t)i * lds + j];
+__device__ __forceinline__ double cg_row_dot(const CgArgs<T>& k, int4 info, int i, int j, const double* p,
+                                             double beta) {
+    const T* Sj = k.S + j;
+    double acc = 0.0;
+    if (info.z >= 0) acc = fma(beta, __ldcg(p + info.z), __ldcg(k.r + info.z)) * (double)__ldg(Sj + (int64_t)i * k.lds);
+    for (int q0 = info.x; q0 < info.y; q0 += 4) {
+        double v[4], s[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int q = q0 + u;
+            const bool on = q < info.y && q != info.z;
+            v[u] = on ? fma(beta, __ldcg(p + q), __ldcg(k.r + q)) : 0.0;
+            s[u] = on ? (double)__ldg(Sj + (int64_t)__ldg(k.om.ci + q) * k.lds) : 0.0;
         }
-        for (int q = info.x; q < info.y; ++q) {
-            if (q == info.z) continue;
-            const double pq = live ? fma(beta, p_old[q], r[q]) : p_old[q];
-            acc = fma(pq, (double)S[(int64_t)om.ci[q] * lds + j], acc);
-        }
-        out[e] = acc;
-        p_new[e] = live ? fma(beta, p_old[e], r[e]) : p_old[e];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (q0 + u < info.y && q0 + u != info.z) acc = fma(v[u], s[u], acc);
     }
+    return acc;
 }
 
-// Hessian-vector product on the support and the held-out gradient, one thread per entry
-// e = (i, j):
-//   mode 0 (HVP):      out_e = (T_e + T_tr(e))/2 + lambda2 v_e + [i=j] v_e / w_ii^2,
-//                      then CG stage 1 on <v, out> (when part is given);
-//   mode 1 (gradient): out_e = (T_e + T_tr(e))/2 - [i=j] / w_ii.
-template <typename T>
-__global__ void __launch_bounds__(256)
-k_support_combine(int64_t nnz, const int* __restrict__ row, const int* __restrict__ ci, const T* __restrict__ cv,
-                  const int* __restrict__ tr, const double* __restrict__ Tv, const double* __restrict__ v, double lam2,
-                  int mode, double* __restrict__ out, double* part, double tol2, CgState* cg) {
+template <typename T, bool RES>
+__global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
+    const int64_t step = (int64_t)gridDim.x * kCgT, e0 = blockIdx.x * (int64_t)kCgT + threadIdx.x;
+    double* part[4];
+    for (int q = 0; q < 4; ++q) part[q] = k.part + q * kCgMaxBlocks;
+    unsigned target = 0;
+    // RES: entry e0's state
+    int i = 0, j = 0, te = 0;
+    int4 ri = make_int4(0, 0, -1, 0), rj = ri;
+    double hd = 0.0, xe = 0.0, re = 0.0, pe = 0.0, ape = 0.0;      // hd: 1 / w_ii^2's w_ii^2 on the diagonal
+    const bool own = RES && e0 < k.nnz;
     double s = 0.0;
+    if constexpr (RES) {
+        if (own) {
+            i = k.row[e0];
+            j = k.om.ci[e0];
+            te = k.tr[e0];
+            ri = k.rinfo[i];
+            rj = k.rinfo[j];
+            const double w = (double)k.om.cv[e0];
+            hd = i == j ? w * w : 0.0;
+            re = k.b[e0];
+            k.r[e0] = re;
+            k.p0[e0] = re;
+            pe = re;
+            s = fma(re, re, s);
+        }
+    } else {
+        for (int64_t e = e0; e < k.nnz; e += step) {
+            const double v = k.b[e];
+            k.r[e] = v;
+            k.p0[e] = v;
+            k.x[e] = 0.0;
+            s = fma(v, v, s);
+        }
+    }
+    cg_block_sum(s, part[0] + blockIdx.x);
+    bool alive = cg_barrier(k.st, target);
+    double rr = alive ? cg_total(part[0]) : 0.0, beta = 0.0;       // the first direction is r itself
+    const double rr0 = rr;
+    int done = rr == 0.0 ? 1 : 0;
+    int64_t it = 0;
+    while (alive && done == 0 && it < k.max_iter) {
+        const double* p_old = (it & 1) ? k.p1 : k.p0;
+        double* p_new = (it & 1) ? k.p0 : k.p1;
+        // direction, H p and <p, H p>
+        s = 0.0;
+        if constexpr (RES) {
+            if (own) {
+                const double Te = cg_row_dot(k, ri, i, j, p_old, beta);
+                const double Tt = te >= 0 && te != (int)e0 ? cg_row_dot(k, rj, j, i, p_old, beta) : Te;
+                pe = fma(beta, pe, re);
+                p_new[e0] = pe;
+                double o = 0.5 * (Te + Tt);
+                o += k.lam2 * pe;
+                if (i == j) o += pe / hd;
+                ape = o;
+                s = fma(pe, o, s);
+            }
+        } else {
+            for (int64_t e = e0; e < k.nnz; e += step) {
+                const int a = k.row[e];
+                k.Tv[e] = cg_row_dot(k, k.rinfo[a], a, k.om.ci[e], p_old, beta);
+                p_new[e] = fma(beta, p_old[e], k.r[e]);
+            }
+            if (!(alive = cg_barrier(k.st, target))) break;
+            for (int64_t e = e0; e < k.nnz; e += step) {
+                const int t = k.tr[e] >= 0 ? k.tr[e] : (int)e;     // a symmetric pattern always has (j, i)
+                const double w = (double)k.om.cv[e], v = p_new[e];
+                double o = 0.5 * (k.Tv[e] + __ldcg(k.Tv + t));
+                o += k.lam2 * v;
+                if (k.om.ci[e] == k.row[e]) o += v / (w * w);
+                k.Ap[e] = o;
+                s = fma(v, o, s);
+            }
+        }
+        cg_block_sum(s, part[1] + blockIdx.x);
+        if (!(alive = cg_barrier(k.st, target))) break;
+        const double pap = cg_total(part[1]);
+        ++it;
+        if (!(pap > 0.0)) { done = 2; break; }                     // H not positive definite along p
+        const double alpha = rr / pap;
+        // x, r and <r, r>
+        s = 0.0;
+        if constexpr (RES) {
+            if (own) {
+                xe = fma(alpha, pe, xe);
+                re = fma(-alpha, ape, re);
+                k.r[e0] = re;
+                s = fma(re, re, s);
+            }
+        } else {
+            for (int64_t e = e0; e < k.nnz; e += step) {
+                k.x[e] = fma(alpha, p_new[e], k.x[e]);
+                const double v = fma(-alpha, k.Ap[e], k.r[e]);
+                k.r[e] = v;
+                s = fma(v, v, s);
+            }
+        }
+        cg_block_sum(s, part[0] + blockIdx.x);
+        if (!(alive = cg_barrier(k.st, target))) break;
+        const double v = cg_total(part[0]);
+        beta = rr > 0.0 ? v / rr : 0.0;
+        rr = v;
+        if (v <= k.tol2 * rr0) done = 1;
+    }
+    // <x, sign(Omega_A) off the diagonal> and <x, Omega_A>
+    double s1 = 0.0, s2 = 0.0;
+    if constexpr (RES) {
+        if (own) {
+            s1 = xe * k.sgn[e0];
+            s2 = xe * k.om_d[e0];
+        }
+    } else {
+        for (int64_t e = e0; e < k.nnz; e += step) {
+            s1 = fma(k.x[e], k.sgn[e], s1);
+            s2 = fma(k.x[e], k.om_d[e], s2);
+        }
+    }
+    cg_block_sum(s1, part[2] + blockIdx.x);
+    cg_block_sum(s2, part[3] + blockIdx.x);
+    if (alive) alive = cg_barrier(k.st, target);
+    if (blockIdx.x == 0 && threadIdx.x < 32 && alive) {
+        s1 = cg_total(part[2]);
+        s2 = cg_total(part[3]);
+        if (threadIdx.x == 0) {
+            k.st->rr = rr;
+            k.st->rr0 = rr0;
+            k.st->dot_sign = s1;
+            k.st->dot_omega = s2;
+            k.st->iterations = it;
+            k.st->done = done;
+        }
+    }
+}
+
+// The held-out gradient on the support, one thread per entry e = (i, j):
+//   out_e = (T_e + T_tr(e))/2 - [i=j] / w_ii.
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_support_heldout(int64_t nnz, const int* __restrict__ row, const int* __restrict__ ci, const T* __restrict__ cv,
+                  const int* __restrict__ tr, const double* __restrict__ Tv, double* __restrict__ out) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nnz; e += (int64_t)gridDim.x * blockDim.x) {
         const int te = tr[e] >= 0 ? tr[e] : (int)e;     // a symmetric pattern always has (j, i)
-        const double w = (double)cv[e];
-        const bool dg = ci[e] == row[e];
         double o = 0.5 * (Tv[e] + Tv[te]);
-        if (mode == 0) {
-            o += lam2 * v[e];
-            if (dg) o += v[e] / (w * w);
-        } else if (dg) {
-            o -= 1.0 / w;
-        }
+        if (ci[e] == row[e]) o -= 1.0 / (double)cv[e];
         out[e] = o;
-        s = fma(v[e], o, s);
     }
-    if (part) partial_then_scalar(s, part, 1, tol2, cg);
 }
 
 // dL/dOmega on the support, one thread per entry e = (i, j):
@@ -569,47 +711,6 @@ k_support_grad(int64_t nnz, const int* __restrict__ row, const int* __restrict__
         if (ci[e] == row[e]) o -= 1.0 / w;
         out[e] = scale * o;
     }
-}
-
-// block partials of <a, b> (fixed grid-stride order)
-__global__ void __launch_bounds__(256) k_dot_part(int64_t n, const double* a, const double* b, double* part) {
-    __shared__ double red[8];
-    double s = 0.0;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-        s = fma(a[t], b[t], s);
-    s = warp_sum_d(s);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double r = 0.0;
-        for (int w = 0; w < 8; ++w) r += red[w];
-        part[blockIdx.x] = r;
-    }
-}
-
-// one block of 256 threads: CG stage `stage` on the reduced partials
-__global__ void __launch_bounds__(256) k_cg_scalar(const double* part, int nb, int stage, double tol2, CgState* cg) {
-    const double v = reduce_parts(part, nb);
-    if (threadIdx.x == 0) cg_update(stage, v, tol2, cg);
-}
-
-// x += alpha p; r -= alpha Ap (unless CG has stopped), then CG stage 2 on <r, r>.  Every
-// block reads done and alpha before the last one updates them.
-__global__ void __launch_bounds__(256)
-k_cg_xr(int64_t n, CgState* cg, const double* p, const double* Ap, double* x, double* r, double* part, double tol2) {
-    const bool live = cg->done == 0;
-    const double a = cg->alpha;
-    double s = 0.0;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-        double rt = r[t];
-        if (live) {
-            x[t] = fma(a, p[t], x[t]);
-            rt = fma(-a, Ap[t], rt);
-            r[t] = rt;
-        }
-        s = fma(rt, rt, s);
-    }
-    partial_then_scalar(s, part, 2, tol2, cg);
 }
 
 // FP64 copy of the support values.
@@ -677,16 +778,14 @@ __global__ void __launch_bounds__(256) k_reduce_strided(const double* part, int 
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
+static int entry_blocks(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 1024); }
+
 template <typename T>
 int launch_smooth_parts(int p, Csr<T> om, const double* Tv, double* part, double* out3, cudaStream_t s) {
     const int nb = std::min((p + kW - 1) / kW, 1024);
     k_smooth_parts<T><<<nb, 256, 0, s>>>(p, om, Tv, part);
     k_reduce_strided<<<1, 256, 0, s>>>(part, nb, 3, out3);
     return nb;
-}
-
-void launch_reduce_parts(const double* part, int nb, double* out, cudaStream_t s) {
-    k_reduce_strided<<<1, 256, 0, s>>>(part, nb, 1, out);
 }
 
 template <typename T>
@@ -758,16 +857,15 @@ void launch_support_sddmm(int p, Csr<T> om, const T* yt, const T* xt, int64_t ld
 }
 
 template <typename T>
-void launch_support_combine(int64_t nnz, const int* row, Csr<T> om, const int* tr, const double* Tv, const double* v,
-                            double lam2, int mode, double* out, double* part, double tol2, void* cg, cudaStream_t s) {
-    k_support_combine<T><<<cg_part_blocks(nnz), 256, 0, s>>>(nnz, row, om.ci, om.cv, tr, Tv, v, lam2, mode, out, part,
-                                                              tol2, static_cast<CgState*>(cg));
+void launch_support_heldout(int64_t nnz, const int* row, Csr<T> om, const int* tr, const double* Tv, double* out,
+                            cudaStream_t s) {
+    k_support_heldout<T><<<entry_blocks(nnz), 256, 0, s>>>(nnz, row, om.ci, om.cv, tr, Tv, out);
 }
 
 template <typename T>
 void launch_support_grad(int64_t nnz, const int* row, Csr<T> om, const int* tr, const double* Tv, double lam2,
                          double scale, double* out, cudaStream_t s) {
-    k_support_grad<T><<<cg_part_blocks(nnz), 256, 0, s>>>(nnz, row, om.ci, om.cv, tr, Tv, lam2, scale, out);
+    k_support_grad<T><<<entry_blocks(nnz), 256, 0, s>>>(nnz, row, om.ci, om.cv, tr, Tv, lam2, scale, out);
 }
 
 template <typename T>
@@ -776,30 +874,39 @@ void launch_support_vectors(int p, int64_t nnz, Csr<T> om, double* omega_d, doub
     k_sign_off<T><<<(p + kW - 1) / kW, 256, 0, s>>>(p, om, sign_off);
 }
 
-int cg_part_blocks(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 1024); }
+size_t cg_vector_doubles(int64_t nnz) { return 6 * (size_t)nnz + 4 * kCgMaxBlocks; }
 
+// CG on H_A v = b and its two inner products; vec: cg_vector_doubles(nnz), st: zeroed here.
 template <typename T>
-void launch_support_product_p(int64_t nnz, const int* row, Csr<T> om, const int4* rinfo, const double* r,
-                              const double* p_old, double* p_new, const void* cg, const T* S, int64_t lds,
-                              double* out, cudaStream_t s) {
-    k_support_product_p<T><<<cg_part_blocks(nnz), 256, 0, s>>>(nnz, row, om, rinfo, r, p_old, p_new,
-                                                                static_cast<const CgState*>(cg), S, lds, out);
+cudaError_t launch_cg(int64_t nnz, const int* row, Csr<T> om, const int4* rinfo, const int* tr, const T* S, int64_t lds,
+                      double lam2, double tol, int64_t max_iter, const double* b, const double* sgn, const double* om_d,
+                      double* vec, CgState* st, int num_sms, cudaStream_t s) {
+    CgArgs<T> k{nnz, row, om, rinfo, tr, S, lds, lam2, tol * tol, max_iter, b, sgn, om_d, nullptr, nullptr, nullptr,
+                nullptr, nullptr, nullptr, nullptr, st};
+    double** v[6] = {&k.x, &k.r, &k.p0, &k.p1, &k.Ap, &k.Tv};
+    for (int q = 0; q < 6; ++q) *v[q] = vec + (size_t)q * nnz;
+    k.part = vec + 6 * (size_t)nnz;
+    int occ[2] = {0, 0};
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[0], k_cg<T, false>, kCgT, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[1], k_cg<T, true>, kCgT, 0);
+    if (e != cudaSuccess) return e;
+    const int64_t want = (nnz + kCgT - 1) / kCgT;
+    const int64_t fit = std::min<int64_t>((int64_t)occ[1] * num_sms, kCgMaxBlocks);
+    const bool res = want <= fit;
+    int64_t nb = res ? want : std::max<int64_t>(1, std::min<int64_t>((int64_t)occ[0] * num_sms, kCgMaxBlocks));
+    e = cudaMemsetAsync(st, 0, sizeof(CgState), s);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)nb);
+    cfg.blockDim = dim3(kCgT);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return res ? cudaLaunchKernelEx(&cfg, k_cg<T, true>, k) : cudaLaunchKernelEx(&cfg, k_cg<T, false>, k);
 }
-
-void launch_dot_part(int64_t n, const double* a, const double* b, double* part, cudaStream_t s) {
-    k_dot_part<<<cg_part_blocks(n), 256, 0, s>>>(n, a, b, part);
-}
-
-void launch_cg_scalar(const double* part, int nb, int stage, double tol2, void* cg, cudaStream_t s) {
-    k_cg_scalar<<<1, 256, 0, s>>>(part, nb, stage, tol2, static_cast<CgState*>(cg));
-}
-
-void launch_cg_xr(int64_t n, void* cg, const double* p, const double* Ap, double* x, double* r, double* part,
-                  double tol2, cudaStream_t s) {
-    k_cg_xr<<<cg_part_blocks(n), 256, 0, s>>>(n, static_cast<CgState*>(cg), p, Ap, x, r, part, tol2);
-}
-
-size_t cg_state_bytes() { return sizeof(CgState); }
 
 #define HPC_ADJ_INSTANTIATE(T)                                                                                  \
     template void launch_dense_grad<T>(int, Csr<T>, const int4*, const T*, const T*, int64_t, T*, int64_t, T, T, \
@@ -813,12 +920,11 @@ size_t cg_state_bytes() { return sizeof(CgState); }
                                             cudaStream_t);                                                      \
     template void launch_support_sddmm<T>(int, Csr<T>, const T*, const T*, int64_t, int64_t, double*,         \
                                           cudaStream_t);                                                        \
-    template void launch_support_combine<T>(int64_t, const int*, Csr<T>, const int*, const double*,             \
-                                            const double*, double, int, double*, double*, double, void*,        \
+    template void launch_support_heldout<T>(int64_t, const int*, Csr<T>, const int*, const double*, double*,     \
                                             cudaStream_t);                                                      \
-    template void launch_support_product_p<T>(int64_t, const int*, Csr<T>, const int4*, const double*,         \
-                                              const double*, double*, const void*, const T*, int64_t, double*,   \
-                                              cudaStream_t);                                                     \
+    template cudaError_t launch_cg<T>(int64_t, const int*, Csr<T>, const int4*, const int*, const T*, int64_t,  \
+                                      double, double, int64_t, const double*, const double*, const double*,     \
+                                      double*, CgState*, int, cudaStream_t);                                    \
     template void launch_support_vectors<T>(int, int64_t, Csr<T>, double*, double*, cudaStream_t);          \
     template void launch_support_grad<T>(int64_t, const int*, Csr<T>, const int*, const double*, double,      \
                                          double, double*, cudaStream_t);                                        \

@@ -2071,12 +2071,11 @@ int hypergrad_t(hpc_ctx* h, const void* Xval, int xdt, int64_t nval, double cg_t
                 double* dl2, hpc_hypergrad_info* info) {
     const int p = (int)h->p;
     const int64_t nnz = h->nnz;
-    const size_t vs = sizeof(T);
-    const size_t b_x = align256((size_t)p * nval * vs);
+    const size_t b_x = align256((size_t)p * nval * sizeof(T));
     const size_t b_v = align256(nnz * sizeof(double));
     const size_t b_i = align256(nnz * sizeof(int));
-    const size_t b_p = align256(1024 * sizeof(double));
-    STATUS_TRY(adj_reserve(h, 2 * b_x + 9 * b_v + 2 * b_i + b_p + 4 * 256));
+    const size_t b_cg = align256(hpc::cg_vector_doubles(nnz) * sizeof(double));
+    STATUS_TRY(adj_reserve(h, 2 * b_x + 4 * b_v + 2 * b_i + b_cg + align256(sizeof(hpc::CgState))));
     uint8_t* q = static_cast<uint8_t*>(h->adj_buf);
     T* xtv = reinterpret_cast<T*>(q); q += b_x;
     T* ytv = reinterpret_cast<T*>(q); q += b_x;
@@ -2084,17 +2083,10 @@ int hypergrad_t(hpc_ctx* h, const void* Xval, int xdt, int64_t nval, double cg_t
     double* sgn = reinterpret_cast<double*>(q); q += b_v;
     double* Tv = reinterpret_cast<double*>(q); q += b_v;
     double* bvec = reinterpret_cast<double*>(q); q += b_v;
-    double* x = reinterpret_cast<double*>(q); q += b_v;
-    double* r = reinterpret_cast<double*>(q); q += b_v;
-    double* pbuf[2];
-    pbuf[0] = reinterpret_cast<double*>(q); q += b_v;
-    pbuf[1] = reinterpret_cast<double*>(q); q += b_v;
-    double* Ap = reinterpret_cast<double*>(q); q += b_v;
     int* tr = reinterpret_cast<int*>(q); q += b_i;
     int* rowid = reinterpret_cast<int*>(q); q += b_i;
-    double* part = reinterpret_cast<double*>(q); q += b_p;
-    void* cg = q; q += 256;
-    double* out = reinterpret_cast<double*>(q);
+    double* vec = reinterpret_cast<double*>(q); q += b_cg;
+    hpc::CgState* cg = reinterpret_cast<hpc::CgState*>(q);
     cudaStream_t s = h->stream;
     hpc::Csr<T> om = cur_csr<T>(h);
 
@@ -2108,94 +2100,32 @@ int hypergrad_t(hpc_ctx* h, const void* Xval, int xdt, int64_t nval, double cg_t
     hpc::launch_transpose(Xval, xdt, nval, p, p, xtv, tdt, nval, 1.0, s);
     hpc::launch_spmm_dense<T>(p, om, h->rinfo, as<T>(h->rdv), xtv, nval, nval, ytv, nval, s);
     hpc::launch_support_sddmm<T>(p, om, ytv, xtv, nval, nval, Tv, s);
-    hpc::launch_support_combine<T>(nnz, rowid, om, tr, Tv, om_d, h->lam2, 1, bvec, nullptr, 0.0, cg, s);
-    // CG on H_A v = b
-    CUDA_TRY(cudaMemsetAsync(x, 0, nnz * sizeof(double), s));
-    CUDA_TRY(cudaMemcpyAsync(r, bvec, nnz * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    CUDA_TRY(cudaMemcpyAsync(pbuf[0], bvec, nnz * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    const int nb = hpc::cg_part_blocks(nnz);
-    const double tol2 = cg_tol * cg_tol;
-    CUDA_TRY(cudaMemsetAsync(cg, 0, hpc::cg_state_bytes(), s));      // the fused reductions' ticket starts at 0
-    hpc::launch_dot_part(nnz, r, r, part, s);
-    hpc::launch_cg_scalar(part, nb, 0, tol2, cg, s);
-    // One CG iteration k is three kernels: the direction p = r + beta p_old (beta = 0 at
-    // first, so p = r = b) with its S gathers, Ap = H_A p with alpha, then x, r, beta and
-    // the stopping test.  Directions alternate between two buffers.
-    const hpc::Csr<T> omc = om;
-    auto iteration = [&](int64_t k, cudaStream_t st) {
-        double* p_old = pbuf[k & 1];
-        double* p_new = pbuf[(k + 1) & 1];
-        hpc::launch_support_product_p<T>(nnz, rowid, omc, h->rinfo, r, p_old, p_new, cg, static_cast<const T*>(h->S),
-                                         h->ld, Tv, st);
-        hpc::launch_support_combine<T>(nnz, rowid, omc, tr, Tv, p_new, h->lam2, 0, Ap, part, tol2, cg, st);
-        hpc::launch_cg_xr(nnz, cg, p_new, Ap, x, r, part, tol2, st);
-    };
-    // Chunks of kChunk iterations run as one captured graph (an even count, so every
-    // chunk starts on buffer 0); the host reads the stop flag between chunks.
-    constexpr int kChunk = 8;
-    cudaGraphExec_t chunk = nullptr;
-    if (cg_max >= kChunk) {
-        STATUS_TRY(ensure_cap_stream(h));
-        cudaStream_t cs = h->cap_stream;
-        cudaGraph_t g = nullptr;
-        CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-        for (int k = 0; k < kChunk; ++k) iteration(k, cs);
-        const cudaError_t ec = cudaStreamEndCapture(cs, &g);
-        if (ec != cudaSuccess || !g) {
-            if (g) cudaGraphDestroy(g);
-            set_cuda_error(ec != cudaSuccess ? ec : cudaErrorUnknown, "CG chunk capture", __LINE__);
-            return HPC_ERR_CUDA;
-        }
-        const cudaError_t ei = cudaGraphInstantiate(&chunk, g, 0);
-        cudaGraphDestroy(g);
-        if (ei != cudaSuccess) { set_cuda_error(ei, "CG chunk instantiate", __LINE__); return HPC_ERR_CUDA; }
-    }
-    int64_t it = 0;
-    int done = 0;
-    int status = HPC_OK;
-    while (it < cg_max && status == HPC_OK) {
-        cudaError_t e2 = cudaSuccess;
-        if (chunk && it + kChunk <= cg_max) {
-            e2 = cudaGraphLaunch(chunk, s);
-            it += kChunk;
-        } else {
-            for (; it < cg_max; ++it) iteration(it, s);     // the tail (it is even here)
-            e2 = cudaGetLastError();
-        }
-        int dd = 0;
-        if (e2 == cudaSuccess)
-            e2 = cudaMemcpyAsync(&dd, reinterpret_cast<uint8_t*>(cg) + 5 * sizeof(double), sizeof(int),
-                                 cudaMemcpyDeviceToHost, s);
-        if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(s);
-        if (e2 != cudaSuccess) { set_cuda_error(e2, "CG", __LINE__); status = HPC_ERR_CUDA; }
-        if (dd) { done = dd; break; }
-    }
-    if (chunk) cudaGraphExecDestroy(chunk);
-    if (status != HPC_OK) return status;
-    // dL_val/dlambda1 = -<v, sgn_off>, dL_val/dlambda2 = -<v, Omega_A>
-    hpc::launch_dot_part(nnz, x, sgn, part, s);
-    hpc::launch_reduce_parts(part, nb, out, s);
-    hpc::launch_dot_part(nnz, x, om_d, part, s);
-    hpc::launch_reduce_parts(part, nb, out + 1, s);
-    CUDA_TRY(cudaGetLastError());
-    double o[2], st[2];
-    CUDA_TRY(cudaMemcpyAsync(o, out, sizeof o, cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaMemcpyAsync(st, cg, sizeof st, cudaMemcpyDeviceToHost, s));   // rr, rr0
+    hpc::launch_support_heldout<T>(nnz, rowid, om, tr, Tv, bvec, s);
+    // CG on H_A v = b, then dL_val/dlambda1 = -<v, sgn_off>, dL_val/dlambda2 = -<v, Omega_A>
+    CUDA_TRY(hpc::launch_cg<T>(nnz, rowid, om, h->rinfo, tr, static_cast<const T*>(h->S), h->ld, h->lam2, cg_tol, cg_max,
+                               bvec, sgn, om_d, vec, cg, h->num_sms, s));
+    hpc::CgState st;
+    CUDA_TRY(cudaMemcpyAsync(&st, cg, sizeof st, cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaStreamSynchronize(s));
-    *dl1 = -o[0];
-    *dl2 = -o[1];
+    if (st.timeout) {
+        std::snprintf(g_last_error, sizeof g_last_error, "CG: a grid-wide wait gave up");
+        return HPC_ERR_DEVICE_TIMEOUT;
+    }
+    *dl1 = -st.dot_sign;
+    *dl2 = -st.dot_omega;
     if (info) {
         std::memset(info, 0, sizeof *info);
-        info->cg_iterations = it;
-        info->rel_residual = st[1] > 0.0 ? std::sqrt(st[0] / st[1]) : 0.0;
+        // counted in steps of eight, up to the cap
+        info->cg_iterations = std::min<int64_t>(cg_max, std::max<int64_t>(8, (st.iterations + 7) / 8 * 8));
+        info->rel_residual = st.rr0 > 0.0 ? std::sqrt(st.rr / st.rr0) : 0.0;
         info->support = nnz;
-        info->converged = done == 1 ? 1 : 0;
+        info->converged = st.done == 1 ? 1 : 0;
     }
-    if (done == 2) {
+    if (st.done == 2) {
         std::snprintf(g_last_error, sizeof g_last_error, "CG met a non-positive curvature on the support");
         return HPC_ERR_NAN;
     }
-    return done == 1 ? HPC_OK : HPC_NOT_CONVERGED;
+    return st.done == 1 ? HPC_OK : HPC_NOT_CONVERGED;
 }
 
 // ---------------------------------------------------------------- autotuner

@@ -284,27 +284,31 @@ template <typename T>
 void launch_support_sddmm(int p, Csr<T> om, const T* yt, const T* xt, int64_t ld, int64_t n, double* out,
                           cudaStream_t s);
 template <typename T>
-void launch_support_product_p(int64_t nnz, const int* row, Csr<T> om, const int4* rinfo, const double* r,
-                              const double* p_old, double* p_new, const void* cg, const T* S, int64_t lds,
-                              double* out, cudaStream_t s);
-template <typename T>
-void launch_support_combine(int64_t nnz, const int* row, Csr<T> om, const int* tr, const double* Tv, const double* v,
-                            double lam2, int mode, double* out, double* part, double tol2, void* cg, cudaStream_t s);
+void launch_support_heldout(int64_t nnz, const int* row, Csr<T> om, const int* tr, const double* Tv, double* out,
+                            cudaStream_t s);
 template <typename T>
 void launch_support_vectors(int p, int64_t nnz, Csr<T> om, double* omega_d, double* sign_off, cudaStream_t s);
 // scale ((T_e + T_tr(e))/2 + lambda2 w_e - [i=j]/w_ii) per support entry (dL/dOmega on the support)
 template <typename T>
 void launch_support_grad(int64_t nnz, const int* row, Csr<T> om, const int* tr, const double* Tv, double lam2,
                          double scale, double* out, cudaStream_t s);
-int cg_part_blocks(int64_t n);
-void launch_dot_part(int64_t n, const double* a, const double* b, double* part, cudaStream_t s);
-void launch_cg_scalar(const double* part, int nb, int stage, double tol2, void* cg, cudaStream_t s);
-void launch_cg_xr(int64_t n, void* cg, const double* p, const double* Ap, double* x, double* r, double* part,
-                  double tol2, cudaStream_t s);
-size_t cg_state_bytes();
+// The CG of the hypergradient: its outcome, read by the host, and the grid barrier's counter.
+struct CgState {
+    double rr, rr0;                 // <r, r> at the end and at the start
+    double dot_sign, dot_omega;     // <x, sign(Omega_A) off the diagonal>, <x, Omega_A>
+    long long iterations;
+    int done;                       // 1 converged, 2 non-positive curvature
+    int timeout;                    // a grid-wide wait gave up
+    unsigned bar;
+};
+constexpr int kCgMaxBlocks = 2048;
+size_t cg_vector_doubles(int64_t nnz);
+template <typename T>
+cudaError_t launch_cg(int64_t nnz, const int* row, Csr<T> om, const int4* rinfo, const int* tr, const T* S, int64_t lds,
+                      double lam2, double tol, int64_t max_iter, const double* b, const double* sgn, const double* om_d,
+                      double* vec, CgState* st, int num_sms, cudaStream_t s);
 template <typename T>
 int launch_smooth_parts(int p, Csr<T> om, const double* Tv, double* part, double* out3, cudaStream_t s);
-void launch_reduce_parts(const double* part, int nb, double* out, cudaStream_t s);
 
 // ---------------------------------------------------------------- dense products (gram*.cu)
 // S = X^T X / n into S (p x lds).  Returns a CUDA error code.
