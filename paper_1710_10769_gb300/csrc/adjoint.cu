@@ -206,50 +206,126 @@ __device__ __forceinline__ void pair_of(long long t, int nt, int& bi, int& bj) {
 
 // dL/dOmega = scale ((W + W^T)/2 + lambda2 Omega - diag(1/w_ii)), W = Omega S, on one pair
 // of TL x TL tiles (I <= J) per CTA, so G is written once and never re-read:
+//  0. the off-diagonal entries (k, w_ik) of the rows of I and J go into a list in shared memory,
+//     row by row; the first S segments that they need are requested at once;
 //  1. the tile S[I, J] is read once; it gives the diagonal terms of both W[I, J]
 //     (w_ii S_ij) and W[J, I] (w_jj S_ji = w_jj S_ij: S is bitwise symmetric);
-//  2. only the rows with off-diagonal entries (few: the iterate is sparse) add their
-//     gathered terms, one warp per row;
-//  3. G[I, J] = (W[I, J] + W[J, I]^T)/2, G[J, I] its transpose, then the support
-//     terms of the same rows, the scale, and 16-byte stores.
+//  2. the list's terms w_ik S[k, J] are added, k ascending: a group of TL / 4 (FP64: TL / 2)
+//     lanes per row, 16 bytes a lane, kAhead entries of the group's rows in flight;
+//  3. G[I, J] = (W[I, J] + W[J, I]^T)/2 and its transpose, by the thread that holds both
+//     entries; then the support terms, a thread per list entry, the scale, and 16-byte stores.
 // The rounding sequence per element is the solver's (W in the canonical order,
 // 0.5 (W_ij + W_ji), the support terms, the scale).
+//
+// What bounds it: memory (S[I, J], the S rows of the neighbours, both halves of G), as long as
+// enough of it is asked for at once.  With a warp per row that went from the row's bounds to its
+// entries to S, one row after the other, the rows with neighbours were a chain of three
+// latencies each, about nine of them per warp where half of the rows have neighbours.
+// Measured on GB300, p = 16384, 28 672 entries (half of the rows with neighbours): 770 -> 594 us.
+// A tile pair whose rows have more than kGradList entries takes the rows one by one, a warp
+// each (offdiag_row, support_terms_row).
+constexpr int kGradList = 512;
+constexpr int kAhead = 4;
+
 template <typename T, int TL>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3)
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3)
 k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __restrict__ rdv,
                   const T* __restrict__ S, int64_t lds, T* __restrict__ G, int64_t ldg, T lam2, T scale, int nt,
                   int vec /* bit 0: 16-byte G stores; bit 1: 16-byte S loads */) {
     __shared__ T a[TL][TL + 1];      // W[I, J], then G[I, J]
     __shared__ T b[TL][TL + 1];      // W[J, I], then G[J, I]
-    __shared__ T dvs[2][TL];         // w_ii of the rows of I and of J
-    __shared__ int imp[2][TL];       // rows of I and of J with off-diagonal entries
-    __shared__ int nimp[2];
+    __shared__ T dvs[2 * TL];        // w_ii of the rows of I, then of J
+    __shared__ int off[2 * TL + 1];  // first list entry of each row
+    __shared__ int lk[kGradList];    // list: column k, w_ik, the entry's row (0 .. 2 TL - 1)
+    __shared__ T lw[kGradList];
+    __shared__ unsigned char lr[kGradList];
+    __shared__ int wsum[2 * TL / 32];
     constexpr int E = TL * TL / 256;
+    static_assert(2 * TL <= 256, "a row per thread");
     int bi, bj;
     pair_of(blockIdx.x, nt, bi, bj);
     const int I0 = bi * TL, J0 = bj * TL;
     const bool dtile = bi == bj;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x < 2) nimp[threadIdx.x] = 0;
-    __syncthreads();
+    // 0. the list
+    int4 info = make_int4(0, 0, -1, 1);
+    int cnt = 0, incl = 0;
+    const int row0 = (int)threadIdx.x < TL ? I0 + (int)threadIdx.x : J0 + (int)threadIdx.x - TL;
     if (threadIdx.x < 2 * TL) {
-        const int side = threadIdx.x / TL, yl = threadIdx.x % TL;
-        const int i = (side ? J0 : I0) + yl;
         T dv = T(0);
-        bool impure = false;
-        if (i < p) {
-            dv = rdv[i];
-            impure = rinfo[i].w == 0;
+        if (row0 < p) {
+            dv = rdv[row0];
+            info = rinfo[row0];
+            cnt = info.y - info.x - (info.z >= 0 ? 1 : 0);
         }
-        dvs[side][yl] = dv;
-        if (impure) imp[side][atomicAdd(&nimp[side], 1)] = yl;
+        dvs[threadIdx.x] = dv;
+        incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) wsum[warp] = incl;
     }
     __syncthreads();
-    // 1. diagonal terms of both tiles from one read of S[I, J]
+    int total = 0;
+#pragma unroll
+    for (int w = 0; w < 2 * TL / 32; ++w) {
+        if (w < warp) incl += wsum[w];
+        total += wsum[w];
+    }
+    const bool listed = total <= kGradList;
+    if (threadIdx.x < 2 * TL) {
+        int at = incl - cnt;
+        off[threadIdx.x] = at;
+        if (threadIdx.x == 2 * TL - 1) off[2 * TL] = total;
+        if (listed)
+            for (int q = info.x; q < info.y; ++q) {
+                if (q == info.z) continue;
+                lk[at] = om.ci[q];
+                lw[at] = om.cv[q];
+                lr[at] = (unsigned char)threadIdx.x;
+                ++at;
+            }
+    }
+    __syncthreads();
     constexpr int VW = 16 / (int)sizeof(T), PR = TL / VW, EV = TL * PR / 256;   // 16-byte vectors
     using V16 = Vec16<T>;
     const bool full = I0 + TL <= p && J0 + TL <= p;
-    if ((vec & 2) && full) {
+    const bool vload = (vec & 2) && full;
+    // the group's cursor over the entries of its rows (grp, grp + 256 / PR, ..)
+    const int grp = threadIdx.x / PR, gl = (threadIdx.x % PR) * VW;
+    constexpr int NG = 256 / PR;
+    int r = grp - NG, t = 0, end = 0;
+    auto next = [&]() -> int {               // the next entry, -1 at the end
+        while (t == end) {
+            r += NG;
+            if (r >= 2 * TL) return -1;
+            t = off[r];
+            end = off[r + 1];
+        }
+        return t++;
+    };
+    auto fetch = [&](int e) -> typename V16::type {
+        const T* src = S + (int64_t)lk[e] * lds + (lr[e] < TL ? J0 : I0) + gl;
+        if (vload) return *reinterpret_cast<const typename V16::type*>(src);
+        T v[VW];
+        const int c = (lr[e] < TL ? J0 : I0) + gl;
+#pragma unroll
+        for (int x = 0; x < VW; ++x) v[x] = c + x < p ? src[x] : T(0);
+        return V16::make(v);
+    };
+    int ent[kAhead];
+    typename V16::type sv4[kAhead];
+    if (listed) {
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            ent[u] = r < 2 * TL ? next() : -1;
+            if (ent[u] >= 0) sv4[u] = fetch(ent[u]);
+        }
+    }
+    // 1. diagonal terms of both tiles from one read of S[I, J]
+    if (vload) {
         typename V16::type u[EV];
 #pragma unroll
         for (int e = 0; e < EV; ++e) {           // all the tile's loads in flight before any use
@@ -263,8 +339,8 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
             V16::unpack(u[e], sv);
 #pragma unroll
             for (int k = 0; k < VW; ++k) {
-                a[y][x + k] = mulT(dvs[0][y], sv[k]);
-                b[x + k][y] = mulT(dvs[1][x + k], sv[k]);
+                a[y][x + k] = mulT(dvs[y], sv[k]);
+                b[x + k][y] = mulT(dvs[TL + x + k], sv[k]);
             }
         }
     } else {
@@ -272,42 +348,64 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
         for (int e = 0; e < E; ++e) {
             const int idx = threadIdx.x + 256 * e, y = idx / TL, x = idx % TL;
             const T sv = (I0 + y < p && J0 + x < p) ? S[(int64_t)(I0 + y) * lds + J0 + x] : T(0);
-            a[y][x] = mulT(dvs[0][y], sv);
-            b[x][y] = mulT(dvs[1][x], sv);
+            a[y][x] = mulT(dvs[y], sv);
+            b[x][y] = mulT(dvs[TL + x], sv);
         }
     }
     __syncthreads();
     // 2. off-diagonal terms of the rows that have them
-    const int n0 = nimp[0], n1 = nimp[1];
-    for (int r = warp; r < n0 + n1; r += kW) {
-        const int side = r < n0 ? 0 : 1;
-        const int yl = side ? imp[1][r - n0] : imp[0][r];
-        const int i = (side ? J0 : I0) + yl;
-        offdiag_row<T, TL>(p, om, rinfo[i], S, lds, side ? I0 : J0, side ? &b[yl][0] : &a[yl][0]);
+    if (listed) {
+        while (ent[0] >= 0) {
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                if (ent[u] < 0) break;
+                const int row = lr[ent[u]];
+                T* w = row < TL ? &a[row][gl] : &b[row - TL][gl];
+                const T wk = lw[ent[u]];
+                T sv[VW];
+                V16::unpack(sv4[u], sv);
+#pragma unroll
+                for (int x = 0; x < VW; ++x) w[x] = fmaT(wk, sv[x], w[x]);
+            }
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                ent[u] = r < 2 * TL ? next() : -1;
+                if (ent[u] >= 0) sv4[u] = fetch(ent[u]);
+            }
+        }
+    } else {
+        for (int row = warp; row < 2 * TL; row += kW) {
+            if (off[row] == off[row + 1]) continue;
+            const int i = row < TL ? I0 + row : J0 + row - TL;
+            offdiag_row<T, TL>(p, om, rinfo[i], S, lds, row < TL ? J0 : I0, row < TL ? &a[row][0] : &b[row - TL][0]);
+        }
     }
     __syncthreads();
-    // 3. symmetrise: G[I, J] in place; G[J, I] is its transpose (a + b = b + a)
+    // 3. symmetrise: G[I, J] and its transpose (a + b = b + a)
 #pragma unroll 4
     for (int e = 0; e < E; ++e) {
         const int idx = threadIdx.x + 256 * e, y = idx / TL, x = idx % TL;
-        a[y][x] = T(0.5) * (a[y][x] + b[x][y]);
+        const T g = T(0.5) * (a[y][x] + b[x][y]);
+        a[y][x] = g;
+        b[x][y] = g;
     }
     __syncthreads();
-    if (!dtile) {
-#pragma unroll 4
-        for (int e = 0; e < E; ++e) {
-            const int idx = threadIdx.x + 256 * e, y = idx / TL, x = idx % TL;
-            b[y][x] = a[x][y];
-        }
-        __syncthreads();
-        for (int r = warp; r < n0 + n1; r += kW) {
-            const int side = r < n0 ? 0 : 1;
-            const int yl = side ? imp[1][r - n0] : imp[0][r];
-            support_terms_row<T, TL>(om, (side ? J0 : I0) + yl, side ? I0 : J0, lam2, side ? &b[yl][0] : &a[yl][0]);
-        }
-    } else {
+    if (dtile) {
         // the diagonal tile: every row has its diagonal entry here
         for (int y = warp; y < TL && I0 + y < p; y += kW) support_terms_row<T, TL>(om, I0 + y, I0, lam2, &a[y][0]);
+    } else if (listed) {
+        for (int e = threadIdx.x; e < total; e += 256) {
+            const int row = lr[e], c = lk[e] - (row < TL ? J0 : I0);
+            if (c < 0 || c >= TL) continue;
+            T* g = row < TL ? &a[row][c] : &b[row - TL][c];
+            *g = fmaT(lam2, lw[e], *g);
+        }
+    } else {
+        for (int row = warp; row < 2 * TL; row += kW) {
+            if (off[row] == off[row + 1]) continue;
+            support_terms_row<T, TL>(om, row < TL ? I0 + row : J0 + row - TL, row < TL ? J0 : I0, lam2,
+                                     row < TL ? &a[row][0] : &b[row - TL][0]);
+        }
     }
     __syncthreads();
     const bool scaled = scale != T(1);
