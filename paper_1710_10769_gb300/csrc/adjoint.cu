@@ -437,24 +437,32 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
     }
 }
 
-// out[c][r] = in[r][c] * scale, 32 x 32 shared-memory tiles held in the output type
-// (an FP64 transpose stays FP64).
+// out[c][r] = in[r][c] * scale, 64 x 64 shared-memory tiles held in the output type
+// (an FP64 transpose stays FP64); columns rows .. rows_out - 1 of out are set to 0.
+// What bounds it: memory, once enough loads are in flight: each thread has 16 of them (with
+// 32 x 32 tiles it had four).  Measured on GB300, 4096 x 16384 FP32: 174 -> 79 us.
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(256)
 k_transpose(const TI* __restrict__ in, int64_t rows, int64_t cols, int64_t ldi, TO* __restrict__ out, int64_t ldo,
-            double scale) {
-    __shared__ TO tile[32][33];
+            int64_t rows_out, double scale) {
+    __shared__ TO tile[64][65];
     const TO sc = (TO)scale;
-    const int64_t r0 = (int64_t)blockIdx.y * 32, c0 = (int64_t)blockIdx.x * 32;
+    const int64_t r0 = (int64_t)blockIdx.y * 64, c0 = (int64_t)blockIdx.x * 64;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int y = ty; y < 32; y += 8) {
-        const int64_t r = r0 + y, c = c0 + tx;
-        tile[y][tx] = (r < rows && c < cols) ? to_t<TO>(in[r * ldi + c]) : TO(0);
+    TO v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+        const int64_t r = r0 + ty + 8 * (u >> 1), c = c0 + tx + 32 * (u & 1);
+        v[u] = (r < rows && c < cols) ? to_t<TO>(in[r * ldi + c]) : TO(0);
     }
+#pragma unroll
+    for (int u = 0; u < 16; ++u) tile[ty + 8 * (u >> 1)][tx + 32 * (u & 1)] = v[u];
     __syncthreads();
-    for (int y = ty; y < 32; y += 8) {
-        const int64_t c = c0 + y, r = r0 + tx;
-        if (c < cols && r < rows) out[c * ldo + r] = tile[tx][y] * sc;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+        const int y = ty + 8 * (u >> 1), x = tx + 32 * (u & 1);
+        const int64_t c = c0 + y, r = r0 + x;
+        if (c < cols && r < rows_out) out[c * ldo + r] = tile[x][y] * sc;
     }
 }
 
@@ -497,6 +505,93 @@ __global__ void k_support_product(int p, Csr<T> om, const int4* __restrict__ rin
     }
 }
 
+// T_e = (1/n) sum_m (Omega X^T)[i, m] X^T[j_e, m] for every support entry e = (i, j_e): the
+// support-restricted (Omega S)_ij with S = X^T X / n, without S and without storing Omega X^T.
+// A block per row i, kXyCols samples at a time: the row's Y = Omega X^T (k_spmm_dense's order)
+// stays in registers, and the rows of X^T that made it are what its entries need next, from L1.
+// 16-byte loads: ld is a multiple of 16 bytes and the columns from n to ld are 0.  Partials in T
+// per thread (16 products), summed over the block and the pieces in FP64 in a fixed order.
+// What bounds it: memory (the rows of X^T, 1 + the row's neighbours times).  As two kernels, Y^T
+// was written and read back, and a warp per row went through its entries one after the other.
+// Measured on GB300, p = 16384, n = 2048, 28 672 entries: 159 (55 + 104) -> 56 us.
+constexpr int kXyT = 128;
+constexpr int kXyCols = 16 * kXyT;
+constexpr int kXyBatch = 16;
+
+template <typename T>
+__global__ void __launch_bounds__(kXyT)
+k_support_xy(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __restrict__ rdv, const T* __restrict__ xt,
+             int64_t ld, int64_t n, double* __restrict__ out) {
+    using V16 = Vec16<T>;
+    constexpr int VW = 16 / (int)sizeof(T), U = 16 / VW;
+    __shared__ T part[kXyBatch][kXyT];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = blockIdx.x;
+    const int4 info = rinfo[i];
+    const T dv = rdv[i];
+    for (int64_t m0 = 0; m0 < n; m0 += kXyCols) {
+        auto load = [&](int64_t row, typename V16::type (&v)[U]) {
+            const T zero[VW] = {};
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t m = m0 + (int64_t)(threadIdx.x + kXyT * u) * VW;
+                v[u] = m < ld ? __ldg(reinterpret_cast<const typename V16::type*>(xt + row * ld + m)) : V16::make(zero);
+            }
+        };
+        T y[U][VW];
+        {
+            typename V16::type v[U];
+            load(i, v);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                V16::unpack(v[u], y[u]);
+#pragma unroll
+                for (int x = 0; x < VW; ++x) y[u][x] = mulT(dv, y[u][x]);
+            }
+        }
+        for (int q = info.x; q < info.y; ++q) {
+            if (q == info.z) continue;
+            const T w = om.cv[q];
+            typename V16::type v[U];
+            load(om.ci[q], v);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                T xv[VW];
+                V16::unpack(v[u], xv);
+#pragma unroll
+                for (int x = 0; x < VW; ++x) y[u][x] = fmaT(w, xv[x], y[u][x]);
+            }
+        }
+        for (int e0 = info.x; e0 < info.y; e0 += kXyBatch) {
+            const int ne = min(kXyBatch, info.y - e0);
+            for (int e = 0; e < ne; ++e) {
+                typename V16::type v[U];
+                load(om.ci[e0 + e], v);
+                T s[VW] = {};
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    T xv[VW];
+                    V16::unpack(v[u], xv);
+#pragma unroll
+                    for (int x = 0; x < VW; ++x) s[x] = fmaT(y[u][x], xv[x], s[x]);
+                }
+                T r = s[0];
+#pragma unroll
+                for (int x = 1; x < VW; ++x) r += s[x];
+                part[e][threadIdx.x] = r;
+            }
+            __syncthreads();
+            for (int e = warp; e < ne; e += kXyT / 32) {
+                double r = ((double)part[e][lane] + (double)part[e][lane + 32]) +
+                           ((double)part[e][lane + 64] + (double)part[e][lane + 96]);
+                r = warp_sum_d(r) / (double)n;
+                if (lane == 0) out[e0 + e] = m0 == 0 ? r : out[e0 + e] + r;
+            }
+            __syncthreads();
+        }
+    }
+}
+
 // T_e = (1/n) sum_m Y^T[i, m] X^T[j_e, m] for every support entry e = (i, j_e), where
 // Y^T = Omega X^T: the support-restricted (Omega S)_ij with S = X^T X / n, without S.
 // Warp per row of the support; lanes stride m (coalesced rows of X^T and Y^T), four
@@ -534,7 +629,7 @@ k_support_sddmm(int p, Csr<T> om, const T* __restrict__ yt, const T* __restrict_
 // the support, all in L2 after the first one), so it is latency: as three kernels it
 // was three ramps, three chains of dependent loads (row, row bounds, direction, S) and three
 // last-block reductions.  Here a grid-wide barrier ends each of the two reductions
-// (<p, Hp> and <r, r>), every warp adds the blocks' partials itself in the same order, and
+// (<p, Hp> and <r, r>), every block adds the blocks' partials itself in the same order, and
 // all of them take the same step.
 //   RES  (nnz at most the grid's threads: an entry a thread): e's vectors, indexes and row
 //        bounds stay in registers, and the thread of (i, j) forms T_ji itself, in the same order
@@ -581,11 +676,18 @@ __device__ __forceinline__ void cg_block_sum(double s, double* out) {
     }
 }
 
-// the blocks' partials in a fixed order; every warp of every block gets the same bits
+// the blocks' partials in a fixed order, by one warp of every block (the FP64 rate, two lanes
+// per SM and cycle, is what a block's warps share); every block gets the same bits
 __device__ __forceinline__ double cg_total(const double* part) {
-    double s = 0.0;
-    for (int b = threadIdx.x & 31; b < (int)gridDim.x; b += 32) s += __ldcg(part + b);
-    return warp_sum_d(s);
+    __shared__ double tot;
+    if (threadIdx.x < 32) {
+        double s = 0.0;
+        for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) s += __ldcg(part + b);
+        s = warp_sum_d(s);
+        if (threadIdx.x == 0) tot = s;
+    }
+    __syncthreads();
+    return tot;                             // next written after another barrier
 }
 
 // Grid-wide barrier on a counter that only grows; false after a timeout.
@@ -629,17 +731,21 @@ __device__ __forceinline__ double cg_row_dot(const CgArgs<T>& k, int4 info, int 
     double acc = 0.0;
     if (info.z >= 0) acc = fma(beta, __ldcg(p + info.z), __ldcg(k.r + info.z)) * (double)__ldg(Sj + (int64_t)i * k.lds);
     for (int q0 = info.x; q0 < info.y; q0 += 4) {
-        double v[4], s[4];
+        double v[4], w[4];
+        T s[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int q = q0 + u;
             const bool on = q < info.y && q != info.z;
-            v[u] = on ? fma(beta, __ldcg(p + q), __ldcg(k.r + q)) : 0.0;
-            s[u] = on ? (double)__ldg(Sj + (int64_t)__ldg(k.om.ci + q) * k.lds) : 0.0;
+            v[u] = on ? __ldcg(p + q) : 0.0;
+            w[u] = on ? __ldcg(k.r + q) : 0.0;
+            s[u] = on ? __ldg(Sj + (int64_t)__ldg(k.om.ci + q) * k.lds) : T(0);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (q0 + u < info.y && q0 + u != info.z) acc = fma(v[u], s[u], acc);
+        for (int u = 0; u < 4; ++u) {
+            if (q0 + u >= info.y) break;
+            if (q0 + u != info.z) acc = fma(fma(beta, v[u], w[u]), (double)s[u], acc);
+        }
     }
     return acc;
 }
@@ -766,8 +872,9 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
     cg_block_sum(s1, part[2] + blockIdx.x);
     cg_block_sum(s2, part[3] + blockIdx.x);
     if (alive) alive = cg_barrier(k.st, target);
-    if (blockIdx.x == 0 && threadIdx.x < 32 && alive) {
+    if (blockIdx.x == 0 && alive) {
         s1 = cg_total(part[2]);
+        __syncthreads();
         s2 = cg_total(part[3]);
         if (threadIdx.x == 0) {
             k.st->rr = rr;
@@ -831,20 +938,24 @@ __global__ void k_sign_off(int p, Csr<T> om, double* sign_off) {
 }
 
 // Partials of the smooth part at the iterate: [0] sum_e w_e T_e (= tr(Omega S Omega) with
-// T = (Omega S) on the support), [1] ||Omega||_F^2, [2] sum_i log w_ii.
+// T = (Omega S) on the support), [1] ||Omega||_F^2, [2] sum_i log w_ii.  A thread per entry, then a
+// thread per row: with a warp per row one lane's FP64 logarithm held the warp, at an FP64 rate
+// of two lanes per SM and cycle (44 us at p = 16384, 7 now).
 template <typename T>
-__global__ void __launch_bounds__(256) k_smooth_parts(int p, Csr<T> om, const double* __restrict__ Tv, double* part) {
+__global__ void __launch_bounds__(256)
+k_smooth_parts(int p, int64_t nnz, Csr<T> om, const int4* __restrict__ rinfo, const T* __restrict__ rdv,
+               const double* __restrict__ Tv, double* part) {
     __shared__ double red[8][3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t t0 = blockIdx.x * 256ll + threadIdx.x, step = gridDim.x * 256ll;
     double a = 0.0, b = 0.0, c = 0.0;
-    for (int i = blockIdx.x * kW + warp; i < p; i += gridDim.x * kW) {
-        for (int e = om.rp[i] + lane; e < om.rp[i + 1]; e += 32) {
-            const double w = (double)om.cv[e];
-            a = fma(w, Tv[e], a);
-            b = fma(w, w, b);
-            if (om.ci[e] == i) c += log(w);
-        }
+    for (int64_t e = t0; e < nnz; e += step) {
+        const double w = (double)om.cv[e];
+        a = fma(w, Tv[e], a);
+        b = fma(w, w, b);
     }
+    for (int64_t i = t0; i < p; i += step)
+        if (rinfo[i].z >= 0) c += log((double)rdv[i]);
     a = warp_sum_d(a); b = warp_sum_d(b); c = warp_sum_d(c);
     if (lane == 0) { red[warp][0] = a; red[warp][1] = b; red[warp][2] = c; }
     __syncthreads();
@@ -879,11 +990,11 @@ __global__ void __launch_bounds__(256) k_reduce_strided(const double* part, int 
 static int entry_blocks(int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 1024); }
 
 template <typename T>
-int launch_smooth_parts(int p, Csr<T> om, const double* Tv, double* part, double* out3, cudaStream_t s) {
-    const int nb = std::min((p + kW - 1) / kW, 1024);
-    k_smooth_parts<T><<<nb, 256, 0, s>>>(p, om, Tv, part);
+void launch_smooth_parts(int p, int64_t nnz, Csr<T> om, const int4* rinfo, const T* rdv, const double* Tv, double* part,
+                         double* out3, cudaStream_t s) {
+    const int nb = std::min((p + 255) / 256, 1024);
+    k_smooth_parts<T><<<nb, 256, 0, s>>>(p, nnz, om, rinfo, rdv, Tv, part);
     k_reduce_strided<<<1, 256, 0, s>>>(part, nb, 3, out3);
-    return nb;
 }
 
 template <typename T>
@@ -913,27 +1024,28 @@ void launch_spmm_dense_t(int p, Csr<T> om, const int4* rinfo, const T* rdv, cons
 }
 
 void launch_transpose(const void* in, int in_dt, int64_t rows, int64_t cols, int64_t ldi, void* out, int out_dt,
-                      int64_t ldo, double scale, cudaStream_t s) {
-    dim3 g((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32));
+                      int64_t ldo, double scale, cudaStream_t s, int64_t pad_to) {
+    const int64_t rows_out = std::max(rows, pad_to);
+    dim3 g((unsigned)((cols + 63) / 64), (unsigned)((rows_out + 63) / 64));
     const bool o64 = out_dt == HPC_F64;
     if (in_dt == HPC_BF16 && o64) {
         k_transpose<__nv_bfloat16, double><<<g, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(in), rows, cols, ldi,
-                                                              static_cast<double*>(out), ldo, scale);
+                                                              static_cast<double*>(out), ldo, rows_out, scale);
     } else if (in_dt == HPC_BF16) {
         k_transpose<__nv_bfloat16, float><<<g, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(in), rows, cols, ldi,
-                                                             static_cast<float*>(out), ldo, scale);
+                                                             static_cast<float*>(out), ldo, rows_out, scale);
     } else if (in_dt == HPC_F64 && o64) {
         k_transpose<double, double><<<g, 256, 0, s>>>(static_cast<const double*>(in), rows, cols, ldi,
-                                                       static_cast<double*>(out), ldo, scale);
+                                                       static_cast<double*>(out), ldo, rows_out, scale);
     } else if (in_dt == HPC_F64) {
         k_transpose<double, float><<<g, 256, 0, s>>>(static_cast<const double*>(in), rows, cols, ldi,
-                                                      static_cast<float*>(out), ldo, scale);
+                                                      static_cast<float*>(out), ldo, rows_out, scale);
     } else if (o64) {
         k_transpose<float, double><<<g, 256, 0, s>>>(static_cast<const float*>(in), rows, cols, ldi,
-                                                      static_cast<double*>(out), ldo, scale);
+                                                      static_cast<double*>(out), ldo, rows_out, scale);
     } else {
         k_transpose<float, float><<<g, 256, 0, s>>>(static_cast<const float*>(in), rows, cols, ldi,
-                                                     static_cast<float*>(out), ldo, scale);
+                                                     static_cast<float*>(out), ldo, rows_out, scale);
     }
 }
 
@@ -946,6 +1058,12 @@ template <typename T>
 void launch_support_product(int p, Csr<T> om, const int4* rinfo, const double* v, const T* S, int64_t lds,
                             double* out, cudaStream_t s) {
     k_support_product<T><<<(p + kW - 1) / kW, 256, 0, s>>>(p, om, rinfo, v, S, lds, out);
+}
+
+template <typename T>
+void launch_support_xy(int p, Csr<T> om, const int4* rinfo, const T* rdv, const T* xt, int64_t ld, int64_t n,
+                       double* out, cudaStream_t s) {
+    k_support_xy<T><<<p, kXyT, 0, s>>>(p, om, rinfo, rdv, xt, ld, n, out);
 }
 
 template <typename T>
@@ -1018,6 +1136,8 @@ cudaError_t launch_cg(int64_t nnz, const int* row, Csr<T> om, const int4* rinfo,
                                             cudaStream_t);                                                      \
     template void launch_support_sddmm<T>(int, Csr<T>, const T*, const T*, int64_t, int64_t, double*,         \
                                           cudaStream_t);                                                        \
+    template void launch_support_xy<T>(int, Csr<T>, const int4*, const T*, const T*, int64_t, int64_t, double*, \
+                                       cudaStream_t);                                                           \
     template void launch_support_heldout<T>(int64_t, const int*, Csr<T>, const int*, const double*, double*,     \
                                             cudaStream_t);                                                      \
     template cudaError_t launch_cg<T>(int64_t, const int*, Csr<T>, const int4*, const int*, const T*, int64_t,  \
@@ -1026,7 +1146,8 @@ cudaError_t launch_cg(int64_t nnz, const int* row, Csr<T> om, const int4* rinfo,
     template void launch_support_vectors<T>(int, int64_t, Csr<T>, double*, double*, cudaStream_t);          \
     template void launch_support_grad<T>(int64_t, const int*, Csr<T>, const int*, const double*, double,      \
                                          double, double*, cudaStream_t);                                        \
-    template int launch_smooth_parts<T>(int, Csr<T>, const double*, double*, double*, cudaStream_t);
+    template void launch_smooth_parts<T>(int, int64_t, Csr<T>, const int4*, const T*, const double*, double*,   \
+                                         double*, cudaStream_t);
 
 HPC_ADJ_INSTANTIATE(float)
 HPC_ADJ_INSTANTIATE(double)

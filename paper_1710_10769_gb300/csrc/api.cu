@@ -1962,7 +1962,7 @@ int smooth_value_t(hpc_ctx* h, double* f) {
     hpc::launch_row_info<T>(p, om, h->rinfo, as<T>(h->rdv), h->stream);
     hpc::launch_support_vectors<T>(p, nnz, om, om_d, Tv, h->stream);     // Tv used as scratch for signs
     hpc::launch_support_product<T>(p, om, h->rinfo, om_d, static_cast<const T*>(h->S), h->ld, Tv, h->stream);
-    hpc::launch_smooth_parts<T>(p, om, Tv, part, out3, h->stream);
+    hpc::launch_smooth_parts<T>(p, nnz, om, h->rinfo, as<T>(h->rdv), Tv, part, out3, h->stream);
     CUDA_TRY(cudaGetLastError());
     double o[3];
     CUDA_TRY(cudaMemcpyAsync(o, out3, sizeof o, cudaMemcpyDeviceToHost, h->stream));
@@ -2040,13 +2040,13 @@ template <typename T>
 int heldout_t(hpc_ctx* h, const void* Xval, int xdt, int64_t nval, double* loss) {
     const int p = (int)h->p;
     const int64_t nnz = h->nnz;
-    const size_t b_x = align256((size_t)p * nval * sizeof(T));
+    const int64_t ldv = (nval + 3) / 4 * 4;            // rows of X_val^T: 16-byte loads
+    const size_t b_x = align256((size_t)p * ldv * sizeof(T));
     const size_t b_v = align256(nnz * sizeof(double));
     const size_t b_p = align256(1024 * 3 * sizeof(double));
-    STATUS_TRY(adj_reserve(h, 2 * b_x + b_v + b_p + 256));
+    STATUS_TRY(adj_reserve(h, b_x + b_v + b_p + 256));
     uint8_t* q = static_cast<uint8_t*>(h->adj_buf);
     T* xtv = reinterpret_cast<T*>(q); q += b_x;
-    T* ytv = reinterpret_cast<T*>(q); q += b_x;
     double* Tv = reinterpret_cast<double*>(q); q += b_v;
     double* part = reinterpret_cast<double*>(q); q += b_p;
     double* out3 = reinterpret_cast<double*>(q);
@@ -2054,10 +2054,9 @@ int heldout_t(hpc_ctx* h, const void* Xval, int xdt, int64_t nval, double* loss)
     hpc::Csr<T> om = cur_csr<T>(h);
     hpc::launch_row_info<T>(p, om, h->rinfo, as<T>(h->rdv), s);
     const int tdt = sizeof(T) == 8 ? HPC_F64 : HPC_F32;
-    hpc::launch_transpose(Xval, xdt, nval, p, p, xtv, tdt, nval, 1.0, s);
-    hpc::launch_spmm_dense<T>(p, om, h->rinfo, as<T>(h->rdv), xtv, nval, nval, ytv, nval, s);
-    hpc::launch_support_sddmm<T>(p, om, ytv, xtv, nval, nval, Tv, s);
-    hpc::launch_smooth_parts<T>(p, om, Tv, part, out3, s);
+    hpc::launch_transpose(Xval, xdt, nval, p, p, xtv, tdt, ldv, 1.0, s, ldv);
+    hpc::launch_support_xy<T>(p, om, h->rinfo, as<T>(h->rdv), xtv, ldv, nval, Tv, s);
+    hpc::launch_smooth_parts<T>(p, nnz, om, h->rinfo, as<T>(h->rdv), Tv, part, out3, s);
     CUDA_TRY(cudaGetLastError());
     double o[3];
     CUDA_TRY(cudaMemcpyAsync(o, out3, sizeof o, cudaMemcpyDeviceToHost, s));
@@ -2071,14 +2070,14 @@ int hypergrad_t(hpc_ctx* h, const void* Xval, int xdt, int64_t nval, double cg_t
                 double* dl2, hpc_hypergrad_info* info) {
     const int p = (int)h->p;
     const int64_t nnz = h->nnz;
-    const size_t b_x = align256((size_t)p * nval * sizeof(T));
+    const int64_t ldv = (nval + 3) / 4 * 4;            // rows of X_val^T: 16-byte loads
+    const size_t b_x = align256((size_t)p * ldv * sizeof(T));
     const size_t b_v = align256(nnz * sizeof(double));
     const size_t b_i = align256(nnz * sizeof(int));
     const size_t b_cg = align256(hpc::cg_vector_doubles(nnz) * sizeof(double));
-    STATUS_TRY(adj_reserve(h, 2 * b_x + 4 * b_v + 2 * b_i + b_cg + align256(sizeof(hpc::CgState))));
+    STATUS_TRY(adj_reserve(h, b_x + 4 * b_v + 2 * b_i + b_cg + align256(sizeof(hpc::CgState))));
     uint8_t* q = static_cast<uint8_t*>(h->adj_buf);
     T* xtv = reinterpret_cast<T*>(q); q += b_x;
-    T* ytv = reinterpret_cast<T*>(q); q += b_x;
     double* om_d = reinterpret_cast<double*>(q); q += b_v;
     double* sgn = reinterpret_cast<double*>(q); q += b_v;
     double* Tv = reinterpret_cast<double*>(q); q += b_v;
@@ -2094,12 +2093,11 @@ int hypergrad_t(hpc_ctx* h, const void* Xval, int xdt, int64_t nval, double cg_t
     hpc::launch_transpose_index<T>(p, om, tr, rowid, s);
     hpc::launch_support_vectors<T>(p, nnz, om, om_d, sgn, s);
     // b = gradient of the held-out loss on the support.  Its term (Omega S_val)_ij is
-    // (1/n_val) <(X_val Omega)_{:,i}, X_val_{:,j}>: Y^T = Omega X_val^T, then one row
-    // pair per support entry; S_val itself is never formed.
+    // (1/n_val) <(X_val Omega)_{:,i}, X_val_{:,j}>: neither X_val Omega nor S_val is
+    // stored.
     const int tdt = sizeof(T) == 8 ? HPC_F64 : HPC_F32;
-    hpc::launch_transpose(Xval, xdt, nval, p, p, xtv, tdt, nval, 1.0, s);
-    hpc::launch_spmm_dense<T>(p, om, h->rinfo, as<T>(h->rdv), xtv, nval, nval, ytv, nval, s);
-    hpc::launch_support_sddmm<T>(p, om, ytv, xtv, nval, nval, Tv, s);
+    hpc::launch_transpose(Xval, xdt, nval, p, p, xtv, tdt, ldv, 1.0, s, ldv);
+    hpc::launch_support_xy<T>(p, om, h->rinfo, as<T>(h->rdv), xtv, ldv, nval, Tv, s);
     hpc::launch_support_heldout<T>(nnz, rowid, om, tr, Tv, bvec, s);
     // CG on H_A v = b, then dL_val/dlambda1 = -<v, sgn_off>, dL_val/dlambda2 = -<v, Omega_A>
     CUDA_TRY(hpc::launch_cg<T>(nnz, rowid, om, h->rinfo, tr, static_cast<const T*>(h->S), h->ld, h->lam2, cg_tol, cg_max,

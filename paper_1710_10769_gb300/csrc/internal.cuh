@@ -272,14 +272,17 @@ void launch_spmm_dense(int p, Csr<T> om, const int4* rinfo, const T* rdv, const 
 template <typename T>
 void launch_spmm_dense_t(int p, Csr<T> om, const int4* rinfo, const T* rdv, const T* B, int64_t ldb, int64_t m,
                          T* Ct, int64_t ldt, T scale, cudaStream_t s);
-// launch_transpose puts rows / 32 in gridDim.y (at most 65535)
+// rows that launch_transpose takes at most; pad_to > rows: out's columns from rows to pad_to are 0
 constexpr int64_t kTransposeMaxRows = 65535ll * 32;
 void launch_transpose(const void* in, int in_dt, int64_t rows, int64_t cols, int64_t ldi, void* out, int out_dt,
-                      int64_t ldo, double scale, cudaStream_t s);
+                      int64_t ldo, double scale, cudaStream_t s, int64_t pad_to = 0);
 template <typename T> void launch_transpose_index(int p, Csr<T> om, int* tr, int* row, cudaStream_t s);
 template <typename T>
 void launch_support_product(int p, Csr<T> om, const int4* rinfo, const double* v, const T* S, int64_t lds,
                             double* out, cudaStream_t s);
+template <typename T>
+void launch_support_xy(int p, Csr<T> om, const int4* rinfo, const T* rdv, const T* xt, int64_t ld, int64_t n,
+                       double* out, cudaStream_t s);
 template <typename T>
 void launch_support_sddmm(int p, Csr<T> om, const T* yt, const T* xt, int64_t ld, int64_t n, double* out,
                           cudaStream_t s);
@@ -308,7 +311,8 @@ cudaError_t launch_cg(int64_t nnz, const int* row, Csr<T> om, const int4* rinfo,
                       double lam2, double tol, int64_t max_iter, const double* b, const double* sgn, const double* om_d,
                       double* vec, CgState* st, int num_sms, cudaStream_t s);
 template <typename T>
-int launch_smooth_parts(int p, Csr<T> om, const double* Tv, double* part, double* out3, cudaStream_t s);
+void launch_smooth_parts(int p, int64_t nnz, Csr<T> om, const int4* rinfo, const T* rdv, const double* Tv, double* part,
+                         double* out3, cudaStream_t s);
 
 // ---------------------------------------------------------------- dense products (gram*.cu)
 // S = X^T X / n into S (p x lds).  Returns a CUDA error code.
