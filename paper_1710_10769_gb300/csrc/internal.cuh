@@ -199,6 +199,12 @@ template <typename T> void launch_set_identity(Csr<T> c, int p, cudaStream_t s);
 template <typename T> void launch_csr_export(const int* rp, const int* ci, const T* cv, int p, int nnz,
                                              int64_t* rp64, int32_t* ci_out, void* val, int vdt,
                                              cudaStream_t s);
+enum : unsigned { kCsrBadArg = 1, kCsrBadDiag = 2, kCsrNotFinite = 3 };
+void launch_csr_check(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int64_t p, int64_t nnz,
+                      unsigned long long* key, cudaStream_t s);
+template <typename T>
+void launch_csr_import(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int64_t p, int64_t nnz, Csr<T> out,
+                       cudaStream_t s);
 void launch_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int64_t* rows,
                      const int64_t* cols, double* out, cudaStream_t s);
 

@@ -2263,6 +2263,56 @@ __global__ void k_csr_export(const int* rp, const int* ci, const T* cv, int p, i
     }
 }
 
+// The checks of hpc_set_omega on a device CSR: the smallest key of a fault, row in the high half,
+// then the place in the row (0: its bounds; 1 + t: entry t; the largest: no diagonal), then the
+// fault, so that the fault reported is the first one in row order.  Rows whose bounds leave
+// 0 .. nnz are not read.  Thread per row.
+template <typename V>
+__global__ void __launch_bounds__(256) k_csr_check(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                                                   const V* __restrict__ v, int64_t p, int64_t nnz,
+                                                   unsigned long long* key) {
+    const int64_t i = blockIdx.x * 256ll + threadIdx.x;
+    if (i >= p) return;
+    unsigned place = 0, fault = 0;
+    const int64_t a = rp[i], b = rp[i + 1];
+    if (i == 0 && (a != 0 || rp[p] != nnz)) {
+        fault = kCsrBadArg;
+    } else if (b < a || a < 0 || b > nnz) {
+        fault = kCsrBadArg;
+    } else {
+        bool diag = false;
+        int64_t last = -1;
+        for (int64_t t = a; t < b && !fault; ++t) {
+            const int64_t c = ci[t];
+            const V x = v[t];
+            place = 1u + (unsigned)min(t - a, (int64_t)0x1ffffffd);
+            if (c < 0 || c >= p || (t > a && c <= last)) fault = kCsrBadArg;
+            else if (c == i && !(x > V(0))) fault = kCsrBadDiag;
+            else if (!isfinite(x)) fault = kCsrNotFinite;
+            diag = diag || c == i;
+            last = c;
+        }
+        if (!fault && !diag) {
+            place = 0x1fffffffu;
+            fault = kCsrBadDiag;
+        }
+    }
+    if (fault) atomicMin(key, (unsigned long long)i << 32 | (unsigned long long)(place << 2 | fault));
+}
+
+template <typename T, typename V>
+__global__ void __launch_bounds__(256) k_csr_import(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                                                    const V* __restrict__ v, int64_t p, int64_t nnz, int* __restrict__ rpo,
+                                                    int* __restrict__ cio, T* __restrict__ vo) {
+    for (int64_t t = blockIdx.x * 256ll + threadIdx.x; t < nnz || t <= p; t += gridDim.x * 256ll) {
+        if (t <= p) rpo[t] = (int)rp[t];
+        if (t < nnz) {
+            cio[t] = ci[t];
+            vo[t] = (T)v[t];
+        }
+    }
+}
+
 __global__ void k_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int64_t* rows,
                            const int64_t* cols, double* out) {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
@@ -2862,6 +2912,23 @@ void launch_csr_export(const int* rp, const int* ci, const T* cv, int p, int nnz
         k_csr_export<T, float><<<256, 256, 0, s>>>(rp, ci, cv, p, nnz, rp64, co, static_cast<float*>(val));
 }
 
+void launch_csr_check(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int64_t p, int64_t nnz,
+                      unsigned long long* key, cudaStream_t s) {
+    const unsigned nb = (unsigned)((p + 255) / 256);
+    if (vdt == HPC_F64) k_csr_check<double><<<nb, 256, 0, s>>>(rp, ci, static_cast<const double*>(v), p, nnz, key);
+    else k_csr_check<float><<<nb, 256, 0, s>>>(rp, ci, static_cast<const float*>(v), p, nnz, key);
+}
+
+template <typename T>
+void launch_csr_import(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int64_t p, int64_t nnz, Csr<T> out,
+                       cudaStream_t s) {
+    const unsigned nb = (unsigned)std::min<int64_t>((std::max(nnz, p + 1) + 255) / 256, 2048);
+    if (vdt == HPC_F64)
+        k_csr_import<T, double><<<nb, 256, 0, s>>>(rp, ci, static_cast<const double*>(v), p, nnz, out.rp, out.ci, out.cv);
+    else
+        k_csr_import<T, float><<<nb, 256, 0, s>>>(rp, ci, static_cast<const float*>(v), p, nnz, out.rp, out.ci, out.cv);
+}
+
 void launch_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int64_t* rows,
                      const int64_t* cols, double* out, cudaStream_t s) {
     k_gather_s<<<128, 256, 0, s>>>(S, is_f64, ld, m, rows, cols, out);
@@ -2881,6 +2948,8 @@ void launch_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int
     template void launch_row_info<T>(int, Csr<T>, int4*, T*, cudaStream_t);                        \
     template void launch_rowblock_max<T>(const T*, int64_t, int, int, unsigned short*, cudaStream_t); \
     template int screen_plan<T>(int, int, std::vector<long long>&);                                 \
+    template void launch_csr_import<T>(const int64_t*, const int32_t*, const void*, int, int64_t, int64_t, Csr<T>, \
+                                       cudaStream_t);                                              \
     template void launch_csr_export<T>(const int*, const int*, const T*, int, int, int64_t*, int32_t*, \
                                        void*, int, cudaStream_t);
 
