@@ -221,14 +221,14 @@ __device__ __forceinline__ void pair_of(long long t, int nt, int& bi, int& bj) {
 // enough of it is asked for at once.  With a warp per row that went from the row's bounds to its
 // entries to S, one row after the other, the rows with neighbours were a chain of three
 // latencies each, about nine of them per warp where half of the rows have neighbours.
-// Measured on GB300, p = 16384, 28 672 entries (half of the rows with neighbours): 770 -> 594 us.
+// Measured on GB300, p = 16384, 28 672 entries (half of the rows with neighbours): 770 -> 572 us.
 // A tile pair whose rows have more than kGradList entries takes the rows one by one, a warp
 // each (offdiag_row, support_terms_row).
 constexpr int kGradList = 512;
 constexpr int kAhead = 4;
 
 template <typename T, int TL>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3)
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 3)
 k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __restrict__ rdv,
                   const T* __restrict__ S, int64_t lds, T* __restrict__ G, int64_t ldg, T lam2, T scale, int nt,
                   int vec /* bit 0: 16-byte G stores; bit 1: 16-byte S loads */) {
@@ -247,6 +247,18 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
     const int I0 = bi * TL, J0 = bj * TL;
     const bool dtile = bi == bj;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int VW = 16 / (int)sizeof(T), PR = TL / VW, EV = TL * PR / 256;   // 16-byte vectors
+    using V16 = Vec16<T>;
+    const bool full = I0 + TL <= p && J0 + TL <= p;
+    const bool vload = (vec & 2) && full;
+    typename V16::type tile[EV];             // S[I, J], asked for before anything else
+    if (vload) {
+#pragma unroll
+        for (int e = 0; e < EV; ++e) {
+            const int idx = threadIdx.x + 256 * e, y = idx / PR, x = (idx % PR) * VW;
+            tile[e] = *reinterpret_cast<const typename V16::type*>(S + (int64_t)(I0 + y) * lds + J0 + x);
+        }
+    }
     // 0. the list
     int4 info = make_int4(0, 0, -1, 1);
     int cnt = 0, incl = 0;
@@ -289,10 +301,6 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
             }
     }
     __syncthreads();
-    constexpr int VW = 16 / (int)sizeof(T), PR = TL / VW, EV = TL * PR / 256;   // 16-byte vectors
-    using V16 = Vec16<T>;
-    const bool full = I0 + TL <= p && J0 + TL <= p;
-    const bool vload = (vec & 2) && full;
     // the group's cursor over the entries of its rows (grp, grp + 256 / PR, ..)
     const int grp = threadIdx.x / PR, gl = (threadIdx.x % PR) * VW;
     constexpr int NG = 256 / PR;
@@ -326,17 +334,11 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
     }
     // 1. diagonal terms of both tiles from one read of S[I, J]
     if (vload) {
-        typename V16::type u[EV];
-#pragma unroll
-        for (int e = 0; e < EV; ++e) {           // all the tile's loads in flight before any use
-            const int idx = threadIdx.x + 256 * e, y = idx / PR, x = (idx % PR) * VW;
-            u[e] = *reinterpret_cast<const typename V16::type*>(S + (int64_t)(I0 + y) * lds + J0 + x);
-        }
 #pragma unroll
         for (int e = 0; e < EV; ++e) {
             const int idx = threadIdx.x + 256 * e, y = idx / PR, x = (idx % PR) * VW;
             T sv[VW];
-            V16::unpack(u[e], sv);
+            V16::unpack(tile[e], sv);
 #pragma unroll
             for (int k = 0; k < VW; ++k) {
                 a[y][x + k] = mulT(dvs[y], sv[k]);
@@ -637,7 +639,8 @@ k_support_sddmm(int p, Csr<T> om, const T* __restrict__ yt, const T* __restrict_
 //        twice the gathers, which no thread waits for longer than for its own.
 //   else a grid-stride loop with T in memory and a third barrier: where the gathers are the
 //        time, they are not made twice.
-// Measured on GB300, p = 16384 (28 672 entries, 88 iterations): 1.30 ms.
+// Measured on GB300, p = 16384, 28 672 entries: 88 iterations in 1.00 ms, 11.4 us each (three
+// kernels in a graph: about 15).
 //
 // Every wait is bounded (kCgWaitNs): after that CgState::timeout is raised and every block
 // leaves.  The cooperative launch keeps all blocks resident.
@@ -668,26 +671,34 @@ __device__ __forceinline__ void cg_block_sum(double s, double* out) {
     __syncthreads();                        // the previous sum's readers are done with red
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double r = 0.0;
+    if (threadIdx.x < 32) {
+        double r = threadIdx.x < kCgT / 32 ? red[threadIdx.x] : 0.0;
 #pragma unroll
-        for (int w = 0; w < kCgT / 32; ++w) r += red[w];
-        *out = r;
+        for (int o = kCgT / 64; o > 0; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
+        if (threadIdx.x == 0) *out = r;
     }
 }
 
-// the blocks' partials in a fixed order, by one warp of every block (the FP64 rate, two lanes
-// per SM and cycle, is what a block's warps share); every block gets the same bits
-__device__ __forceinline__ double cg_total(const double* part) {
-    __shared__ double tot;
+// The blocks' partials in a fixed order (total), and ratio = num / total or total / num, by one
+// warp of every block: the FP64 rate is two lanes per SM and cycle, and a division by every warp
+// of the block took longer than the barrier.  Every block gets the same bits.
+struct CgSum {
+    double total, ratio;
+};
+template <bool INV>
+__device__ __forceinline__ CgSum cg_total(const double* part, double num) {
+    __shared__ CgSum out;
     if (threadIdx.x < 32) {
         double s = 0.0;
         for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) s += __ldcg(part + b);
         s = warp_sum_d(s);
-        if (threadIdx.x == 0) tot = s;
+        if (threadIdx.x == 0) {
+            out.total = s;
+            out.ratio = INV ? s / num : num / s;
+        }
     }
     __syncthreads();
-    return tot;                             // next written after another barrier
+    return out;                             // next written after another barrier
 }
 
 // Grid-wide barrier on a counter that only grows; false after a timeout.
@@ -750,6 +761,40 @@ __device__ __forceinline__ double cg_row_dot(const CgArgs<T>& k, int4 info, int 
     return acc;
 }
 
+// The S entries of one row's sum for a fixed column, kept in registers for rows of at most kKeep
+// entries: an iteration then loads only r and p, all at once.
+constexpr int kKeep = 8;
+template <typename T>
+struct CgRow {
+    T s[kKeep];
+    __device__ __forceinline__ void init(const CgArgs<T>& k, int4 info, int j) {
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u)
+            s[u] = info.x + u < info.y ? __ldg(k.S + (int64_t)__ldg(k.om.ci + info.x + u) * k.lds + j) : T(0);
+    }
+    __device__ __forceinline__ double dot(const CgArgs<T>& k, int4 info, int i, int j, const double* p, double beta) const {
+        if (info.y - info.x > kKeep) return cg_row_dot(k, info, i, j, p, beta);
+        double v[kKeep], w[kKeep];
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u) {
+            const bool on = info.x + u < info.y;
+            v[u] = on ? __ldcg(p + info.x + u) : 0.0;
+            w[u] = on ? __ldcg(k.r + info.x + u) : 0.0;
+        }
+        const int dz = info.z - info.x;      // the diagonal's place, below 0 if there is none
+        double acc = 0.0;
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u)
+            if (u == dz) acc = fma(beta, v[u], w[u]) * (double)s[u];
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u) {
+            if (info.x + u >= info.y) break;
+            if (u != dz) acc = fma(fma(beta, v[u], w[u]), (double)s[u], acc);
+        }
+        return acc;
+    }
+};
+
 template <typename T, bool RES>
 __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
     const int64_t step = (int64_t)gridDim.x * kCgT, e0 = blockIdx.x * (int64_t)kCgT + threadIdx.x;
@@ -759,7 +804,8 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
     // RES: entry e0's state
     int i = 0, j = 0, te = 0;
     int4 ri = make_int4(0, 0, -1, 0), rj = ri;
-    double hd = 0.0, xe = 0.0, re = 0.0, pe = 0.0, ape = 0.0;      // hd: 1 / w_ii^2's w_ii^2 on the diagonal
+    double hd = 0.0, xe = 0.0, re = 0.0, pe = 0.0, ape = 0.0;      // hd: lambda2, on the diagonal + 1 / w_ii^2
+    CgRow<T> si, sj;
     const bool own = RES && e0 < k.nnz;
     double s = 0.0;
     if constexpr (RES) {
@@ -769,8 +815,10 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
             te = k.tr[e0];
             ri = k.rinfo[i];
             rj = k.rinfo[j];
+            si.init(k, ri, j);
+            sj.init(k, rj, i);
             const double w = (double)k.om.cv[e0];
-            hd = i == j ? w * w : 0.0;
+            hd = i == j ? k.lam2 + 1.0 / (w * w) : k.lam2;
             re = k.b[e0];
             k.r[e0] = re;
             k.p0[e0] = re;
@@ -788,7 +836,7 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
     }
     cg_block_sum(s, part[0] + blockIdx.x);
     bool alive = cg_barrier(k.st, target);
-    double rr = alive ? cg_total(part[0]) : 0.0, beta = 0.0;       // the first direction is r itself
+    double rr = alive ? cg_total<true>(part[0], 1.0).total : 0.0, beta = 0.0;       // the first direction is r itself
     const double rr0 = rr;
     int done = rr == 0.0 ? 1 : 0;
     int64_t it = 0;
@@ -799,15 +847,12 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
         s = 0.0;
         if constexpr (RES) {
             if (own) {
-                const double Te = cg_row_dot(k, ri, i, j, p_old, beta);
-                const double Tt = te >= 0 && te != (int)e0 ? cg_row_dot(k, rj, j, i, p_old, beta) : Te;
+                const double Te = si.dot(k, ri, i, j, p_old, beta);
+                const double Tt = te >= 0 && te != (int)e0 ? sj.dot(k, rj, j, i, p_old, beta) : Te;
                 pe = fma(beta, pe, re);
                 p_new[e0] = pe;
-                double o = 0.5 * (Te + Tt);
-                o += k.lam2 * pe;
-                if (i == j) o += pe / hd;
-                ape = o;
-                s = fma(pe, o, s);
+                ape = fma(hd, pe, 0.5 * (Te + Tt));
+                s = fma(pe, ape, s);
             }
         } else {
             for (int64_t e = e0; e < k.nnz; e += step) {
@@ -828,10 +873,10 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
         }
         cg_block_sum(s, part[1] + blockIdx.x);
         if (!(alive = cg_barrier(k.st, target))) break;
-        const double pap = cg_total(part[1]);
+        const CgSum pap = cg_total<false>(part[1], rr);
         ++it;
-        if (!(pap > 0.0)) { done = 2; break; }                     // H not positive definite along p
-        const double alpha = rr / pap;
+        if (!(pap.total > 0.0)) { done = 2; break; }               // H not positive definite along p
+        const double alpha = pap.ratio;
         // x, r and <r, r>
         s = 0.0;
         if constexpr (RES) {
@@ -851,10 +896,10 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
         }
         cg_block_sum(s, part[0] + blockIdx.x);
         if (!(alive = cg_barrier(k.st, target))) break;
-        const double v = cg_total(part[0]);
-        beta = rr > 0.0 ? v / rr : 0.0;
-        rr = v;
-        if (v <= k.tol2 * rr0) done = 1;
+        const CgSum v = cg_total<true>(part[0], rr);
+        beta = rr > 0.0 ? v.ratio : 0.0;
+        rr = v.total;
+        if (rr <= k.tol2 * rr0) done = 1;
     }
     // <x, sign(Omega_A) off the diagonal> and <x, Omega_A>
     double s1 = 0.0, s2 = 0.0;
@@ -873,9 +918,9 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
     cg_block_sum(s2, part[3] + blockIdx.x);
     if (alive) alive = cg_barrier(k.st, target);
     if (blockIdx.x == 0 && alive) {
-        s1 = cg_total(part[2]);
+        s1 = cg_total<true>(part[2], 1.0).total;
         __syncthreads();
-        s2 = cg_total(part[3]);
+        s2 = cg_total<true>(part[3], 1.0).total;
         if (threadIdx.x == 0) {
             k.st->rr = rr;
             k.st->rr0 = rr0;
