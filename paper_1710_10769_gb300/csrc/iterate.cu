@@ -1937,6 +1937,14 @@ k_ls_eval(const T* __restrict__ S, int64_t ld, int p, Buckets<T> bk, int stride,
 // Obs form of the line-search partials (Alg. 3 step 11): tr(D S D) restricted to
 // row i is ||X D_i||^2 / n with X D_i = sum_e D_e X^T[j_e, :]; lanes hold 4
 // consecutive samples of each 128-sample chunk of n.  [1]-[3] as in k_ls_eval.
+//
+// What bounds it: the rows of X^T that a row's entries gather, one warp per row.  A lane takes an
+// entry's M prox steps, so they are computed once instead of by every lane, and the entries
+// that move are listed in shared memory, in order, kObsAhead of their rows in flight: entry by
+// entry it was a chain of two dependent loads and M prox steps each.  The sums keep their order.
+// Measured on GB300, p = 40000, n = 100, 28 windows: 15.6 -> 8.5 ms, 260 us each near the estimate.
+constexpr int kObsAhead = 8;
+
 template <int M>
 __device__ void ls_eval_obs_body(const float* __restrict__ Xt, int64_t ldx, int64_t n, int p,
                                  const Buckets<float>& bk, double tau0, int stride, double* part_ls, Ctrl* ctrl,
@@ -1945,6 +1953,8 @@ __device__ void ls_eval_obs_body(const float* __restrict__ Xt, int64_t ldx, int6
     const int gw = (bid * kThreads + threadIdx.x) >> 5;
     const int nw = (nblocks * kThreads) >> 5;
     const bool skip = (flags0 != 0) || (ctrl->ls_accept >= 0);
+    __shared__ __align__(16) float s_d[kWarps][32][M];
+    __shared__ int s_j[kWarps][32];
     const float lam1 = (float)ctrl->lam1;
     const int h_base = ctrl->ls_base;
     float tau[M], tl1[M];
@@ -1953,7 +1963,9 @@ __device__ void ls_eval_obs_body(const float* __restrict__ Xt, int64_t ldx, int6
         tau[m] = (float)ldexp(tau0, -(h_base + m));
         tl1[m] = tau[m] * lam1;
     }
-    F2 q[M]{}, n2[M]{}, ph[M]{};
+    // [1]-[3] first, so that their sums are out of the registers when the gathers begin
+    {
+    F2 n2[M]{}, ph[M]{};
     int nb[M];
 #pragma unroll
     for (int m = 0; m < M; ++m) nb[m] = 0;
@@ -1973,33 +1985,75 @@ __device__ void ls_eval_obs_body(const float* __restrict__ Xt, int64_t ldx, int6
                 }
             }
         }
+    }
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        const F2 b = warp_sum(n2[m]), c = warp_sum(ph[m]);
+        int dd = nb[m];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dd += __shfl_xor_sync(kFull, dd, o);
+        if (lane == 0) {
+            red[warp][m][1] = acc_value(b);
+            red[warp][m][2] = acc_value(c); red[warp][m][3] = (double)dd;
+        }
+    }
+    }
+    F2 q[M]{};
+    for (int i = skip ? p : gw; i < p; i += nw) {
+        const int beg = bk.off[i], L = bk.len[i];
         for (int64_t c0 = 0; c0 < n; c0 += 128) {
             const int64_t c = c0 + lane * 4;
             float u[M][4];
 #pragma unroll
             for (int m = 0; m < M; ++m) u[m][0] = u[m][1] = u[m][2] = u[m][3] = 0.f;
             bool any = false;
-            for (int e = 0; e < L; ++e) {
-                const int je = bk.col_b[beg + e];
-                const float om = bk.om_b[beg + e], g = bk.g[beg + e];
-                float d[M];
+            for (int e0 = 0; e0 < L; e0 += 32) {
+                // 32 entries, one per lane; those that move go into the warp's list in order
+                const int e = e0 + lane;
                 bool act = false;
+                int je = 0;
+                float d[M];
+                if (e < L) {
+                    je = bk.col_b[beg + e];
+                    const float om = bk.om_b[beg + e], g = bk.g[beg + e];
 #pragma unroll
-                for (int m = 0; m < M; ++m) {
-                    d[m] = prox_entry(om, g, tau[m], tl1[m], je == i) - om;
-                    act |= d[m] != 0.f;
+                    for (int m = 0; m < M; ++m) {
+                        d[m] = prox_entry(om, g, tau[m], tl1[m], je == i) - om;
+                        act |= d[m] != 0.f;
+                    }
                 }
-                if (!act) continue;
-                any = true;
-                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (c < ldx) x = __ldg(reinterpret_cast<const float4*>(Xt + (int64_t)je * ldx + c));
+                const unsigned moved = __ballot_sync(kFull, act);
+                if (act) {
+                    const int at = __popc(moved & ((1u << lane) - 1u));
+                    s_j[warp][at] = je;
 #pragma unroll
-                for (int m = 0; m < M; ++m) {
-                    u[m][0] = fmaf(d[m], x.x, u[m][0]);
-                    u[m][1] = fmaf(d[m], x.y, u[m][1]);
-                    u[m][2] = fmaf(d[m], x.z, u[m][2]);
-                    u[m][3] = fmaf(d[m], x.w, u[m][3]);
+                    for (int m = 0; m < M; ++m) s_d[warp][at][m] = d[m];
                 }
+                __syncwarp();
+                const int cnt = __popc(moved);
+                any |= cnt > 0;
+                for (int t = 0; t < cnt; t += kObsAhead) {
+                    float4 x[kObsAhead];
+#pragma unroll
+                    for (int v = 0; v < kObsAhead; ++v) {
+                        x[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (t + v < cnt && c < ldx)
+                            x[v] = __ldg(reinterpret_cast<const float4*>(Xt + (int64_t)s_j[warp][t + v] * ldx + c));
+                    }
+#pragma unroll
+                    for (int v = 0; v < kObsAhead; ++v) {
+                        if (t + v >= cnt) break;
+#pragma unroll
+                        for (int m = 0; m < M; ++m) {
+                            const float dm = s_d[warp][t + v][m];
+                            u[m][0] = fmaf(dm, x[v].x, u[m][0]);
+                            u[m][1] = fmaf(dm, x[v].y, u[m][1]);
+                            u[m][2] = fmaf(dm, x[v].z, u[m][2]);
+                            u[m][3] = fmaf(dm, x[v].w, u[m][3]);
+                        }
+                    }
+                }
+                __syncwarp();
             }
             if (!any) break;
 #pragma unroll
@@ -2015,14 +2069,8 @@ __device__ void ls_eval_obs_body(const float* __restrict__ Xt, int64_t ldx, int6
     const double inv_n = 1.0 / (double)n;
 #pragma unroll
     for (int m = 0; m < M; ++m) {
-        const F2 a = warp_sum(q[m]), b = warp_sum(n2[m]), c = warp_sum(ph[m]);
-        int dd = nb[m];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dd += __shfl_xor_sync(kFull, dd, o);
-        if (lane == 0) {
-            red[warp][m][0] = acc_value(a) * inv_n; red[warp][m][1] = acc_value(b);
-            red[warp][m][2] = acc_value(c); red[warp][m][3] = (double)dd;
-        }
+        const F2 a = warp_sum(q[m]);
+        if (lane == 0) red[warp][m][0] = acc_value(a) * inv_n;
     }
     __syncthreads();
     if (threadIdx.x < M * 4) {
