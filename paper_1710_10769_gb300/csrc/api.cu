@@ -176,6 +176,7 @@ struct hpc_ctx {
     void* yp[2] = {nullptr, nullptr};
     int2* pairs = nullptr;
     int64_t npairs = 0;
+    void* obs_bnd = nullptr;      // the block pairs' bounds (ObsBounds)
     CUtensorMap obs_maps[4];
     // device buffers the handle holds (address -> bytes), for hpc_get_info
     std::unordered_map<void*, size_t> held;
@@ -360,15 +361,23 @@ int regrow(hpc_ctx* h, int64_t need) {
     return HPC_OK;
 }
 
-// Obs (Alg. 3 steps 2, 4-6): Y^T = Omega X^T, its MMA panels, and the paired-tile
-// Z GEMM with the screening emission.
+// Obs (Alg. 3 steps 2, 4-6): Y^T = Omega X^T, its MMA panels, the block pairs that can emit,
+// and the paired-tile Z GEMM with the screening emission on them.
 int obs_screen(hpc_ctx* h, const hpc::IterBufs<float>& b, cudaStream_t s) {
     const int p = (int)h->p;
     hpc::launch_row_info<float>(p, b.cur, h->rinfo, as<float>(h->rdv), s);
-    hpc::launch_spmm_dense<float>(p, b.cur, h->rinfo, as<float>(h->rdv), h->xt, h->ldx, h->ldx, h->yt, h->ldx, s);
-    hpc::launch_obs_split(h->precision, h->yt, p, h->ldx, h->ldx, h->yp[0], h->yp[1], h->n, h->p, s);
-    cudaError_t e = hpc::launch_obs_pairs(h->precision, h->obs_maps, h->pairs, h->npairs, h->n, p, b.cur.rp, b.cur.ci,
-                                          b.cur.cv, b.em, h->d_ctrl, s, h->tune.gram_chunk, h->tune.gram_lead);
+    cudaError_t e = cudaSuccess;
+    if (h->obs_bnd) {
+        e = hpc::launch_obs_rows(h->precision, h->n, h->p, b.cur, h->rinfo, as<float>(h->rdv), h->xt, h->ldx, h->yt,
+                                 h->yp[0], h->yp[1], h->obs_bnd, h->pairs, h->npairs, h->d_ctrl, s, h->tune.gram_chunk,
+                                 h->tune.gram_lead);
+    } else {
+        hpc::launch_spmm_dense<float>(p, b.cur, h->rinfo, as<float>(h->rdv), h->xt, h->ldx, h->ldx, h->yt, h->ldx, s);
+        hpc::launch_obs_split(h->precision, h->yt, p, h->ldx, h->ldx, h->yp[0], h->yp[1], h->n, h->p, s);
+    }
+    if (e != cudaSuccess) { set_cuda_error(e, "obs rows", __LINE__); return HPC_ERR_CUDA; }
+    e = hpc::launch_obs_pairs(h->precision, h->obs_maps, h->pairs, h->npairs, h->obs_bnd, h->n, p, b.cur.rp, b.cur.ci,
+                              b.cur.cv, b.em, h->d_ctrl, s, h->tune.gram_chunk, h->tune.gram_lead);
     if (e != cudaSuccess) { set_cuda_error(e, "obs pair GEMM", __LINE__); return HPC_ERR_CUDA; }
     return HPC_OK;
 }
@@ -1152,6 +1161,7 @@ int load_x(hpc_ctx* h, const void* X, int xdt, int on_host) {
         hpc::launch_transpose(Xd, xdt, h->n, h->p, h->p, h->xt, HPC_F32, h->ldx, 1.0, h->stream);
         hpc::launch_obs_split(prec, h->xt, h->p, h->ldx, h->ldx, h->xp[0], h->xp[1], h->n, h->p, h->stream);
         e = cudaGetLastError();
+        if (e == cudaSuccess && h->obs_bnd) e = hpc::launch_obs_reset(h->obs_bnd, h->p, h->xt, h->ldx, h->stream);
     } else if (prec == HPC_PREC_FP64 || prec == HPC_PREC_FP32) {
         e = hpc::gram_simt(Xd, xdt, h->n, h->p, h->S, h->vdt, h->ld, h->stream, &launches);
     } else {
@@ -1257,7 +1267,7 @@ void destroy(hpc_ctx* h) {
     void* ptrs[] = {h->S, h->rp[0], h->rp[1], h->ci[0], h->ci[1], h->cv[0], h->cv[1], h->bk_cnt, h->bk_off,
                     h->bk_cur, h->bk_len, h->cnt2, h->scan_part, h->part_obj, h->part_ls, h->d_ctrl, h->gram_scratch,
                     h->rinfo, h->rdv, h->adj_buf, h->offlist, h->xt, h->yt, h->xp[0], h->xp[1],
-                    h->yp[0], h->yp[1], h->pairs, h->bk_uoff, h->pmask, h->seqoff, h->bk_long,
+                    h->yp[0], h->yp[1], h->pairs, h->obs_bnd, h->bk_uoff, h->pmask, h->seqoff, h->bk_long,
                     h->m1, h->m1g, h->colmax, h->pairs_list, h->row_items, h->x_stage, h->bar, h->loop_ws};
     for (void* q : ptrs) release(h, q);
     if (h->h_ctrl) cudaFreeHost(h->h_ctrl);
@@ -1395,6 +1405,7 @@ int hpc_create(hpc_handle* out, const void* X, hpc_dtype xdt, int64_t n, int64_t
         h->npairs = (int64_t)pl.size();
         CK(hold(h, &h->pairs, pl.size() * sizeof(int2)));
         CK(cudaMemcpy(h->pairs, pl.data(), pl.size() * sizeof(int2), cudaMemcpyHostToDevice));
+        if (hpc::obs_bounds_bytes(p)) CK(hold(h, &h->obs_bnd, hpc::obs_bounds_bytes(p)));
         if (!hpc::obs_make_maps(prec, h->yp[0], h->yp[1], h->xp[0], h->xp[1], n, p, h->obs_maps)) {
             std::snprintf(g_last_error, sizeof g_last_error, "TMA descriptors of the Obs panels could not be encoded");
             return fail(HPC_ERR_NOT_IMPLEMENTED);

@@ -264,7 +264,26 @@ void launch_obs_split(int precision, const float* in, int64_t rows, int64_t cols
                       int64_t n, int64_t p, cudaStream_t s);
 bool obs_make_maps(int precision, const void* y_hi, const void* y_lo, const void* x_hi, const void* x_lo, int64_t n,
                    int64_t p, CUtensorMap* maps);
-cudaError_t launch_obs_pairs(int precision, const CUtensorMap* maps, const int2* pairs, int64_t npairs, int64_t n,
+// The block pairs that a pass has to take: per pair a certified bound of |n Z| in it, per block
+// of rows the norms that carry the bounds from pass to pass (all in one buffer).
+struct ObsBounds {
+    int *count, *poison;                    // pairs selected; set when a pass was cut short
+    unsigned *nx, *s, *r, *y, *yprev;       // per block: |x_j|, |s_i|, |d_i|, |y_i|, the last pass's |y_i| (float bits)
+    float *eps_prev, *dold;                 // the last pass's obs_eps and w_ii
+    float* b;                               // per pair
+    int* sel;
+    unsigned char *mark, *fresh;            // per pair: off-diagonal support in it; taken by the last pass
+    int nb, npairs;
+};
+size_t obs_bounds_bytes(int64_t p);         // 0: no bounds at this size
+ObsBounds obs_bounds(void* buf, int64_t p);
+cudaError_t launch_obs_reset(void* bounds, int64_t p, const float* xt, int64_t ldx, cudaStream_t s);
+cudaError_t launch_obs_rows(int precision, int64_t n, int64_t p, Csr<float> om, const int4* rinfo, const float* rdv,
+                            const float* xt, int64_t ldx, float* yt, void* hi, void* lo, void* bounds,
+                            const int2* pairs, int64_t npairs, const Ctrl* ctrl, cudaStream_t s, int64_t chunk_k,
+                            int64_t lead_k);
+cudaError_t launch_obs_pairs(int precision, const CUtensorMap* maps, const int2* pairs, int64_t npairs, void* bounds,
+                             int64_t n,
                              int p, const int* rp, const int* ci, const float* cv, Emit<float> em,
                              Ctrl* ctrl, cudaStream_t s, int64_t chunk_k = 0, int64_t lead_k = 0);
 

@@ -31,6 +31,7 @@ namespace {
 constexpr int kT = 128;                    // tile edge (UMMA M = N = 128)
 constexpr int kRowB = 128;                 // bytes per swizzle row
 constexpr int kPanelTile = kT * kRowB;     // 16 KB
+constexpr int kObsBand = 8;                // row blocks per band of the pair list
 constexpr uint32_t kTmemCols = 256;        // one accumulator pair: two 128-column FP32 accumulators
 constexpr long long kWaitLimit = 1ll << 22;     // polls of at most 1 us each
 
@@ -212,11 +213,15 @@ __device__ __forceinline__ void row_tile_support(const int* __restrict__ rp, con
 // pair_full / pair_empty hand the pair slots around, sup_full the masks, acc_full /
 // acc_empty the accumulator pairs.  Every wait is bounded; after an abort every
 // role stops, the loads in flight drain and TMEM is freed.
+//
+// Only the pairs of ob.sel are taken (see k_obs_list); each leaves the largest |n Z_ij|
+// and |n Z_ji| that it found in ob.b.  The K steps whose 16 (TF32: 8) elements are all padding
+// are left out: at n = 100 one step in eight.
 template <int MODE>
 __global__ void __launch_bounds__(kObsThreads, 1)
 k_obs_pair(const __grid_constant__ CUtensorMap ya, const __grid_constant__ CUtensorMap yb,
            const __grid_constant__ CUtensorMap xa, const __grid_constant__ CUtensorMap xb, const int2* __restrict__ pairs,
-           int npairs, int k_tiles, int p, int64_t n, const int* __restrict__ rp, const int* __restrict__ ci,
+           const ObsBounds ob, float eps, int k_tiles, int p, int64_t n, const int* __restrict__ rp, const int* __restrict__ ci,
            const float* __restrict__ cv, Emit<float> em, Ctrl* __restrict__ ctrl, int chunk_kt, int lead_kt) {
     using C = ObsCfg<MODE>;
     constexpr int R = C::kRing;
@@ -233,16 +238,26 @@ k_obs_pair(const __grid_constant__ CUtensorMap ya, const __grid_constant__ CUten
     uint64_t* pair_empty = pair_full + R;        // [R]
     uint64_t* sup_full = pair_empty + R;         // [R]
     int2* s_pair = reinterpret_cast<int2*>(sup_full + R);                                  // [R]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_pair + R);
+    int* s_id = reinterpret_cast<int*>(s_pair + R);                                        // [R]
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_id + R);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    static_assert(8 * (2 * C::kStages + 4 + 3 * R) + 8 * R + 8 <= C::kCtlBytes, "control area");
+    static_assert(8 * (2 * C::kStages + 4 + 3 * R) + 12 * R + 8 <= C::kCtlBytes, "control area");
     static_assert(C::kSmem <= 232448, "shared memory per block");
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (chunk_kt < 1) chunk_kt = 1;
     if (lead_kt < chunk_kt) lead_kt = chunk_kt;
     const int nch = num_chunks(k_tiles, chunk_kt, lead_kt);
+    // without bounds (ob.b null) every pair is taken
+    const bool bounded = ob.b != nullptr;
+    const int npairs = bounded ? __ldcg(ob.count) : ob.npairs;
 
+    // this pass's norms and eps become the last pass's, and the maxima start at 0 again
+    if (bounded && blockIdx.x == 0 && threadIdx.x == 0) *ob.eps_prev = eps;
+    for (int t = blockIdx.x * kObsThreads + threadIdx.x; bounded && t < ob.nb; t += gridDim.x * kObsThreads) {
+        ob.yprev[t] = ob.y[t];
+        ob.s[t] = ob.r[t] = ob.y[t] = 0u;
+    }
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&empty[s], 1); }
         for (int b = 0; b < 2; ++b) { ptx::mbar_init(&acc_full[b], 1); ptx::mbar_init(&acc_empty[b], kEpiWarps); }
@@ -281,9 +296,11 @@ k_obs_pair(const __grid_constant__ CUtensorMap ya, const __grid_constant__ CUten
                                             kWaitLimit))
                     return false;
                 const int idx = nxt;
-                const int2 pr = idx < npairs ? pairs[idx] : make_int2(-1, -1);
+                const int id = idx >= npairs ? -1 : bounded ? ob.sel[idx] : idx;
+                const int2 pr = id >= 0 ? pairs[id] : make_int2(-1, -1);
                 if (idx < npairs) nxt = atomicAdd(&ctrl->obs_next, 1);
                 s_pair[slot] = pr;
+                s_id[slot] = id;
                 ptx::mbar_arrive(&pair_full[slot]);
                 ++pub;
                 pub_done = pr.x < 0;
@@ -359,8 +376,11 @@ k_obs_pair(const __grid_constant__ CUtensorMap ya, const __grid_constant__ CUten
                             const uint32_t st = ptx::smem_u32(smem + s * C::kStageBytes);
                             const uint32_t a_hi = st, b_hi = st + kPanelTile, a_lo = st + 2 * kPanelTile,
                                            b_lo = st + 3 * kPanelTile;
+                            const int steps = (int)min((int64_t)(C::kBK / C::kMmaK),
+                                                       (n - (int64_t)kt * C::kBK + C::kMmaK - 1) / C::kMmaK);
 #pragma unroll
                             for (int kk = 0; kk < C::kBK / C::kMmaK; ++kk) {
+                                if (kk >= steps) break;
                                 const uint32_t off = kk * 32;
                                 const uint32_t acc0 = (kt > kt0 || kk > 0) ? 1u : 0u;
                                 umma<MODE>(d, smem_desc_sw128(a_hi + off), smem_desc_sw128(b_hi + off), idesc, acc0);
@@ -476,6 +496,15 @@ k_obs_pair(const __grid_constant__ CUtensorMap ya, const __grid_constant__ CUten
             const uint32_t sm[2] = {half ? m4.z : m4.x, half ? m4.w : m4.y};
             const int before0 = half ? __popc(m4.x) + __popc(m4.y) : 0;
             const bool mine = g < p;
+            // the pair's largest |n Z| as integers, which order non-negative floats and put NaN last
+            if (bounded) {
+                uint32_t mx = 0u;
+#pragma unroll
+                for (int q = 0; q < 64; ++q)
+                    mx = max(mx, max(__float_as_uint(za[q]) & 0x7fffffffu, __float_as_uint(zb[q]) & 0x7fffffffu));
+                mx = __reduce_max_sync(kFull, mx);
+                if (lane == 0) atomicMax(reinterpret_cast<unsigned*>(ob.b) + s_id[slot], mx);
+            }
             uint32_t eb[2];
             int cnt = 0;
 #pragma unroll
@@ -546,6 +575,7 @@ k_obs_pair(const __grid_constant__ CUtensorMap ya, const __grid_constant__ CUten
     if (*abort_flag) {
         if (threadIdx.x == 0) {
             atomicOr(&ctrl->flags, kFlagTimeout);
+            if (bounded) *ob.poison = 1;
             for (long long g = issued > C::kStages ? issued - C::kStages : 0; g < issued; ++g) {
                 const int s = (int)(g % C::kStages);
                 const uint32_t ph = (uint32_t)(g / C::kStages) & 1u;
@@ -560,6 +590,177 @@ k_obs_pair(const __grid_constant__ CUtensorMap ya, const __grid_constant__ CUten
     }
 }
 
+// ---------------------------------------------------------------- which block pairs a pass needs
+// A pass over all block pairs is 2 p^2 n products (times three in BF16X3) however little Omega
+// has moved: about 1 ms at p = 40000, n = 100, every iteration.  But a pair emits nothing unless
+// it holds support or a |Z_ij| above lambda1, and near the estimate Z hardly moves.  So each
+// pair keeps a certified bound of the largest |n Z_ij|, |n Z_ji| in it, and a pass takes only
+// the pairs on the diagonal, with an off-diagonal support entry, or whose bound exceeds the
+// threshold: the emitted entries are those of a full pass.
+//
+// With y_i the stored FP32 rows of Y^T and n z_ij = <y_i, x_j> exactly:
+//   y_i = s_i y_i(last pass) + d_i with s_i = w_ii / w_ii(last pass), so that a row with the
+//   diagonal alone has d_i = 0 up to rounding, and |n z_ij| <= |s_i| |n z_ij(last)| + |d_i| |x_j|;
+//   the tensor product differs from n z_ij by at most eps |y_i| |x_j| (obs_eps).
+// Per 128-row block the largest |s_i|, |d_i|, |y_i| and |x_j| stand for all rows; every operation
+// rounds up (the norms carry 1% for their FP32 sums).  NaN and infinities make a bound that no
+// comparison passes: such pairs are taken.
+// Measured on GB300, solves in ms, without and with bounds: p = 24000, n = 100, lambda1 = 0.55
+// 16.4 -> 12.0; p = 24000, n = 130, lambda1 = 0.46 21.6 -> 16.1; p = 12000, n = 100 8.3 -> 7.9;
+// p = 40000, n = 100, lambda1 = 0.46, where nearly every pair holds an entry to emit, the same.
+
+// position of block pair (I, J), I <= J, in obs_pair_list's order
+__host__ __device__ __forceinline__ long long obs_pair_index(int I, int J, int nb) {
+    const int b0 = I / kObsBand * kObsBand, hb = nb - b0 < kObsBand ? nb - b0 : kObsBand, c = J - b0;
+    const long long before = (long long)b0 * nb - (long long)b0 * (b0 - 1) / 2;
+    return before + (c <= hb ? (long long)c * (c + 1) / 2 : hb * (hb + 1) / 2 + (long long)(c - hb) * hb) + (I - b0);
+}
+
+__device__ __forceinline__ float warp_sum_up(float x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+    return x;
+}
+
+template <int MODE>
+__device__ __forceinline__ void split_store(float x, void* hi, void* lo, int64_t t) {
+    if constexpr (MODE == kObsTf32) {
+        uint32_t u;
+        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(u) : "f"(x));
+        static_cast<float*>(hi)[t] = __uint_as_float(u);
+    } else {
+        const __nv_bfloat16 h = __float2bfloat16_rn(x);
+        static_cast<__nv_bfloat16*>(hi)[t] = h;
+        static_cast<__nv_bfloat16*>(lo)[t] = __float2bfloat16_rn(x - __bfloat162float(h));
+    }
+}
+
+// Y^T = Omega X^T in k_spmm_dense's order (w_ii x_i first, then the neighbours ascending), its
+// panels, and the bounds' |s_i|, |d_i|, |y_i| per block of rows.  Warp per row; ld = n padded
+// to 64, the padding of X^T is zero.
+template <int MODE>
+__global__ void __launch_bounds__(256)
+k_obs_rows(int p, int64_t rows_pad, Csr<float> om, const int4* __restrict__ rinfo, const float* __restrict__ rdv,
+           const float* __restrict__ xt, int64_t ld, float* __restrict__ yt, void* hi, void* lo, const ObsBounds ob) {
+    __shared__ unsigned m[3];
+    const int lane = threadIdx.x & 31;
+    const int64_t i = blockIdx.x * 8ll + (threadIdx.x >> 5);
+    if (threadIdx.x < 3) m[threadIdx.x] = 0u;
+    __syncthreads();
+    if (i < p) {
+        const int4 info = rinfo[i];
+        const float dv = rdv[i], s = __fdiv_rn(dv, ob.dold[i]);
+        float d2 = 0.f, y2 = 0.f;
+        for (int64_t c0 = lane; c0 < ld; c0 += 128) {
+            float acc[4], old[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int64_t c = c0 + 32 * v;
+                acc[v] = c < ld ? __fmul_rn(dv, xt[i * ld + c]) : 0.f;
+                old[v] = c < ld ? yt[i * ld + c] : 0.f;
+            }
+            for (int q = info.x; q < info.y; ++q) {
+                if (q == info.z) continue;
+                const int64_t k = om.ci[q];
+                const float w = om.cv[q];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const int64_t c = c0 + 32 * v;
+                    if (c < ld) acc[v] = __fmaf_rn(w, xt[k * ld + c], acc[v]);
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int64_t c = c0 + 32 * v;
+                if (c < ld) {
+                    yt[i * ld + c] = acc[v];
+                    split_store<MODE>(acc[v], hi, lo, i * ld + c);
+                    const float d = __fmaf_rn(-s, old[v], acc[v]);
+                    d2 = __fmaf_rn(d, d, d2);
+                    y2 = __fmaf_rn(acc[v], acc[v], y2);
+                }
+            }
+        }
+        d2 = warp_sum_up(d2);
+        y2 = warp_sum_up(y2);
+        if (lane == 0) {
+            ob.dold[i] = dv;
+            // 1e-18: squares below the smallest float
+            atomicMax(&m[0], __float_as_uint(fabsf(s)));
+            atomicMax(&m[1], __float_as_uint(__fmaf_ru(sqrtf(d2), 1.01f, 1e-18f)));
+            atomicMax(&m[2], __float_as_uint(__fmaf_ru(sqrtf(y2), 1.01f, 1e-18f)));
+        }
+    } else if (i < rows_pad) {
+        for (int64_t c = lane; c < ld; c += 32) split_store<MODE>(0.f, hi, lo, i * ld + c);
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        unsigned* out = threadIdx.x == 0 ? ob.s : threadIdx.x == 1 ? ob.r : ob.y;
+        const unsigned v = m[threadIdx.x] & 0x7fffffffu;
+        if (v) atomicMax(out + blockIdx.x * 8 / kT, v);
+    }
+}
+
+// the largest |x_j| of each 128-row block of X^T
+__global__ void __launch_bounds__(256) k_obs_norms(int p, const float* __restrict__ xt, int64_t ld, unsigned* nx) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = blockIdx.x * 8ll + (threadIdx.x >> 5);
+    if (i >= p) return;
+    float x2 = 0.f;
+    for (int64_t c = lane; c < ld; c += 32) x2 = __fmaf_rn(xt[i * ld + c], xt[i * ld + c], x2);
+    x2 = warp_sum_up(x2);
+    if (lane == 0) atomicMax(nx + i / kT, __float_as_uint(__fmaf_ru(sqrtf(x2), 1.01f, 1e-18f)) & 0x7fffffffu);
+}
+
+// the block pairs with an off-diagonal support entry; warp per row
+__global__ void __launch_bounds__(256) k_obs_mark(int p, const int* __restrict__ rp, const int* __restrict__ ci,
+                                                  const ObsBounds ob) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ob.count = 0;
+    const int lane = threadIdx.x & 31;
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= p) return;
+    const int I = i / kT;
+    for (int q = rp[i] + lane; q < rp[i + 1]; q += 32) {
+        const int J = ci[q] / kT;
+        if (J > I) ob.mark[obs_pair_index(I, J, ob.nb)] = 1;
+    }
+}
+
+// The pairs to take, a thread per pair.
+__global__ void __launch_bounds__(256) k_obs_list(const int2* __restrict__ pairs, int npairs, int64_t n, float eps,
+                                                  const ObsBounds ob, const Ctrl* __restrict__ ctrl) {
+    const float thr = (float)((double)(float)ctrl->lam1 * (double)n * (1.0 - 0x1p-20));     // k_obs_pair's
+    const int lane = threadIdx.x & 31;
+    const bool all = *ob.poison != 0;
+    const float eps_prev = *ob.eps_prev;
+    for (int64_t t0 = blockIdx.x * 256ll; t0 < npairs; t0 += gridDim.x * 256ll) {
+        const int64_t t = t0 + threadIdx.x;
+        bool take = false;
+        if (t < npairs) {
+            const int2 pr = pairs[t];
+            const int I = pr.x, J = pr.y;
+            const float nxi = __uint_as_float(ob.nx[I]), nxj = __uint_as_float(ob.nx[J]);
+            // the larger of a[I] |x|_J and a[J] |x|_I, NaN kept
+            auto cross = [&](const unsigned* a) {
+                const float u = __fmul_ru(__uint_as_float(a[I]), nxj), v = __fmul_ru(__uint_as_float(a[J]), nxi);
+                return __uint_as_float(max(__float_as_uint(u) & 0x7fffffffu, __float_as_uint(v) & 0x7fffffffu));
+            };
+            float b = ob.b[t];
+            if (ob.fresh[t]) b = __fmaf_ru(eps_prev, cross(ob.yprev), b);
+            b = __fmaf_ru(__uint_as_float(max(ob.s[I], ob.s[J])), b, cross(ob.r));
+            take = all || I == J || ob.mark[t] || !(__fmaf_ru(eps, cross(ob.y), b) <= thr);
+            ob.mark[t] = 0;
+            ob.fresh[t] = take;
+            ob.b[t] = take ? 0.f : b;
+        }
+        const unsigned vote = __ballot_sync(kFull, take);
+        int at = 0;
+        if (lane == 0 && vote) at = atomicAdd(ob.count, __popc(vote));
+        at = __shfl_sync(kFull, at, 0);
+        if (take) ob.sel[at + __popc(vote & ((1u << lane) - 1u))] = (int)t;
+    }
+}
+
 // FP32 rows (rows x ldi, K contiguous) -> K-major panels (rows_pad x n_pad) of the MMA input type.
 template <int MODE>
 __global__ void k_obs_split(const float* __restrict__ in, int64_t rows, int64_t cols, int64_t ldi, void* hi, void* lo,
@@ -568,15 +769,7 @@ __global__ void k_obs_split(const float* __restrict__ in, int64_t rows, int64_t 
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = t / n_pad, k = t % n_pad;
         const float x = (r < rows && k < cols) ? in[r * ldi + k] : 0.f;
-        if constexpr (MODE == kObsTf32) {
-            uint32_t u;
-            asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(u) : "f"(x));
-            static_cast<float*>(hi)[t] = __uint_as_float(u);
-        } else {
-            const __nv_bfloat16 h = __float2bfloat16_rn(x);
-            static_cast<__nv_bfloat16*>(hi)[t] = h;
-            static_cast<__nv_bfloat16*>(lo)[t] = __float2bfloat16_rn(x - __bfloat162float(h));
-        }
+        split_store<MODE>(x, hi, lo, t);
     }
 }
 
@@ -599,10 +792,10 @@ int64_t obs_npairs(int64_t p) {
 void obs_pair_list(int64_t p, std::vector<int2>& out) {
     const int64_t nb = (p + kT - 1) / kT;
     out.clear();
-    // bands of 8 row blocks, columns left to right: pairs in flight share panels in L2
-    for (int64_t b0 = 0; b0 < nb; b0 += 8)
+    // bands of kObsBand row blocks, columns left to right: pairs in flight share panels in L2
+    for (int64_t b0 = 0; b0 < nb; b0 += kObsBand)
         for (int64_t bj = 0; bj < nb; ++bj)
-            for (int64_t bi = b0; bi < std::min<int64_t>(b0 + 8, nb); ++bi)
+            for (int64_t bi = b0; bi < std::min<int64_t>(b0 + kObsBand, nb); ++bi)
                 if (bi <= bj) out.push_back(make_int2((int)bi, (int)bj));
 }
 
@@ -631,10 +824,88 @@ bool obs_make_maps(int precision, const void* y_hi, const void* y_lo, const void
 // K elements -> whole stages of kbk elements, at least one.
 static int kt_of(int64_t k, int kbk) { return (int)std::max<int64_t>(1, std::min<int64_t>(k / kbk, 1 << 30)); }
 
-cudaError_t launch_obs_pairs(int precision, const CUtensorMap* maps, const int2* pairs, int64_t npairs, int64_t n,
+// The tensor product's error over |y_i| |x_j|: the operands' rounding (BF16 hi + lo: 2^-18 each
+// and lo lo left out, together below 2^-15; TF32: 2^-11 each, below 2^-9), and 2^-19 per
+// accumulation step of the longest chunk (16 elements and up to three products; 17 terms, each
+// cut at the largest one's last bit) and per chunk sum.
+static float obs_eps(bool tf32, int64_t ldx, int64_t chunk_k, int64_t lead_k) {
+    if (chunk_k <= 0) chunk_k = 256;
+    if (lead_k <= 0) lead_k = 4 * chunk_k;
+    const double k = (double)std::min<int64_t>(std::max(chunk_k, lead_k) + 64, ldx);
+    const double steps = (tf32 ? k / 8 : 3 * k / 16) + (double)ldx / (double)chunk_k + 2;
+    return (float)((tf32 ? 0x1p-9 : 0x1p-15) + steps * 0x1p-19);
+}
+
+// Bounds are kept from kObsBoundPairs block pairs on (p about 11500): below, a pass over all pairs
+// takes less than the kernels that choose among them cost (p = 2000: 3.0 ms without, 3.2 with
+// bounds; p = 6000 4.6, 4.6; p = 12000 8.3, 7.9).
+constexpr int64_t kObsBoundPairs = 4096;
+size_t obs_bounds_bytes(int64_t p) {
+    if (obs_npairs(p) < kObsBoundPairs) return 0;
+    const size_t nb = (size_t)(p + kT - 1) / kT, np = (size_t)obs_npairs(p);
+    return (3 + 5 * nb + (size_t)p + 2 * np) * 4 + 2 * np;
+}
+
+ObsBounds obs_bounds(void* buf, int64_t p) {
+    const size_t nb = (size_t)(p + kT - 1) / kT, np = (size_t)obs_npairs(p);
+    ObsBounds ob{};
+    unsigned* q = static_cast<unsigned*>(buf);
+    auto take = [&](size_t k) { unsigned* r = q; q += k; return r; };
+    ob.nb = (int)nb;
+    ob.count = reinterpret_cast<int*>(take(1));
+    ob.poison = reinterpret_cast<int*>(take(1));
+    ob.eps_prev = reinterpret_cast<float*>(take(1));
+    ob.nx = take(nb);
+    ob.s = take(nb);
+    ob.r = take(nb);
+    ob.y = take(nb);
+    ob.yprev = take(nb);
+    ob.dold = reinterpret_cast<float*>(take((size_t)p));
+    ob.b = reinterpret_cast<float*>(take(np));
+    ob.sel = reinterpret_cast<int*>(take(np));
+    ob.mark = reinterpret_cast<unsigned char*>(q);
+    ob.fresh = ob.mark + np;
+    return ob;
+}
+
+// After a load: |x_j|, and bounds that no comparison passes (NaN), so that the next pass takes
+// every pair.
+cudaError_t launch_obs_reset(void* buf, int64_t p, const float* xt, int64_t ldx, cudaStream_t s) {
+    const ObsBounds ob = obs_bounds(buf, p);
+    cudaError_t e = cudaMemsetAsync(buf, 0, obs_bounds_bytes(p), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ob.b, 0xff, (size_t)obs_npairs(p) * sizeof(float), s);
+    if (e != cudaSuccess) return e;
+    k_obs_norms<<<(unsigned)((p + 7) / 8), 256, 0, s>>>((int)p, xt, ldx, ob.nx);
+    return cudaGetLastError();
+}
+
+// Y^T, its panels, and the list of block pairs of this pass.
+cudaError_t launch_obs_rows(int precision, int64_t n, int64_t p, Csr<float> om, const int4* rinfo, const float* rdv,
+                            const float* xt, int64_t ldx, float* yt, void* hi, void* lo, void* bounds,
+                            const int2* pairs, int64_t npairs, const Ctrl* ctrl, cudaStream_t s, int64_t chunk_k,
+                            int64_t lead_k) {
+    const ObsBounds ob = obs_bounds(bounds, p);
+    const int64_t rows_pad = (p + kT - 1) / kT * kT;
+    const unsigned nb = (unsigned)(rows_pad / 8);
+    const bool tf32 = precision == HPC_PREC_TF32;
+    if (tf32) k_obs_rows<kObsTf32><<<nb, 256, 0, s>>>((int)p, rows_pad, om, rinfo, rdv, xt, ldx, yt, hi, lo, ob);
+    else k_obs_rows<kObsBf16x3><<<nb, 256, 0, s>>>((int)p, rows_pad, om, rinfo, rdv, xt, ldx, yt, hi, lo, ob);
+    k_obs_mark<<<(unsigned)((p + 7) / 8), 256, 0, s>>>((int)p, om.rp, om.ci, ob);
+    const float eps = obs_eps(tf32, ldx, chunk_k, lead_k);
+    const unsigned lb = (unsigned)std::min<int64_t>((npairs + 255) / 256, 4096);
+    k_obs_list<<<lb, 256, 0, s>>>(pairs, (int)npairs, n, eps, ob, ctrl);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_obs_pairs(int precision, const CUtensorMap* maps, const int2* pairs, int64_t npairs, void* bounds,
+                             int64_t n,
                              int p, const int* rp, const int* ci, const float* cv, Emit<float> em,
                              Ctrl* ctrl, cudaStream_t s, int64_t chunk_k, int64_t lead_k) {
     const int64_t n_pad = (n + 63) / 64 * 64;
+    ObsBounds ob{};
+    if (bounds) ob = obs_bounds(bounds, p);
+    ob.npairs = (int)npairs;
+    const float eps = obs_eps(precision == HPC_PREC_TF32, n_pad, chunk_k, lead_k);
     // K elements per accumulation chunk (the Gram's BF16X3 / TF32 default when none is given)
     if (chunk_k <= 0) chunk_k = 256;
     if (lead_k <= 0) lead_k = 4 * chunk_k;
@@ -663,7 +934,7 @@ cudaError_t launch_obs_pairs(int precision, const CUtensorMap* maps, const int2*
         cudaError_t e = set_smem_once((const void*)k_obs_pair<kObsTf32>, C::kSmem, kSmemSlotObsTf32);
         if (e != cudaSuccess) return e;
         k_obs_pair<kObsTf32><<<grid, kObsThreads, C::kSmem, s>>>(maps[0], maps[1], maps[2], maps[3], pairs,
-                                                                 (int)npairs, (int)(n_pad / C::kBK), p, n, rp, ci,
+                                                                 ob, eps, (int)(n_pad / C::kBK), p, n, rp, ci,
                                                                  cv, em, ctrl, kt_of(chunk_k, C::kBK),
                                                                  kt_of(lead_k, C::kBK));
     } else {
@@ -671,7 +942,7 @@ cudaError_t launch_obs_pairs(int precision, const CUtensorMap* maps, const int2*
         cudaError_t e = set_smem_once((const void*)k_obs_pair<kObsBf16x3>, C::kSmem, kSmemSlotObsBf16x3);
         if (e != cudaSuccess) return e;
         k_obs_pair<kObsBf16x3><<<grid, kObsThreads, C::kSmem, s>>>(maps[0], maps[1], maps[2], maps[3], pairs,
-                                                                   (int)npairs, (int)(n_pad / C::kBK), p, n, rp, ci,
+                                                                   ob, eps, (int)(n_pad / C::kBK), p, n, rp, ci,
                                                                    cv, em, ctrl, kt_of(chunk_k, C::kBK),
                                                                    kt_of(lead_k, C::kBK));
     }
