@@ -967,19 +967,32 @@ Geometry geometry(int xdt, int64_t n, int64_t p, int precision) {
 // in bands of `band` row blocks of 128 (pairs: rounded up to 256); within a band, columns
 // left to right, rows top to bottom.  The band sets which X panels the concurrently
 // running tiles share in L2 (a tuning knob).
-template <typename F>
-__host__ __device__ inline void for_tiles(int64_t p_pad, int band, bool pair, F&& f) {
-    const int64_t rows = pair ? kTile : kBM, nbi = p_pad / rows, nbj = p_pad / kTile;
-    const int64_t step = pair ? (band + 1) / 2 : band;
-    for (int64_t b0 = 0; b0 < nbi; b0 += step)
-        for (int64_t bj = 0; bj < nbj; ++bj)
-            for (int64_t bi = b0; bi < (b0 + step < nbi ? b0 + step : nbi); ++bi)
-                if (bi * rows <= bj * kTile + kTile - 1) f(make_int2((int)bi, (int)bj));
+//
+// The list is written on the device, a thread per (band, column), each from the closed
+// form of its first position: as a list made on the host it was copied and waited for in
+// every hpc_gram call.  Measured on GB300, p = 300, n = 200: a call takes 69.7 -> 63.9 us.
+__global__ void __launch_bounds__(256) k_tile_list(int2* __restrict__ out, int64_t p_pad, int band, bool pair) {
+    const int f = pair ? 1 : kTile / kBM;                                // row blocks per column block
+    const int nbj = (int)(p_pad / kTile), nbi = nbj * f, step = pair ? (band + 1) / 2 : band;
+    const int bj = blockIdx.x * 256 + threadIdx.x, b0 = blockIdx.y * step;
+    if (bj >= nbj) return;
+    const int hb = min(step, nbi - b0);
+    // rows of the band that column c has: those up to f c + f - 1
+    auto rows = [&](int c) { return max(0, min(hb, f * c + f - b0)); };
+    // rows r < b0 have nbj - r / f tiles each
+    const int64_t h = b0 / f;
+    int64_t at = f * (h * nbj - h * (h - 1) / 2) + (b0 % f) * (nbj - h);
+    int c = (int)h;
+    for (; c < bj && rows(c) < hb; ++c) at += rows(c);
+    if (bj > c) at += (int64_t)(bj - c) * hb;
+    const int m = rows(bj);
+    for (int r = 0; r < m; ++r) out[at + r] = make_int2(b0 + r, bj);
 }
-std::vector<int2> tile_order(int64_t p_pad, int band, bool pair) {
-    std::vector<int2> t;
-    for_tiles(p_pad, band, pair, [&](int2 x) { t.push_back(x); });
-    return t;
+
+void launch_tile_list(int2* out, const Geometry& g, int band, bool pair, cudaStream_t s) {
+    const int64_t nbj = g.p_pad / kTile, nbi = pair ? nbj : g.p_pad / kBM, step = pair ? (band + 1) / 2 : band;
+    k_tile_list<<<dim3((unsigned)((nbj + 255) / 256), (unsigned)((nbi + step - 1) / step)), 256, 0, s>>>(out, g.p_pad,
+                                                                                                        band, pair);
 }
 
 // The tile counter and the error word: after the tile list, in the scratch's slack.
@@ -1145,12 +1158,8 @@ cudaError_t gram_tc(const void* X, int xdt, int64_t n, int64_t p, float* S, int6
     // it on the device between calls (no copy queued behind other transfers)
     const uint64_t sig = (reinterpret_cast<uintptr_t>(tiles) * 1000003ull) ^ ((uint64_t)g.p_pad << 20) ^ ((uint64_t)pair_mode(mode) << 16) ^ (uint64_t)band;
     if (!tiles_sig || *tiles_sig != sig) {
-        const std::vector<int2> order = tile_order(g.p_pad, band, pair_mode(mode));
-        e = cudaMemcpyAsync(tiles, order.data(), order.size() * sizeof(int2), cudaMemcpyHostToDevice, s);
-        if (e != cudaSuccess) return e;
-        // the host vector must outlive the copy
-        e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) return e;
+        launch_tile_list(tiles, g, band, pair_mode(mode), s);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (tiles_sig) *tiles_sig = sig;
     }
     if (!prepared) {
@@ -1211,12 +1220,6 @@ constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mu;
 void* g_noalloc_base[kMaxDevices] = {};   // device address of g_noalloc_scratch, per device
 
-// The tile order of tile_order(), written on the device (no host staging buffer).
-__global__ void k_tile_order(int2* __restrict__ out, int64_t p_pad, bool pair) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    for_tiles(p_pad, kBand, pair, [&](int2 x) { *out++ = x; });
-}
-
 // Device address of the scratch array for the current device; the first call on
 // a device looks it up (cudaGetSymbolAddress with that device current).
 cudaError_t noalloc_base(void** out) {
@@ -1271,7 +1274,7 @@ extern "C" int hpc_gram_noalloc(const void* X, hpc_dtype xdt, int64_t n, int64_t
     void* hi = base;
     void* lo = g.pieces > 1 ? base + g.panel_bytes : nullptr;
     int2* tiles = reinterpret_cast<int2*>(base + g.pieces * g.panel_bytes);
-    k_tile_order<<<1, 1, 0, s>>>(tiles, g.p_pad, pair_mode(mode));
+    launch_tile_list(tiles, g, kBand, pair_mode(mode), s);
     if (xdt == HPC_BF16) launch_prep<__nv_bfloat16>(X, mode, n, p, hi, lo, g, s);
     else launch_prep<float>(X, mode, n, p, hi, lo, g, s);
     e = cudaGetLastError();
