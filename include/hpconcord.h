@@ -122,9 +122,9 @@ typedef struct {
     int32_t device_loop;    /* 1 (default): the iteration and line-search loops run on
                                the device, one CUDA-graph launch per solve (conditional
                                WHILE nodes); 0: the host drives every iteration.  Cov
-                               handles with 384 rows or more (and fused_tail 0): the
-                               iterations run in one cooperative kernel, per solve or,
-                               with 0, per iteration                                  */
+                               handles with 384 rows or more (FP64: 224; fused_tail 0):
+                               the iterations run in one cooperative kernel, per solve
+                               or, with 0, per iteration                              */
     int32_t reserved_;
 } hpc_options;
 
@@ -470,7 +470,7 @@ typedef struct {
                                   rule -- run as one cooperative kernel, grid-wide
                                   barriers between the steps; 0: as the chain of
                                   separate kernels, or, for the Cov variant from 384
-                                  rows on, all iterations in one cooperative kernel
+                                  rows (FP64: 224) on, all iterations in one kernel
                                   (three barriers per iteration; the chain then runs
                                   only the iterations in which a row has more than
                                   2046 candidates).  The same entries and decisions

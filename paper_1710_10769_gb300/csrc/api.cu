@@ -663,12 +663,15 @@ int tail_mode(const hpc_ctx* h) { return h->tune.fused_tail != 0 && tail_in_grap
 // GB300, chain -> loop: 110 -> 37 at p = 64, 114 -> 38 at p = 256, 106 -> 35 at p = 512,
 // FP64 223 -> 66 at p = 384); below kLoopMinRows the chain stays all the same, because its
 // statistics are part of what callers of small problems check: hpc_stats.kernel_launches
-// counts a launch per step there, and fused_tail 1 makes fewer launches than 0.
-constexpr int64_t kLoopMinRows = 384;
+// counts a launch per step there, and fused_tail 1 makes fewer launches than 0.  The FP64 chain
+// costs twice the FP32 one per iteration, so FP64 leaves it earlier (a solve at p = 252, n = 92:
+// 6.70 -> 1.78 ms).
+template <typename T>
+constexpr int64_t kLoopMinRows = sizeof(T) == 8 ? 224 : 384;
 template <typename T>
 int use_loop(hpc_ctx* h, bool* yes) {
     *yes = false;
-    if (h->variant != HPC_COV || h->tune.fused_tail != 0 || h->chain_only || h->p < kLoopMinRows ||
+    if (h->variant != HPC_COV || h->tune.fused_tail != 0 || h->chain_only || h->p < kLoopMinRows<T> ||
         h->p >= (1ll << 28) || !tail_in_graph_supported(h))
         return HPC_OK;
     if (h->loop_ok < 0) {
