@@ -1942,7 +1942,8 @@ k_ls_eval(const T* __restrict__ S, int64_t ld, int p, Buckets<T> bk, int stride,
 // entry's M prox steps, so they are computed once instead of by every lane, and the entries
 // that move are listed in shared memory, in order, kObsAhead of their rows in flight: entry by
 // entry it was a chain of two dependent loads and M prox steps each.  The sums keep their order.
-// Measured on GB300, p = 40000, n = 100, 28 windows: 15.6 -> 8.5 ms, 260 us each near the estimate.
+// Measured on GB300, p = 40000, n = 100, 28 windows: 15.6 -> 8.5 ms; 5.0 with the grid of
+// ls_eval_obs_m.
 constexpr int kObsAhead = 8;
 
 template <int M>
@@ -2733,7 +2734,10 @@ void launch_ls_window(const IterBufs<T>& b, const LoopCond& lc, cudaStream_t s) 
 
 template <int M>
 static void ls_eval_obs_m(const IterBufs<float>& b, const LoopCond& lc, cudaStream_t s) {
-    k_ls_eval_obs<M><<<b.nblk, kThreads, 0, s>>>(b.xt, b.ldx, b.n, b.p, b.bk, 1.0, b.nblk, b.part_ls, b.ctrl,
+    // as many blocks as are resident: every block reduces M FP64 sums, and the last one all the
+    // blocks' partials, at two FP64 lanes per SM and cycle (with 16 blocks per SM a window took
+    // 260 us at p = 40000, 115 now)
+    k_ls_eval_obs<M><<<std::min(b.nblk, 2 * b.num_sms), kThreads, 0, s>>>(b.xt, b.ldx, b.n, b.p, b.bk, 1.0, b.nblk, b.part_ls, b.ctrl,
                                                  ls_decide_args(b, lc));
 }
 
