@@ -606,7 +606,8 @@ k_obs_pair(const __grid_constant__ CUtensorMap ya, const __grid_constant__ CUten
 // rounds up (the norms carry 1% for their FP32 sums).  NaN and infinities make a bound that no
 // comparison passes: such pairs are taken.
 // Measured on GB300, solves in ms, without and with bounds: p = 24000, n = 100, lambda1 = 0.55
-// 16.4 -> 12.0; p = 24000, n = 130, lambda1 = 0.46 21.6 -> 16.1; p = 12000, n = 100 8.3 -> 7.9;
+// 16.4 -> 12.0; p = 24000, n = 130, lambda1 = 0.46 21.6 -> 16.1; p = 12000, n = 100 8.3 -> 7.9
+// (7.2, 10.8 and 4.8 with the line search's later form);
 // p = 40000, n = 100, lambda1 = 0.46, where nearly every pair holds an entry to emit, the same.
 
 // position of block pair (I, J), I <= J, in obs_pair_list's order
@@ -637,7 +638,8 @@ __device__ __forceinline__ void split_store(float x, void* hi, void* lo, int64_t
 
 // Y^T = Omega X^T in k_spmm_dense's order (w_ii x_i first, then the neighbours ascending), its
 // panels, and the bounds' |s_i|, |d_i|, |y_i| per block of rows.  Warp per row; ld = n padded
-// to 64, the padding of X^T is zero.
+// to 64, the padding of X^T is zero.  Four neighbours' rows are in flight: the passes of a dense
+// iterate, up to 1500 neighbours a row, took 0.46 ms with one, 0.24 with four (p = 40000).
 template <int MODE>
 __global__ void __launch_bounds__(256)
 k_obs_rows(int p, int64_t rows_pad, Csr<float> om, const int4* __restrict__ rinfo, const float* __restrict__ rdv,
@@ -659,14 +661,25 @@ k_obs_rows(int p, int64_t rows_pad, Csr<float> om, const int4* __restrict__ rinf
                 acc[v] = c < ld ? __fmul_rn(dv, xt[i * ld + c]) : 0.f;
                 old[v] = c < ld ? yt[i * ld + c] : 0.f;
             }
-            for (int q = info.x; q < info.y; ++q) {
-                if (q == info.z) continue;
-                const int64_t k = om.ci[q];
-                const float w = om.cv[q];
+            for (int q0 = info.x; q0 < info.y; q0 += 4) {       // four neighbours' rows in flight
+                float w[4], x[4][4];
 #pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const int64_t c = c0 + 32 * v;
-                    if (c < ld) acc[v] = __fmaf_rn(w, xt[k * ld + c], acc[v]);
+                for (int u = 0; u < 4; ++u) {
+                    const int q = q0 + u;
+                    const bool on = q < info.y && q != info.z;
+                    const int64_t k = on ? om.ci[q] : 0;
+                    w[u] = on ? om.cv[q] : 0.f;
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        const int64_t c = c0 + 32 * v;
+                        x[u][v] = on && c < ld ? xt[k * ld + c] : 0.f;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (q0 + u >= info.y || q0 + u == info.z) continue;
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) acc[v] = __fmaf_rn(w[u], x[u][v], acc[v]);
                 }
             }
 #pragma unroll
