@@ -1942,7 +1942,7 @@ k_ls_eval(const T* __restrict__ S, int64_t ld, int p, Buckets<T> bk, int stride,
 // entry's M prox steps, so they are computed once instead of by every lane, and the entries
 // that move are listed in shared memory, in order, kObsAhead of their rows in flight: entry by
 // entry it was a chain of two dependent loads and M prox steps each.  The sums keep their order.
-// Measured on GB300, p = 40000, n = 100, 28 windows: 15.6 -> 8.5 ms; 5.0 with the grid of
+// Measured on GB300, p = 40000, n = 100, 28 windows: 15.7 -> 8.5 ms; 4.9 with the grid of
 // ls_eval_obs_m.
 constexpr int kObsAhead = 8;
 
