@@ -216,7 +216,8 @@ __device__ __forceinline__ void row_tile_support(const int* __restrict__ rp, con
 //
 // Only the pairs of ob.sel are taken (see k_obs_list); each leaves the largest |n Z_ij|
 // and |n Z_ji| that it found in ob.b.  The K steps whose 16 (TF32: 8) elements are all padding
-// are left out: at n = 100 one step in eight.
+// are left out: at n = 100 one step in eight.  Every stage holds samples (k_tiles counts no
+// stage of padding alone), so that a chunk's first step, which resets its accumulator, runs.
 template <int MODE>
 __global__ void __launch_bounds__(kObsThreads, 1)
 k_obs_pair(const __grid_constant__ CUtensorMap ya, const __grid_constant__ CUtensorMap yb,
@@ -834,6 +835,8 @@ bool obs_make_maps(int precision, const void* y_hi, const void* y_lo, const void
     return true;
 }
 
+// Stages of kbk elements that hold samples (the panels are padded to 64, two stages of TF32).
+static int k_stages(int64_t n, int kbk) { return (int)((n + kbk - 1) / kbk); }
 // K elements -> whole stages of kbk elements, at least one.
 static int kt_of(int64_t k, int kbk) { return (int)std::max<int64_t>(1, std::min<int64_t>(k / kbk, 1 << 30)); }
 
@@ -947,7 +950,7 @@ cudaError_t launch_obs_pairs(int precision, const CUtensorMap* maps, const int2*
         cudaError_t e = set_smem_once((const void*)k_obs_pair<kObsTf32>, C::kSmem, kSmemSlotObsTf32);
         if (e != cudaSuccess) return e;
         k_obs_pair<kObsTf32><<<grid, kObsThreads, C::kSmem, s>>>(maps[0], maps[1], maps[2], maps[3], pairs,
-                                                                 ob, eps, (int)(n_pad / C::kBK), p, n, rp, ci,
+                                                                 ob, eps, k_stages(n, C::kBK), p, n, rp, ci,
                                                                  cv, em, ctrl, kt_of(chunk_k, C::kBK),
                                                                  kt_of(lead_k, C::kBK));
     } else {
@@ -955,7 +958,7 @@ cudaError_t launch_obs_pairs(int precision, const CUtensorMap* maps, const int2*
         cudaError_t e = set_smem_once((const void*)k_obs_pair<kObsBf16x3>, C::kSmem, kSmemSlotObsBf16x3);
         if (e != cudaSuccess) return e;
         k_obs_pair<kObsBf16x3><<<grid, kObsThreads, C::kSmem, s>>>(maps[0], maps[1], maps[2], maps[3], pairs,
-                                                                   ob, eps, (int)(n_pad / C::kBK), p, n, rp, ci,
+                                                                   ob, eps, k_stages(n, C::kBK), p, n, rp, ci,
                                                                    cv, em, ctrl, kt_of(chunk_k, C::kBK),
                                                                    kt_of(lead_k, C::kBK));
     }
