@@ -76,6 +76,7 @@ struct hpc_ctx {
     int cur = 0;
     int64_t csr_cap = 0;
     int64_t nnz = 0;
+    bool omega_sym = true;          // the iterate equals its transpose, entry by entry
     // screening output and candidate structure
     int64_t cap = 0;                // emission capacity
     int* em_row = nullptr;
@@ -264,6 +265,12 @@ int grow_csr(hpc_ctx* h, int64_t newcap) {
     return HPC_OK;
 }
 
+// Records whether the iterate is symmetric; the captured loop depends on it (use_loop).
+void set_symmetric(hpc_ctx* h, bool sym) {
+    if (sym != h->omega_sym) h->epoch += 1;
+    h->omega_sym = sym;
+}
+
 int set_identity(hpc_ctx* h) {
     if (h->vdt == HPC_F64)
         hpc::launch_set_identity<double>({h->rp[h->cur], h->ci[h->cur], as<double>(h->cv[h->cur])}, (int)h->p, h->stream);
@@ -271,6 +278,28 @@ int set_identity(hpc_ctx* h) {
         hpc::launch_set_identity<float>({h->rp[h->cur], h->ci[h->cur], as<float>(h->cv[h->cur])}, (int)h->p, h->stream);
     CUDA_TRY(cudaGetLastError());
     h->nnz = h->p;
+    set_symmetric(h, true);
+    return HPC_OK;
+}
+
+// Whether the iterate that hpc_set_omega left in the current buffers is symmetric; waits for it.
+int check_symmetric(hpc_ctx* h) {
+    if (h->variant != HPC_COV) {
+        CUDA_TRY(cudaStreamSynchronize(h->stream));
+        return HPC_OK;
+    }
+    int* d = reinterpret_cast<int*>(h->d_ctrl + 1);
+    int asym = 0;
+    CUDA_TRY(cudaMemsetAsync(d, 0, sizeof(int), h->stream));
+    const int c = h->cur;
+    if (h->vdt == HPC_F64)
+        hpc::launch_csr_asymmetric<double>({h->rp[c], h->ci[c], static_cast<double*>(h->cv[c])}, (int)h->p, d, h->stream);
+    else
+        hpc::launch_csr_asymmetric<float>({h->rp[c], h->ci[c], static_cast<float*>(h->cv[c])}, (int)h->p, d, h->stream);
+    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaMemcpyAsync(&asym, d, sizeof asym, cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    set_symmetric(h, asym == 0);
     return HPC_OK;
 }
 
@@ -659,7 +688,9 @@ int tail_mode(const hpc_ctx* h) { return h->tune.fused_tail != 0 && tail_in_grap
 // Whether the handle's iterations run in the one-launch loop (loop.cu): the Cov
 // variant with the tail form left to the library (fused_tail 0), on a device that runs
 // cooperative kernels in graph loops, from kLoopMinRows rows on.  Allocates the loop's
-// workspace at the first call.  It is the faster form at every size (us per iteration on
+// workspace at the first call.  An iterate that is not symmetric (hpc_set_omega takes any) stays
+// with the chain, which removes the duplicates that it gives in a row's candidates; the loop's
+// buckets hold a column once.  It is the faster form at every size (us per iteration on
 // GB300, chain -> loop: 110 -> 37 at p = 64, 114 -> 38 at p = 256, 106 -> 35 at p = 512,
 // FP64 223 -> 66 at p = 384); below kLoopMinRows the chain stays all the same, because its
 // statistics are part of what callers of small problems check: hpc_stats.kernel_launches
@@ -671,7 +702,7 @@ constexpr int64_t kLoopMinRows = sizeof(T) == 8 ? 224 : 384;
 template <typename T>
 int use_loop(hpc_ctx* h, bool* yes) {
     *yes = false;
-    if (h->variant != HPC_COV || h->tune.fused_tail != 0 || h->chain_only || h->p < kLoopMinRows<T> ||
+    if (h->variant != HPC_COV || h->tune.fused_tail != 0 || h->chain_only || !h->omega_sym || h->p < kLoopMinRows<T> ||
         h->p >= (1ll << 28) || !tail_in_graph_supported(h))
         return HPC_OK;
     if (h->loop_ok < 0) {
@@ -1473,7 +1504,7 @@ int hpc_create(hpc_handle* out, const void* X, hpc_dtype xdt, int64_t n, int64_t
     h->nblk = (int)std::min<int64_t>((p + 7) / 8, 152 * 16);
     CK(hold(h, &h->part_obj, (size_t)h->nblk * 4 * sizeof(double)));
     CK(hold(h, &h->part_ls, (size_t)h->nblk * 16 * 4 * sizeof(double)));
-    CK(hold(h, &h->d_ctrl, sizeof(hpc::Ctrl) + sizeof(unsigned long long)));      // and hpc_set_omega's fault key
+    CK(hold(h, &h->d_ctrl, sizeof(hpc::Ctrl) + sizeof(unsigned long long)));      // and a word of hpc_set_omega's checks
     CK(cudaMemsetAsync(h->d_ctrl, 0, sizeof(hpc::Ctrl), h->stream));
     CK(hold(h, &h->bar, hpc::kBarWords * sizeof(unsigned)));
     CK(cudaMemsetAsync(h->bar, 0, hpc::kBarWords * sizeof(unsigned), h->stream));
@@ -1611,9 +1642,8 @@ static int set_omega_device(hpc_handle h, int64_t nnz, const int64_t* row_ptr, c
         hpc::launch_csr_import<float>(row_ptr, col, val, vdt, h->p, nnz,
                                       {h->rp[c], h->ci[c], static_cast<float*>(h->cv[c])}, h->stream);
     CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
     h->nnz = nnz;
-    return HPC_OK;
+    return check_symmetric(h);
 }
 
 int hpc_set_omega(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32_t* col, const void* val,
@@ -1660,7 +1690,7 @@ int hpc_set_omega(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32
         CUDA_TRY(cudaStreamSynchronize(h->stream));
     }
     h->nnz = nnz;
-    return HPC_OK;
+    return check_symmetric(h);
 }
 
 }  // extern "C"

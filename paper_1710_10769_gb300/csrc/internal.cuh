@@ -205,6 +205,8 @@ void launch_csr_check(const int64_t* rp, const int32_t* ci, const void* v, int v
 template <typename T>
 void launch_csr_import(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int64_t p, int64_t nnz, Csr<T> out,
                        cudaStream_t s);
+// *asym = 1 if some entry (i, j) has no equal entry (j, i).
+template <typename T> void launch_csr_asymmetric(Csr<T> c, int p, int* asym, cudaStream_t s);
 void launch_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int64_t* rows,
                      const int64_t* cols, double* out, cudaStream_t s);
 

@@ -2362,6 +2362,26 @@ __global__ void __launch_bounds__(256) k_csr_import(const int64_t* __restrict__ 
     }
 }
 
+// One warp per row: each entry's transpose by binary search in its column's row.
+template <typename T>
+__global__ void __launch_bounds__(256) k_csr_asymmetric(Csr<T> c, int p, int* asym) {
+    const int lane = threadIdx.x & 31;
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= p) return;
+    bool bad = false;
+    for (int q = c.rp[i] + lane; q < c.rp[i + 1]; q += 32) {
+        const int j = c.ci[q];
+        int lo = c.rp[j], hi = c.rp[j + 1];
+        const int end = hi;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (c.ci[mid] < i) lo = mid + 1; else hi = mid;
+        }
+        bad |= !(lo < end && c.ci[lo] == i && c.cv[lo] == c.cv[q]);
+    }
+    if (bad) *asym = 1;
+}
+
 __global__ void k_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int64_t* rows,
                            const int64_t* cols, double* out) {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
@@ -2981,6 +3001,11 @@ void launch_csr_import(const int64_t* rp, const int32_t* ci, const void* v, int 
         k_csr_import<T, float><<<nb, 256, 0, s>>>(rp, ci, static_cast<const float*>(v), p, nnz, out.rp, out.ci, out.cv);
 }
 
+template <typename T>
+void launch_csr_asymmetric(Csr<T> c, int p, int* asym, cudaStream_t s) {
+    k_csr_asymmetric<T><<<(p + 7) / 8, 256, 0, s>>>(c, p, asym);
+}
+
 void launch_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int64_t* rows,
                      const int64_t* cols, double* out, cudaStream_t s) {
     k_gather_s<<<128, 256, 0, s>>>(S, is_f64, ld, m, rows, cols, out);
@@ -3002,6 +3027,7 @@ void launch_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int
     template int screen_plan<T>(int, int, std::vector<long long>&);                                 \
     template void launch_csr_import<T>(const int64_t*, const int32_t*, const void*, int, int64_t, int64_t, Csr<T>, \
                                        cudaStream_t);                                              \
+    template void launch_csr_asymmetric<T>(Csr<T>, int, int*, cudaStream_t);                       \
     template void launch_csr_export<T>(const int*, const int*, const T*, int, int, int64_t*, int32_t*, \
                                        void*, int, cudaStream_t);
 
