@@ -1618,9 +1618,10 @@ int hpc_get_omega(hpc_handle h, int64_t* nnz_inout, int64_t* row_ptr, int32_t* c
     return HPC_OK;
 }
 
-// hpc_set_omega from device arrays: checked and converted where they are (copies to the host and
-// back, and the checks there, took about 0.3 ms at 28 672 entries).  The check runs on the legacy default stream, which
-// waits for the blocking streams that may still be writing the arrays, as the copies did.
+// hpc_set_omega from arrays that kernels of this device can read (device_readable): checked and
+// converted where they are (copies to the host and back, and the checks there, took about 0.3 ms
+// at 28 672 entries).  The check runs on the legacy default stream, which waits for the blocking
+// streams that may still be writing the arrays, as the copies did.
 static int set_omega_device(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32_t* col, const void* val,
                             hpc_dtype vdt) {
     unsigned long long* d_key = reinterpret_cast<unsigned long long*>(h->d_ctrl + 1);
@@ -1650,14 +1651,32 @@ int hpc_set_omega(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32
                   hpc_dtype vdt, int on_device) {
     if (!h || !row_ptr || !col || !val || nnz < h->p || (vdt != HPC_F32 && vdt != HPC_F64)) return HPC_ERR_ARG;
     const int64_t p = h->p;
-    if (on_device) return set_omega_device(h, nnz, row_ptr, col, val, vdt);
+    const size_t vs = dtype_size(vdt);
+    if (on_device && hpc::device_readable(row_ptr, (p + 1) * sizeof(int64_t), sizeof(int64_t)) &&
+        hpc::device_readable(col, nnz * sizeof(int32_t), sizeof(int32_t)) && hpc::device_readable(val, nnz * vs, vs))
+        return set_omega_device(h, nnz, row_ptr, col, val, vdt);
     std::vector<int64_t> rp(p + 1);
     std::vector<int32_t> ci(nnz);
     std::vector<double> v(nnz);
-    std::memcpy(rp.data(), row_ptr, (p + 1) * sizeof(int64_t));
-    std::memcpy(ci.data(), col, nnz * sizeof(int32_t));
-    if (vdt == HPC_F64) std::memcpy(v.data(), val, nnz * sizeof(double));
-    else for (int64_t t = 0; t < nnz; ++t) v[t] = static_cast<const float*>(val)[t];
+    // other device addresses come by copies, which refuse what the device does not hold
+    const auto fetch = [&](void* dst, const void* src, size_t bytes) {
+        if (on_device) {
+            const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyDeviceToHost);
+            if (e != cudaSuccess) (void)cudaGetLastError();
+            return e;
+        }
+        std::memcpy(dst, src, bytes);
+        return cudaSuccess;
+    };
+    CUDA_TRY(fetch(rp.data(), row_ptr, (p + 1) * sizeof(int64_t)));
+    CUDA_TRY(fetch(ci.data(), col, nnz * sizeof(int32_t)));
+    if (vdt == HPC_F64) {
+        CUDA_TRY(fetch(v.data(), val, nnz * sizeof(double)));
+    } else {
+        std::vector<float> f(nnz);
+        CUDA_TRY(fetch(f.data(), val, nnz * sizeof(float)));
+        for (int64_t t = 0; t < nnz; ++t) v[t] = f[t];
+    }
     // validate: row_ptr monotone, columns sorted and in range, positive diagonal present
     if (rp[0] != 0 || rp[p] != nnz) return HPC_ERR_ARG;
     for (int64_t i = 0; i < p; ++i) {

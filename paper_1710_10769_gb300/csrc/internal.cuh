@@ -382,6 +382,10 @@ size_t gram_tc_scratch_bytes(int xdt, int64_t n, int64_t p, int precision);
 // code of the bounded wait that gave up); synchronises s.
 int gram_tc_take_error(const void* scratch, int xdt, int64_t n, int64_t p, int precision, cudaStream_t s);
 
+// Whether kernels on the current device can read bytes at q, aligned to `align`: device or managed
+// memory whose allocation holds all of them.
+bool device_readable(const void* q, size_t bytes, size_t align);
+
 // Raise a kernel's dynamic shared-memory limit once per device (the attribute call
 // is a host round trip that must stay out of the iteration loop).
 cudaError_t set_smem_once(const void* func, int bytes, int slot);

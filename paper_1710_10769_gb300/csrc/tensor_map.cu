@@ -55,6 +55,29 @@ bool encode_tensor_map_2d_sw128(CUtensorMap* map, const void* base, int elem_byt
                   CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
+bool device_readable(const void* q, size_t bytes, size_t align) {
+    using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Range range = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult st = cudaDriverEntryPointSymbolNotFound;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &st);
+        if (e != cudaSuccess) (void)cudaGetLastError();
+        return e == cudaSuccess && st == cudaDriverEntryPointSuccess ? reinterpret_cast<Range>(fn) : nullptr;
+    }();
+    int dev = 0;
+    cudaPointerAttributes a{};
+    if (reinterpret_cast<uintptr_t>(q) % align != 0 || !range) return false;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, q) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    if (!(a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev))) return false;
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(q);
+    return range(&base, &size, at) == CUDA_SUCCESS && at >= base && at - base <= size && bytes <= size - (at - base);
+}
+
 cudaError_t set_smem_once(const void* func, int bytes, int slot) {
     static std::mutex mu;
     static bool done[64][kSmemSlots] = {};
