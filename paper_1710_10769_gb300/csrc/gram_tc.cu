@@ -806,14 +806,9 @@ cudaError_t launch_mirror(float* S, int64_t lds, int64_t p, uint16_t* m1, int nb
     const int nb = (int)((p + kMirT - 1) / kMirT);
     const long long pairs = (long long)nb * (nb + 1) / 2;
     if (pairs > 0x7fffffffll) return cudaErrorNotSupported;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_mirror_max<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMirSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_mirror_max<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMirSmem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    const cudaError_t e = m1 ? set_smem_once((const void*)k_mirror_max<true>, kMirSmem, kSmemSlotMirrorMax)
+                             : set_smem_once((const void*)k_mirror_max<false>, kMirSmem, kSmemSlotMirror);
+    if (e != cudaSuccess) return e;
     // the interior blocks' float4 rows need 16-byte aligned rows: S aligned and lds a multiple of 4
     const int vec = (lds % 4 == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0) ? 1 : 0;
     if (m1) k_mirror_max<true><<<(unsigned)pairs, 256, kMirSmem, s>>>(S, lds, (int)p, nb, m1, nbm, vec);

@@ -389,7 +389,10 @@ bool device_readable(const void* q, size_t bytes, size_t align);
 // Raise a kernel's dynamic shared-memory limit once per device (the attribute call
 // is a host round trip that must stay out of the iteration loop).
 cudaError_t set_smem_once(const void* func, int bytes, int slot);
-enum : int { kSmemSlotScreenF = 0, kSmemSlotScreenD = 1, kSmemSlotObsBf16x3 = 2, kSmemSlotObsTf32 = 3, kSmemSlots = 4 };
+enum : int {
+    kSmemSlotScreenF = 0, kSmemSlotScreenD, kSmemSlotObsBf16x3, kSmemSlotObsTf32, kSmemSlotLoopF, kSmemSlotLoopD,
+    kSmemSlotMirror, kSmemSlotMirrorMax, kSmemSlots
+};
 
 // Set the text returned by hpc_last_error() for this thread (api.cu).
 void set_last_error(const char* msg);

@@ -1711,12 +1711,9 @@ int loop_grid(int p, int nbm, int num_sms, int* rows) {
         loop_smem_bytes<T>(R) > 220 * 1024)
         return 0;
     int v = 0;
-    static bool attr = false;
-    if (!attr) {
-        if (cudaFuncSetAttribute(k_loop<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess)
-            return 0;
-        attr = true;
-    }
+    if (set_smem_once((const void*)k_loop<T>, 220 * 1024, sizeof(T) == 4 ? kSmemSlotLoopF : kSmemSlotLoopD) !=
+        cudaSuccess)
+        return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_loop<T>, kLT, loop_smem_bytes<T>(R)) != cudaSuccess ||
         v < 1)
         return 0;
