@@ -2194,8 +2194,7 @@ int hypergrad_t(hpc_ctx* h, const void* Xval, int xdt, int64_t nval, double cg_t
     *dl2 = -st.dot_omega;
     if (info) {
         std::memset(info, 0, sizeof *info);
-        // counted in steps of eight, up to the cap
-        info->cg_iterations = std::min<int64_t>(cg_max, std::max<int64_t>(8, (st.iterations + 7) / 8 * 8));
+        info->cg_iterations = st.iterations;
         info->rel_residual = st.rr0 > 0.0 ? std::sqrt(st.rr / st.rr0) : 0.0;
         info->support = nnz;
         info->converged = st.done == 1 ? 1 : 0;
