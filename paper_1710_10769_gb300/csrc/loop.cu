@@ -121,21 +121,10 @@ __device__ __forceinline__ void st_ent(Ent<double>* q, unsigned cf, double om, d
     reinterpret_cast<double2*>(q)[1] = make_double2(g, w);
 }
 
-// Partials as stored between blocks: a compensated pair or a double.
-__device__ __forceinline__ F2 ld_part(const F2* q) {
-    const float2 v = __ldcg(reinterpret_cast<const float2*>(q));
-    F2 a;
-    a.hi = v.x;
-    a.lo = v.y;
-    return a;
-}
-__device__ __forceinline__ double ld_part(const double* q) { return __ldcg(q); }
-
 enum : int { kCtrTask = 0, kCtrHeavy = 2, kCtrPage = 4, kCtrBig = 5, kCtrFull = 6, kCtrCount = 8 };
 
 template <typename T>
 struct LoopK {
-    using A = typename AccOf<T>::type;
     const T* S;
     int64_t ld;
     int p, R;
@@ -160,7 +149,7 @@ struct LoopK {
     int nbp;
     unsigned* mg;        // bits of max |S_ij|, i != j (rounded up)
     int* ctr;            // counters: tasks (2), tasks of long rows (2), pages, entries of big, pool full
-    A* part_a;           // 2 x kNA x grid
+    double* part_a;      // 2 x kNA x grid
     int* part_i;         // 2 x kNI x grid
     unsigned* bar;
     Ctrl* ctrl;
@@ -177,7 +166,6 @@ struct LoopK {
 // Shared memory of a block, laid out by the host's sizes.
 template <typename T>
 struct LoopSmem {
-    using A = typename AccOf<T>::type;
     unsigned key[kLW][kSlots];          // a row's slots by column
     unsigned heavy[2][kLW];             // a quarter block's largest |W_ij|, per warp
     int hit_i[kLW][kHitCap];            // entries (i, j) waiting for W_ji
@@ -185,7 +173,7 @@ struct LoopSmem {
     T hit_w[kLW][kHitCap];
     T del[kLW][kWin][32];
     unsigned jf[kLW][32];
-    A red_a[kLW][kNA];
+    double red_a[kLW][kNA];
     int red_i[kLW][kNI];
     double sum_a[kNA];
     int sum_i[kNI], pre_i[kNI];
@@ -209,6 +197,19 @@ __device__ __forceinline__ F2 shfl_xor_acc(const F2& x, int o) {
     r.hi = __shfl_xor_sync(kFull, x.hi, o);
     r.lo = __shfl_xor_sync(kFull, x.lo, o);
     return r;
+}
+
+// Quantity t summed over the block's warps, a fixed tree: FP64 from here on, as the chain's sums
+// (a thread's and a warp's sums are compensated FP32 pairs).
+__device__ __forceinline__ double warps_sum(const double (*red)[kNA], int t) {
+    double a[kLW];
+#pragma unroll
+    for (int w = 0; w < kLW; ++w) a[w] = red[w][t];
+#pragma unroll
+    for (int n = kLW / 2; n >= 1; n >>= 1)
+#pragma unroll
+        for (int w = 0; w < n; ++w) a[w] += a[w + n];
+    return a[0];
 }
 
 // Grid-wide barrier on a counter that only grows: one release add per block, then
@@ -1256,12 +1257,12 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
                     acc_merge(v[0], shfl_xor_acc(v[0], 1));
                     const int qi = lane >> 1;
                     if (!(lane & 1)) {
-                        if (qi < kQA) sm.red_a[warp][wn * kQA + qi] = v[0];
-                        else if (qi == kQA && first && wn == 0) sm.red_a[warp][2 * kQA] = v[0];
+                        if (qi < kQA) sm.red_a[warp][wn * kQA + qi] = acc_value(v[0]);
+                        else if (qi == kQA && first && wn == 0) sm.red_a[warp][2 * kQA] = acc_value(v[0]);
                     }
                 } else {
-                    if (lane < kQA) sm.red_a[warp][wn * kQA + lane] = A{};
-                    if (lane == kQA && first && wn == 0) sm.red_a[warp][2 * kQA] = A{};
+                    if (lane < kQA) sm.red_a[warp][wn * kQA + lane] = 0.0;
+                    if (lane == kQA && first && wn == 0) sm.red_a[warp][2 * kQA] = 0.0;
                 }
 #pragma unroll
                 for (int m = 0; m < kWin; ++m) {
@@ -1286,9 +1287,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
             for (int t = tid; t < kNA + kNI; t += kLT) {
                 if (t < kNA) {
                     if (t < na || (first && t == 2 * kQA)) {
-                        A a = sm.red_a[0][t];
-                        for (int w = 1; w < kLW; ++w) acc_merge(a, sm.red_a[w][t]);
-                        k.part_a[((size_t)pbuf * kNA + t) * nb + bid] = a;
+                        k.part_a[((size_t)pbuf * kNA + t) * nb + bid] = warps_sum(sm.red_a, t);
                     }
                 } else {
                     const int u = t - kNA;
@@ -1306,13 +1305,13 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
             static_assert((kNA + kNI) * 8 <= kLT, "one pass over the quantities");
             {
                 const int t = tid >> 3, sub = tid & 7;
-                A a{};
+                double a = 0.0;
                 int c = 0, pre = 0;
                 if (t < kNA) {
                     if (t < na || (first && t == 2 * kQA)) {
-                        const A* src = k.part_a + ((size_t)pbuf * kNA + t) * nb;
+                        const double* src = k.part_a + ((size_t)pbuf * kNA + t) * nb;
 #pragma unroll 8
-                        for (int b = sub; b < nb; b += 8) acc_merge(a, ld_part(src + b));
+                        for (int b = sub; b < nb; b += 8) a += __ldcg(src + b);
                     }
                 } else if (t < kNA + kNI) {
                     const int u = t - kNA;
@@ -1328,12 +1327,12 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
                 }
 #pragma unroll
                 for (int o = 4; o > 0; o >>= 1) {
-                    acc_merge(a, shfl_xor_acc(a, o));
+                    a += __shfl_xor_sync(kFull, a, o);
                     c += __shfl_xor_sync(kFull, c, o);
                     pre += __shfl_xor_sync(kFull, pre, o);
                 }
                 // quantities that this window did not write keep their earlier sums
-                if (sub == 0 && t < kNA && (t < na || (first && t == 2 * kQA))) sm.sum_a[t] = acc_value(a);
+                if (sub == 0 && t < kNA && (t < na || (first && t == 2 * kQA))) sm.sum_a[t] = a;
                 if (sub == 0 && t >= kNA && t < kNA + kNI && (t - kNA < nii || (first && t - kNA >= 2 * kQI))) {
                     sm.sum_i[t - kNA] = c;
                     sm.pre_i[t - kNA] = pre;
@@ -1575,28 +1574,28 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
             }
         }
         const A a = warp_sum(ow), b = warp_sum(lg), c = warp_sum(ab);
-        if (lane == 0) { sm.red_a[warp][0] = a; sm.red_a[warp][1] = b; sm.red_a[warp][2] = c; }
-        __syncthreads();
-        if (tid < 3) {
-            A x = sm.red_a[0][tid];
-            for (int w = 1; w < kLW; ++w) acc_merge(x, sm.red_a[w][tid]);
-            k.part_a[((size_t)pbuf * kNA + tid) * nb + bid] = x;
+        if (lane == 0) {
+            sm.red_a[warp][0] = acc_value(a);
+            sm.red_a[warp][1] = acc_value(b);
+            sm.red_a[warp][2] = acc_value(c);
         }
+        __syncthreads();
+        if (tid < 3) k.part_a[((size_t)pbuf * kNA + tid) * nb + bid] = warps_sum(sm.red_a, tid);
         if (!loop_barrier(k.bar, target, ctrl, &sm.ok)) {
             if (bid == 0 && tid == 0) end_loops(k);
             return;
         }
         if (bid == 0 && warp < 3) {
-            A x{};
-            for (int t = lane; t < nb; t += 32) acc_merge(x, ld_part(k.part_a + ((size_t)pbuf * kNA + warp) * nb + t));
+            double x = 0.0;
+            for (int t = lane; t < nb; t += 32) x += __ldcg(k.part_a + ((size_t)pbuf * kNA + warp) * nb + t);
             x = warp_sum(x);
             if (lane == 0) sm.red_a[0][kQA + warp] = x;
         }
         __syncthreads();
         if (bid == 0 && tid == 0) {
             const double norm2 = sm.sum_a[2 * kQA];
-            ctrl->f_cur = -acc_value(sm.red_a[0][kQA + 1]) + 0.5 * acc_value(sm.red_a[0][kQA]) + 0.5 * lam2d * norm2;
-            ctrl->pen_cur = ctrl->lam1 * acc_value(sm.red_a[0][kQA + 2]);
+            ctrl->f_cur = -sm.red_a[0][kQA + 1] + 0.5 * sm.red_a[0][kQA] + 0.5 * lam2d * norm2;
+            ctrl->pen_cur = ctrl->lam1 * sm.red_a[0][kQA + 2];
             ctrl->norm2_cur = norm2;
         }
     }
@@ -1651,7 +1650,6 @@ size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 template <typename T>
 LoopK<T> loop_args(const IterBufs<T>& b, void* ws, int R, size_t* bytes) {
-    using A = typename AccOf<T>::type;
     LoopK<T> k{};
     k.S = b.S;
     k.ld = b.ld;
@@ -1691,7 +1689,7 @@ LoopK<T> loop_args(const IterBufs<T>& b, void* ws, int R, size_t* bytes) {
     if (!b.m1) k.bnd = nullptr;
     k.slack = reinterpret_cast<float*>(take(p * sizeof(float)));
     k.mg = reinterpret_cast<unsigned*>(take(sizeof(unsigned)));
-    k.part_a = reinterpret_cast<A*>(take(2 * (size_t)kNA * b.num_sms * sizeof(A)));
+    k.part_a = reinterpret_cast<double*>(take(2 * (size_t)kNA * b.num_sms * sizeof(double)));
     k.part_i = reinterpret_cast<int*>(take(2 * (size_t)kNI * b.num_sms * sizeof(int)));
     k.ctr = reinterpret_cast<int*>(take(kCtrCount * sizeof(int)));
     if (bytes) *bytes = (size_t)(q - static_cast<uint8_t*>(ws));
