@@ -282,27 +282,6 @@ int set_identity(hpc_ctx* h) {
     return HPC_OK;
 }
 
-// Whether the iterate that hpc_set_omega left in the current buffers is symmetric; waits for it.
-int check_symmetric(hpc_ctx* h) {
-    if (h->variant != HPC_COV) {
-        CUDA_TRY(cudaStreamSynchronize(h->stream));
-        return HPC_OK;
-    }
-    int* d = reinterpret_cast<int*>(h->d_ctrl + 1);
-    int asym = 0;
-    CUDA_TRY(cudaMemsetAsync(d, 0, sizeof(int), h->stream));
-    const int c = h->cur;
-    if (h->vdt == HPC_F64)
-        hpc::launch_csr_asymmetric<double>({h->rp[c], h->ci[c], static_cast<double*>(h->cv[c])}, (int)h->p, d, h->stream);
-    else
-        hpc::launch_csr_asymmetric<float>({h->rp[c], h->ci[c], static_cast<float*>(h->cv[c])}, (int)h->p, d, h->stream);
-    CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaMemcpyAsync(&asym, d, sizeof asym, cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
-    set_symmetric(h, asym == 0);
-    return HPC_OK;
-}
-
 template <typename T>
 hpc::IterBufs<T> bufs(hpc_ctx* h) {
     hpc::IterBufs<T> b{};
@@ -1504,7 +1483,7 @@ int hpc_create(hpc_handle* out, const void* X, hpc_dtype xdt, int64_t n, int64_t
     h->nblk = (int)std::min<int64_t>((p + 7) / 8, 152 * 16);
     CK(hold(h, &h->part_obj, (size_t)h->nblk * 4 * sizeof(double)));
     CK(hold(h, &h->part_ls, (size_t)h->nblk * 16 * 4 * sizeof(double)));
-    CK(hold(h, &h->d_ctrl, sizeof(hpc::Ctrl) + sizeof(unsigned long long)));      // and a word of hpc_set_omega's checks
+    CK(hold(h, &h->d_ctrl, sizeof(hpc::Ctrl) + sizeof(hpc::CsrChecks)));      // and hpc_set_omega's checks
     CK(cudaMemsetAsync(h->d_ctrl, 0, sizeof(hpc::Ctrl), h->stream));
     CK(hold(h, &h->bar, hpc::kBarWords * sizeof(unsigned)));
     CK(cudaMemsetAsync(h->bar, 0, hpc::kBarWords * sizeof(unsigned), h->stream));
@@ -1624,14 +1603,14 @@ int hpc_get_omega(hpc_handle h, int64_t* nnz_inout, int64_t* row_ptr, int32_t* c
 // streams that may still be writing the arrays, as the copies did.
 static int set_omega_device(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32_t* col, const void* val,
                             hpc_dtype vdt) {
-    unsigned long long* d_key = reinterpret_cast<unsigned long long*>(h->d_ctrl + 1);
-    unsigned long long key = ~0ull;
-    CUDA_TRY(cudaMemsetAsync(d_key, 0xff, sizeof key, cudaStreamLegacy));
-    hpc::launch_csr_check(row_ptr, col, val, vdt, h->p, nnz, d_key, cudaStreamLegacy);
+    hpc::CsrChecks* d_chk = reinterpret_cast<hpc::CsrChecks*>(h->d_ctrl + 1);
+    hpc::CsrChecks chk;
+    CUDA_TRY(cudaMemsetAsync(d_chk, 0xff, sizeof chk, cudaStreamLegacy));
+    hpc::launch_csr_check(row_ptr, col, val, vdt, h->vdt, h->p, nnz, d_chk, cudaStreamLegacy);
     CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaMemcpy(&key, d_key, sizeof key, cudaMemcpyDeviceToHost));
-    if (key != ~0ull) {
-        const unsigned fault = (unsigned)key & 3u;
+    CUDA_TRY(cudaMemcpy(&chk, d_chk, sizeof chk, cudaMemcpyDeviceToHost));
+    if (chk.key != ~0ull) {
+        const unsigned fault = (unsigned)chk.key & 3u;
         return fault == hpc::kCsrBadArg ? HPC_ERR_ARG : fault == hpc::kCsrBadDiag ? HPC_ERR_NONPOS_DIAG : HPC_ERR_NAN;
     }
     if (nnz > h->csr_cap) STATUS_TRY(grow_csr(h, 2 * nnz));
@@ -1643,8 +1622,10 @@ static int set_omega_device(hpc_handle h, int64_t nnz, const int64_t* row_ptr, c
         hpc::launch_csr_import<float>(row_ptr, col, val, vdt, h->p, nnz,
                                       {h->rp[c], h->ci[c], static_cast<float*>(h->cv[c])}, h->stream);
     CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
     h->nnz = nnz;
-    return check_symmetric(h);
+    set_symmetric(h, chk.symmetric != 0);
+    return HPC_OK;
 }
 
 int hpc_set_omega(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32_t* col, const void* val,
@@ -1709,7 +1690,16 @@ int hpc_set_omega(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32
         CUDA_TRY(cudaStreamSynchronize(h->stream));
     }
     h->nnz = nnz;
-    return check_symmetric(h);
+    // the same comparison that device arrays get
+    hpc::CsrChecks* d_chk = reinterpret_cast<hpc::CsrChecks*>(h->d_ctrl + 1);
+    hpc::CsrChecks chk;
+    CUDA_TRY(cudaMemsetAsync(d_chk, 0xff, sizeof chk, h->stream));
+    hpc::launch_csr_symmetric(h->rp[c], h->ci[c], h->cv[c], h->vdt, p, nnz, d_chk, h->stream);
+    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaMemcpyAsync(&chk, d_chk, sizeof chk, cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    set_symmetric(h, chk.symmetric != 0);
+    return HPC_OK;
 }
 
 }  // extern "C"

@@ -200,13 +200,21 @@ template <typename T> void launch_csr_export(const int* rp, const int* ci, const
                                              int64_t* rp64, int32_t* ci_out, void* val, int vdt,
                                              cudaStream_t s);
 enum : unsigned { kCsrBadArg = 1, kCsrBadDiag = 2, kCsrNotFinite = 3 };
-void launch_csr_check(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int64_t p, int64_t nnz,
-                      unsigned long long* key, cudaStream_t s);
+// Their outcome; all bits are set before a launch.
+struct CsrChecks {
+    unsigned long long key;         // the first fault in row order
+    unsigned long long symmetric;   // 0: some entry (i, j) has no equal entry (j, i)
+};
+static_assert(sizeof(Ctrl) % 8 == 0, "CsrChecks lies behind the control block");
+// The faults, and the symmetry of the entries as values of type out_dt.
+void launch_csr_check(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int out_dt, int64_t p, int64_t nnz,
+                      CsrChecks* out, cudaStream_t s);
+// The symmetry alone, of a handle's arrays.
+void launch_csr_symmetric(const int* rp, const int* ci, const void* v, int vdt, int64_t p, int64_t nnz, CsrChecks* out,
+                          cudaStream_t s);
 template <typename T>
 void launch_csr_import(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int64_t p, int64_t nnz, Csr<T> out,
                        cudaStream_t s);
-// *asym = 1 if some entry (i, j) has no equal entry (j, i).
-template <typename T> void launch_csr_asymmetric(Csr<T> c, int p, int* asym, cudaStream_t s);
 void launch_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int64_t* rows,
                      const int64_t* cols, double* out, cudaStream_t s);
 

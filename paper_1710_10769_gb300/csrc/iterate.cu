@@ -2349,6 +2349,33 @@ __global__ void __launch_bounds__(256) k_csr_check(const int64_t* __restrict__ r
     if (fault) atomicMin(key, (unsigned long long)i << 32 | (unsigned long long)(place << 2 | fault));
 }
 
+// Whether every entry (i, j) has an equal entry (j, i), as values of type T: a warp per row, the
+// transpose by binary search in its column's row.  rp and ci may still hold faults: nothing
+// outside of 0 .. nnz is read, columns outside of 0 .. p - 1 are left out.
+template <typename T, typename I, typename V>
+__global__ void __launch_bounds__(256) k_csr_symmetric(const I* __restrict__ rp, const int32_t* __restrict__ ci,
+                                                       const V* __restrict__ v, int64_t p, int64_t nnz,
+                                                       unsigned long long* symmetric) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = blockIdx.x * 8ll + (threadIdx.x >> 5);
+    if (i >= p) return;
+    const int64_t a = max((int64_t)0, (int64_t)rp[i]), b = min(nnz, (int64_t)rp[i + 1]);
+    if (b - a > p) return;                  // a fault: k_csr_check's finding
+    bool bad = false;
+    for (int64_t q = a + lane; q < b; q += 32) {
+        const int64_t j = ci[q];
+        if (j < 0 || j >= p) continue;
+        int64_t lo = max((int64_t)0, (int64_t)rp[j]), hi = min(nnz, (int64_t)rp[j + 1]);
+        const int64_t end = hi;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (ci[mid] < i) lo = mid + 1; else hi = mid;
+        }
+        bad |= !(lo < end && ci[lo] == i && (T)v[lo] == (T)v[q]);
+    }
+    if (bad) *symmetric = 0;
+}
+
 template <typename T, typename V>
 __global__ void __launch_bounds__(256) k_csr_import(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                                     const V* __restrict__ v, int64_t p, int64_t nnz, int* __restrict__ rpo,
@@ -2360,26 +2387,6 @@ __global__ void __launch_bounds__(256) k_csr_import(const int64_t* __restrict__ 
             vo[t] = (T)v[t];
         }
     }
-}
-
-// One warp per row: each entry's transpose by binary search in its column's row.
-template <typename T>
-__global__ void __launch_bounds__(256) k_csr_asymmetric(Csr<T> c, int p, int* asym) {
-    const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (i >= p) return;
-    bool bad = false;
-    for (int q = c.rp[i] + lane; q < c.rp[i + 1]; q += 32) {
-        const int j = c.ci[q];
-        int lo = c.rp[j], hi = c.rp[j + 1];
-        const int end = hi;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (c.ci[mid] < i) lo = mid + 1; else hi = mid;
-        }
-        bad |= !(lo < end && c.ci[lo] == i && c.cv[lo] == c.cv[q]);
-    }
-    if (bad) *asym = 1;
 }
 
 __global__ void k_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int64_t* rows,
@@ -2984,11 +2991,28 @@ void launch_csr_export(const int* rp, const int* ci, const T* cv, int p, int nnz
         k_csr_export<T, float><<<256, 256, 0, s>>>(rp, ci, cv, p, nnz, rp64, co, static_cast<float*>(val));
 }
 
-void launch_csr_check(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int64_t p, int64_t nnz,
-                      unsigned long long* key, cudaStream_t s) {
-    const unsigned nb = (unsigned)((p + 255) / 256);
-    if (vdt == HPC_F64) k_csr_check<double><<<nb, 256, 0, s>>>(rp, ci, static_cast<const double*>(v), p, nnz, key);
-    else k_csr_check<float><<<nb, 256, 0, s>>>(rp, ci, static_cast<const float*>(v), p, nnz, key);
+template <typename V>
+static void csr_check(const int64_t* rp, const int32_t* ci, const V* v, int out_dt, int64_t p, int64_t nnz,
+                      CsrChecks* out, cudaStream_t s) {
+    k_csr_check<V><<<(unsigned)((p + 255) / 256), 256, 0, s>>>(rp, ci, v, p, nnz, &out->key);
+    const unsigned nb = (unsigned)((p + 7) / 8);
+    if (out_dt == HPC_F64) k_csr_symmetric<double><<<nb, 256, 0, s>>>(rp, ci, v, p, nnz, &out->symmetric);
+    else k_csr_symmetric<float><<<nb, 256, 0, s>>>(rp, ci, v, p, nnz, &out->symmetric);
+}
+
+void launch_csr_check(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int out_dt, int64_t p, int64_t nnz,
+                      CsrChecks* out, cudaStream_t s) {
+    if (vdt == HPC_F64) csr_check(rp, ci, static_cast<const double*>(v), out_dt, p, nnz, out, s);
+    else csr_check(rp, ci, static_cast<const float*>(v), out_dt, p, nnz, out, s);
+}
+
+void launch_csr_symmetric(const int* rp, const int* ci, const void* v, int vdt, int64_t p, int64_t nnz, CsrChecks* out,
+                          cudaStream_t s) {
+    const unsigned nb = (unsigned)((p + 7) / 8);
+    if (vdt == HPC_F64)
+        k_csr_symmetric<double><<<nb, 256, 0, s>>>(rp, ci, static_cast<const double*>(v), p, nnz, &out->symmetric);
+    else
+        k_csr_symmetric<float><<<nb, 256, 0, s>>>(rp, ci, static_cast<const float*>(v), p, nnz, &out->symmetric);
 }
 
 template <typename T>
@@ -2999,11 +3023,6 @@ void launch_csr_import(const int64_t* rp, const int32_t* ci, const void* v, int 
         k_csr_import<T, double><<<nb, 256, 0, s>>>(rp, ci, static_cast<const double*>(v), p, nnz, out.rp, out.ci, out.cv);
     else
         k_csr_import<T, float><<<nb, 256, 0, s>>>(rp, ci, static_cast<const float*>(v), p, nnz, out.rp, out.ci, out.cv);
-}
-
-template <typename T>
-void launch_csr_asymmetric(Csr<T> c, int p, int* asym, cudaStream_t s) {
-    k_csr_asymmetric<T><<<(p + 7) / 8, 256, 0, s>>>(c, p, asym);
 }
 
 void launch_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int64_t* rows,
@@ -3027,7 +3046,6 @@ void launch_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int
     template int screen_plan<T>(int, int, std::vector<long long>&);                                 \
     template void launch_csr_import<T>(const int64_t*, const int32_t*, const void*, int, int64_t, int64_t, Csr<T>, \
                                        cudaStream_t);                                              \
-    template void launch_csr_asymmetric<T>(Csr<T>, int, int*, cudaStream_t);                       \
     template void launch_csr_export<T>(const int*, const int*, const T*, int, int, int64_t*, int32_t*, \
                                        void*, int, cudaStream_t);
 
