@@ -472,8 +472,9 @@ typedef struct {
                                   separate kernels, or, for the Cov variant from 384
                                   rows (FP64: 224) on, all iterations in one kernel
                                   (three barriers per iteration; the chain then runs
-                                  only the iterations in which a row has more than
-                                  2046 candidates).  The same entries and decisions
+                                  the iterations that it does faster: dense ones,
+                                  hub rows, screen_bounds 0 at large p).  Symmetric
+                                  iterates only.  The same entries and decisions
                                   every way (the line search's sums are grouped
                                   differently, which moves F in its last bits and a
                                   decision only at an exact tie).  Where only the tail

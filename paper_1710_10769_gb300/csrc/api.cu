@@ -555,6 +555,7 @@ int load_ctrl(hpc_ctx* h, int64_t k, bool use_stop) {
     c.loop_full = 0;
     c.loop_fulls = 0;
     c.chain_left = 0;
+    c.loop_debt = 0;
     c.flags = 0;
     c.converged = 0;
     c.lam1 = h->lam1;

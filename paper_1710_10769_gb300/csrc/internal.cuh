@@ -54,9 +54,10 @@ struct Ctrl {
     int n_pairs, n_row_items;     // items the bound screening keeps (pure rows; rows with neighbours)
     long long loop_attempts;      // of iter_attempts: iterations of the one-launch loop (loop.cu)
     long long loop_launches;      // its launches
-    int loop_full;                // the loop met a row with more candidates than its buckets hold
+    int loop_full;                // the loop left the next iterations to the chain
     int loop_fulls;               // how often since the last reset
     int chain_left, pad5_;        // iterations the chain runs before the loop tries again
+    unsigned loop_debt, pad6_;    // what its passes so far took beyond the chain's time (loop.cu, in_debt)
 };
 
 // Rows with at most this many candidate entries (before de-dup) are handled one

@@ -2909,6 +2909,7 @@ __global__ void k_point_begin(Ctrl* ctrl, PathOut out, cudaGraphConditionalHandl
         ctrl->ls_trials = 0;
         ctrl->converged = 0;
         ctrl->loop_fulls = 0;
+        ctrl->loop_debt = 0;
         ctrl->t_point = globaltimer_ns();
     }
     ctrl->path_keep = 0;

@@ -52,10 +52,11 @@
 // (The bounds without this memory keep nearly every block once lambda1 is near the noise
 // of S: at p = 8192, lambda1 = 0.05 a pass then reads 1.7 GB of S.)
 //
-// A row that collects more than kMaxE - 2 candidates, or more pages than the pool has,
-// ends the launch with Ctrl::loop_full set and the iterate unchanged; the chain of
-// kernels then runs the next iterations (one at first, twice as many after every further
-// full bucket) before the loop tries again.
+// A row that collects more than kMaxE - 2 candidates, or more pages than the pool has, or a pass
+// that the chain does faster (dense iterates and hub rows, see in_debt) ends the launch with
+// Ctrl::loop_full set and the iterate unchanged; the chain of kernels then runs the next
+// iterations (one at first, twice as many after every further end of this kind) before the loop
+// tries again.  No phase of a launch is long, then, which the bounded waits need.
 //
 // Measured on GB300 (us per iteration, the chain of kernels -> this loop): 140 -> 46 at
 // p = 65536 (n = 32768), 120 -> 43 at p = 16384, 98 -> 30 at p = 1001, 220 -> 50 in FP64 at
@@ -82,6 +83,7 @@ constexpr int kWin = 4;                  // step sizes per line-search window
 constexpr int kItemCap = 4096;           // owned support entries kept in shared memory
 constexpr int kHitCap = 64;              // entries waiting for their W_ji, per warp
 constexpr int kMaxR = 2048;              // rows per block
+constexpr int kHeavyTerms = 32;          // rows with more terms are screened by four warps a block
 constexpr int kQA = 3 * kWin;            // accumulated partials per window: quadratic form, ||D||^2, phi
 constexpr int kQI = 2 * kWin;            // counted partials per window: w+_ii <= 0, entries kept
 constexpr int kNA = 2 * kQA + 1;         // and ||Omega||^2
@@ -121,7 +123,8 @@ __device__ __forceinline__ void st_ent(Ent<double>* q, unsigned cf, double om, d
     reinterpret_cast<double2*>(q)[1] = make_double2(g, w);
 }
 
-enum : int { kCtrTask = 0, kCtrHeavy = 2, kCtrPage = 4, kCtrBig = 5, kCtrFull = 6, kCtrCount = 8 };
+enum : int { kFullPool = 1, kFullDense = 2 };      // bits of kCtrFull
+enum : int { kCtrPage, kCtrBig, kCtrFull, kCtrCount = 4 };
 
 template <typename T>
 struct LoopK {
@@ -148,7 +151,9 @@ struct LoopK {
     float* slack;        // p: the rounding term of the row
     int nbp;
     unsigned* mg;        // bits of max |S_ij|, i != j (rounded up)
-    int* ctr;            // counters: tasks (2), tasks of long rows (2), pages, entries of big, pool full
+    ulonglong2* todo;    // 2: tasks in the list, and of long rows: their number, and from bit 32 on their
+                         // terms in units of 64
+    int* ctr;            // counters: pages, entries of big, full rows
     double* part_a;      // 2 x kNA x grid
     int* part_i;         // 2 x kNI x grid
     unsigned* bar;
@@ -181,6 +186,10 @@ struct LoopSmem {
     short item_r[kItemCap];             // their rows
     int ni, npl, nlong, nhuge, ok, e0, e1, pool_full;
     int wsum[kLW], wbig[kLW];
+    int sup;                            // sum of n_i^2 / 64 over the owned rows of n_i entries
+    unsigned debt, sup_debt;            // in_debt's; one thread's
+    int leave[2];                       // outcomes of leave_support and leave_tasks
+    int units;                          // pairs of 32-entry chunks of the rows with more than 32 candidates
     // the decision, the same in every block
     int flags, accept, nnz, nnz_pre, more, converged, full;
     double n2;
@@ -283,7 +292,7 @@ __device__ __forceinline__ void put_slot(const LoopK<T>& k, int row, unsigned cf
     int id = __ldcg(pt);
     if (id == 0) {
         const int n = 1 + atomicAdd(k.ctr + kCtrPage, 1);
-        if (n > k.npool) { k.ctr[kCtrFull] = 1; return; }
+        if (n > k.npool) { atomicOr(k.ctr + kCtrFull, kFullPool); return; }
         const int old = atomicCAS(pt, 0, n);
         id = old ? old : n;
     }
@@ -647,16 +656,19 @@ __device__ __forceinline__ void screen_support(const LoopK<T>& k, const Csr<T>& 
 }
 
 // The warp's blocks 8 oc .. 8 oc + 7 of row i with their bit in `bits` onto the task list
-// (heavy: from the back of it).
+// (heavy: from the back of it); terms: the row's.
 template <typename T>
-__device__ __forceinline__ void push_tasks(const LoopK<T>& k, int par, bool heavy, int i, int oc, unsigned bits,
-                                           int lane) {
+__device__ __forceinline__ void push_tasks(const LoopK<T>& k, int par, bool heavy, int terms, int i, int oc,
+                                           unsigned bits, int lane) {
     const int c = __popc(bits);
     const int incl = warp_incl_scan(c, lane);
     const int total = __shfl_sync(kFull, incl, 31);
     if (!total) return;
     int base = 0;
-    if (lane == 0) base = atomicAdd(k.ctr + (heavy ? kCtrHeavy : kCtrTask) + par, total);
+    if (lane == 0) {
+        const unsigned long long work = ((unsigned long long)total * terms + 32) >> 6;
+        base = (int)atomicAdd(heavy ? &k.todo[par].y : &k.todo[par].x, work << 32 | (unsigned)total);
+    }
     int pos = __shfl_sync(kFull, base, 0) + incl - c;
     while (bits) {
         const int v = __ffs(bits) - 1;
@@ -691,15 +703,16 @@ __device__ __forceinline__ void pure_row_tasks(const LoopK<T>& k, int i, T d, T 
                         bits |= 1u << v;
             }
         }
-        push_tasks(k, par, false, i, oc, bits, lane);
+        push_tasks(k, par, false, 1, i, oc, bits, lane);
     }
 }
 
 // The certified bounds of row i after a change of its weights, and the tasks they leave
 // (one warp).  term(e): column, |change| rounded up, and whether the column left the
-// support, for e < n; init: the bounds start here.  slack: the row's rounding term.
+// support, for e < n; init: the bounds start here.  terms, slack: the row's length, its rounding
+// term.
 template <typename T, typename F>
-__device__ __forceinline__ void bound_row(const LoopK<T>& k, int i, int n, bool init, bool heavy, float slack, T lam1,
+__device__ __forceinline__ void bound_row(const LoopK<T>& k, int i, int n, bool init, int terms, float slack, T lam1,
                                           int par, int lane, F&& term) {
     constexpr int V = 16 / (int)sizeof(T), BJ = 32 * V;
     const bool vec = (k.nbm & 7) == 0;
@@ -786,7 +799,7 @@ __device__ __forceinline__ void bound_row(const LoopK<T>& k, int i, int n, bool 
             m[0] = make_float4(B[0], B[1], B[2], B[3]);
             m[1] = make_float4(B[4], B[5], B[6], B[7]);
         }
-        push_tasks(k, par, heavy, i, oc, bits, lane);
+        push_tasks(k, par, terms > kHeavyTerms, terms, i, oc, bits, lane);
     }
 }
 
@@ -803,6 +816,61 @@ __device__ __forceinline__ float warp_sum_up(float x) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x = __fadd_ru(x, __shfl_xor_sync(kFull, x, o));
     return x;
+}
+
+// Which passes the chain of kernels does faster.  The loop keeps 16 warps per SM and a row with
+// its block, where the chain spreads a row over the grid and keeps more loads in flight; the chain
+// pays 70 to 100 us for its launches and has no memory in its bounds.  Measured on GB300:
+//   screening  the loop 0.18 to 0.3 us per 1000 terms (a term: 128 FP32 columns of one neighbour's
+//              row of S), the chain 0.1 us per 1000 of all blocks of the rows with
+//              neighbours where the iterate is dense: level at half of them;
+//   support    W_ij and W_ji by gathers, 1.3 us per 1000 of sum n_i^2 over the rows of the
+//              block that has most, as 6 terms each;
+//   search     1 us per pair of 32-entry chunks of a block's rows: level at about 400.
+// A pass that loses may be worth it (bounds that start anew keep more blocks than they do a pass
+// later, if the rows are short), so the losses add up to a debt, and the loop leaves when that
+// passes half a full pass.  Without bounds there is nothing to wait for.
+// us of the chain and of the loop per iteration, without the rule: p = 8192, n = 1000, lambda1 = 0.07
+// (130 entries a row) 8200, 18300; p = 2000, 90 entries a row 640, 1080; a hub row of 700
+// entries at p = 700 430, 710.
+// Terms are counted by 1024 here.
+constexpr unsigned kWorkEven = 512, kWorkBlind = 1370, kSupEven = 340;
+constexpr unsigned kDebtLeast = 256, kDebtMost = 32768;
+constexpr int kShortMean = 32;
+constexpr int kUnitsMax = 400;
+constexpr int kTasksFew = 1 << 16, kHeavyFew = 256, kSupFew = 900;
+__device__ __forceinline__ int row_units(int entries) {
+    const int c = (entries + 31) >> 5;
+    return c * (c + 1) / 2;
+}
+__device__ __forceinline__ int row_sup(int entries) { return min(entries, 1 << 13) * min(entries, 1 << 13) >> 6; }
+__device__ __forceinline__ unsigned sup_terms(int sup) { return 3u * (unsigned)sup >> 3; }
+// One more pass that does `work` where both forms are level at `even`; whether to leave before it.
+__device__ __forceinline__ bool in_debt(unsigned& debt, unsigned work, unsigned even, unsigned credit) {
+    debt = work > even ? debt + (work - even) : debt - min(debt, kWorkEven / 2);
+    return debt > min(kDebtLeast + credit, kDebtMost);
+}
+// Whether to leave before a pass of many tasks (the same answer in the whole grid), and whether
+// this block leaves its support entries out, which ends the launch after the screening barrier.
+// Block-wide calls.  Passes with few do not come here, and the calls are not inlined: with the
+// arithmetic in line every pass took 2 us longer (47.8 -> 50.5 us at p = 400).
+template <typename T>
+__device__ __noinline__ bool leave_tasks(LoopSmem<T>& sm, unsigned long long terms64, int nnz, int nbm, int p) {
+    const unsigned whole = (unsigned)((unsigned long long)nbm * (unsigned)nnz >> 10);
+    if (threadIdx.x == 0)
+        sm.leave[1] = in_debt(sm.debt, (unsigned)(terms64 >> 4), kWorkEven + whole / 2,
+                              nnz / kShortMean < p ? whole / 2 : 0u);
+    __syncthreads();
+    return sm.leave[1] != 0;
+}
+template <typename T>
+__device__ __noinline__ bool leave_support(LoopSmem<T>& sm, int* full) {
+    if (threadIdx.x == 0) {
+        sm.leave[0] = in_debt(sm.sup_debt, sup_terms(sm.sup), kSupEven, 0u);
+        if (sm.leave[0]) atomicOr(full, kFullDense);
+    }
+    __syncthreads();
+    return sm.leave[0] != 0;
 }
 
 // After a timeout: no further pass of either graph loop.
@@ -842,7 +910,6 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
     const double lam2d = ctrl->lam2;
     const int iter_limit = ctrl->iter_limit, use_stop = ctrl->use_stop;
     const int ng = k.m1g ? k.nbm / 8 : 0;
-    constexpr int kHeavyTerms = 32;    // rows with more terms are screened by four warps a block
     unsigned target = 0;
     int iter = ctrl->iter;
     long long trials = 0;
@@ -853,7 +920,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
     int pbuf = 0;                      // partial buffer
     int buf = 0;                       // CSR buffer of the current iterate: 0 cur, 1 next
     int last_h = 0;
-    if (tid == 0) { sm.flags = 0; sm.full = 0; sm.accept = -1; sm.converged = 0; sm.n2 = 0.0; sm.nlong = 0; sm.nhuge = 0; sm.ni = 0; sm.npl = 0; }
+    if (tid == 0) { sm.flags = 0; sm.full = 0; sm.accept = -1; sm.converged = 0; sm.n2 = 0.0; sm.nlong = 0; sm.nhuge = 0; sm.ni = 0; sm.npl = 0; sm.sup = 0; sm.units = 0; }
     __syncthreads();
 
     // ---------------- set-up of the owned rows from the current iterate
@@ -878,6 +945,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         s_mv[r] = 0;
         if (!pure) {
             s_list[atomicAdd(&sm.nlong, 1)] = r;
+            atomicAdd(&sm.sup, row_sup(re - rb));
             const int at = atomicAdd(&sm.ni, re - rb);
             for (int q = rb; q < re; ++q)
                 if (at + q - rb < kItemCap) { sm.items[at + q - rb] = q; sm.item_r[at + q - rb] = (short)r; }
@@ -903,9 +971,17 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         if (k.m1) atomicMax(k.mg, __float_as_uint(m) & 0x7fffffffu);
         if (pure && k.m1 && !(mulT(dv, (T)m) <= lam1)) s_pl[atomicAdd(&sm.npl, 1)] = r;
     }
+    __syncthreads();
+    if (tid == 0) {
+        unsigned d = 0u;
+        sm.debt = ctrl->loop_debt;
+        sm.sup_debt = 0u;
+        if (in_debt(d, sup_terms(sm.sup), kSupEven, 0u)) atomicOr(k.ctr + kCtrFull, kFullDense);
+    }
     bool alive = loop_barrier(k.bar, target, ctrl, &sm.ok);
     const float mg = __uint_as_float(__ldcg(k.mg));
-    if (alive && k.bnd) {
+    bool dense = alive && (__ldcg(k.ctr + kCtrFull) & kFullDense) != 0;
+    if (alive && k.bnd && !dense) {
         // the tasks of the rows of the diagonal alone; the bounds of the others, from their
         // weights
         for (int li = warp; li < sm.npl; li += kLW) pure_row_tasks(k, i0 + s_pl[li], s_dv[s_pl[li]], lam1, par, lane);
@@ -915,7 +991,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
             float sw = 0.0f;
             for (int q = ri.x + lane; q < ri.y; q += 32) sw = __fadd_ru(sw, abs_up(k.cur.cv[q]));
             const float slack = slack_of<T>(ri.y - ri.x + 1, warp_sum_up(sw), mg);
-            bound_row(k, i, ri.y - ri.x, true, ri.y - ri.x > kHeavyTerms, slack, lam1, par, lane, [&](int e, int& c, float& w, bool&) {
+            bound_row(k, i, ri.y - ri.x, true, ri.y - ri.x, slack, lam1, par, lane, [&](int e, int& c, float& w, bool&) {
                 c = k.cur.ci[ri.x + e];
                 w = abs_up(k.cur.cv[ri.x + e]);
             });
@@ -926,17 +1002,23 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
     bool run = alive && iter < iter_limit;
 
     while (run) {
+        if (!k.bnd) dense |= ((unsigned long long)k.nbm * (unsigned)nnz_now >> 10) > kWorkBlind;
+        if (dense) break;
         const Csr<T> om = buf ? k.next : k.cur;
         const Csr<T> out = buf ? k.cur : k.next;
         const long long t_scr = tid == 0 && bid == 0 ? tail_clock_ns() : 0;
-        ++attempts;
         // ---------------- screen
         if (bid == 0 && tid == 0) k.ctr[kCtrBig] = 0;
         Hits<T> hits{sm.hit_i[warp], sm.hit_j[warp], sm.hit_w[warp], 0, 0};
         // the owned rows' support entries, then a share of the (row, block) tasks
-        screen_support(k, om, i0, nr, sm.items, sm.item_r, sm.ni, s_rb, s_rc, sm.e0, sm.e1, lam2, hits.emitted);
+        if (sm.sup < kSupFew || !leave_support(sm, k.ctr + kCtrFull))
+            screen_support(k, om, i0, nr, sm.items, sm.item_r, sm.ni, s_rb, s_rc, sm.e0, sm.e1, lam2, hits.emitted);
         {
-            const int nt = k.bnd ? __ldcg(k.ctr + kCtrTask + par) : 0, nh = k.bnd ? __ldcg(k.ctr + kCtrHeavy + par) : 0;
+            const ulonglong2 todo = k.bnd ? __ldcg(k.todo + par) : make_ulonglong2(0, 0);
+            const int nt = (int)todo.x, nh = (int)todo.y;
+            // the same in every block: the pass is left to the chain before its tasks
+            if (nt > kTasksFew || nh > kHeavyFew) dense = leave_tasks(sm, (todo.x >> 32) + (todo.y >> 32), nnz_now, k.nbm, k.p);
+            if (dense) break;
             const bool all = !k.bnd || nt > k.ntask_cap - nh || nt < 0 || nh < 0;
             const int* list = k.tasks + (size_t)par * k.ntask_cap;
             if (!all) {
@@ -960,9 +1042,12 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         // ---------------- build
         // this parity's list was read by every block before the barrier: empty it for the
         // accept step of the next iteration
-        if (bid == nb - 1 && tid == 0) { k.ctr[kCtrTask + par] = 0; k.ctr[kCtrHeavy + par] = 0; }
-        if (tid == 0) { sm.nlong = 0; sm.nhuge = 0; sm.pool_full = __ldcg(k.ctr + kCtrFull); }
+        if (bid == nb - 1 && tid == 0) k.todo[par] = make_ulonglong2(0, 0);
+        if (tid == 0) { sm.nlong = 0; sm.nhuge = 0; sm.units = 0; sm.pool_full = __ldcg(k.ctr + kCtrFull); }
         __syncthreads();
+        dense = (sm.pool_full & kFullDense) != 0;      // a block has left its support out
+        if (dense) break;
+        ++attempts;
         const bool pool_full = sm.pool_full != 0;
         int em = hits.emitted, bad = 0, full = 0;
         A o2{};
@@ -990,6 +1075,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
                 } else {
                     s_rc[r] = pure ? -1 - c : c;
                     kind = c + (pure ? 1 : 0) <= 32 ? 1 : 2;
+                    if (kind == 2) atomicAdd(&sm.units, row_units(c + (pure ? 1 : 0)));
                 }
             }
             const unsigned b1 = __ballot_sync(kFull, kind == 1), b2 = __ballot_sync(kFull, kind == 2);
@@ -1004,7 +1090,10 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
             if (tid == kLT - 1) { sm.nlong = p1 + __popc(b1); sm.nhuge = p2 + __popc(b2); }
             __syncthreads();
         }
-        const int nsmall = sm.nlong, nlong = nsmall + sm.nhuge;
+        // too much for one block: as a full bucket
+        const bool many = sm.units > kUnitsMax;
+        if (many && tid == 0) ++full;
+        const int nsmall = many ? 0 : sm.nlong, nlong = many ? 0 : nsmall + sm.nhuge;
         auto row_at = [&](int li) { return li < nsmall ? s_list[li] : s_list[R - 1 - (li - nsmall)]; };
         auto ents_of = [&](int r) { return s_eo[r] < 0 ? k.ents + (size_t)(i0 + r) * kSlots : k.big + s_eo[r]; };
         // rows of more than kSlots candidates: the whole block on one, keys in shared memory
@@ -1397,7 +1486,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         // ---------------- accept: the owned rows of Omega+
         const T tau = tau_pow2<T>(h), tl1 = tau * lam1;
         const int par2 = par ^ 1;
-        if (tid == 0) { sm.ni = 0; sm.npl = 0; }
+        if (tid == 0) { sm.ni = 0; sm.npl = 0; sm.sup = 0; sm.units = 0; }
         __syncthreads();
         if (bid == 0 && tid == 0) { k.ctr[kCtrPage] = 0; k.ctr[kCtrFull] = 0; }
         // entries per row (s_rc of a long row becomes its entry count)
@@ -1489,7 +1578,10 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
             __syncwarp();
             if (!pure) {
                 int at = 0;
-                if (lane == 0) at = atomicAdd(&sm.ni, o - rb);
+                if (lane == 0) {
+                    at = atomicAdd(&sm.ni, o - rb);
+                    atomicAdd(&sm.sup, row_sup(o - rb));
+                }
                 at = __shfl_sync(kFull, at, 0);
                 for (int q = lane; q < o - rb; q += 32)
                     if (at + q < kItemCap) { sm.items[at + q] = rb + q; sm.item_r[at + q] = (short)r; }
@@ -1505,7 +1597,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
             if (!pure && k.bnd) {
                 const float slack = slack_of<T>(o - rb + 1, warp_sum_up(sw), mg);
                 if (lane == 0) k.slack[i] = slack;
-                bound_row(k, i, L, init, o - rb > kHeavyTerms, slack, lam1, par2, lane, [&](int e, int& c, float& w, bool& left) {
+                bound_row(k, i, L, init, o - rb, slack, lam1, par2, lane, [&](int e, int& c, float& w, bool& left) {
                     const Ent<T> x = ld_ent(re + e);
                     c = (int)(x.cf & kColMask);
                     const T v = prox_entry(x.om, x.g, tau, tl1, c == i);
@@ -1621,11 +1713,13 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
                 }
             }
         }
-        ctrl->loop_full = sm.full;
-        if (sm.full) ctrl->chain_left = 1 << min(ctrl->loop_fulls++, 6);
+        const int leave = sm.full || (dense && run) ? 1 : 0;
+        ctrl->loop_full = leave;
+        ctrl->loop_debt = leave ? 0u : sm.debt;
+        if (leave) ctrl->chain_left = 1 << min(ctrl->loop_fulls++, 6);
         if (k.use_cond) {
-            cudaGraphSetConditional(k.chain_cond, sm.full ? 1u : 0u);
-            cudaGraphSetConditional(k.outer_cond, sm.full ? 1u : 0u);
+            cudaGraphSetConditional(k.chain_cond, leave ? 1u : 0u);
+            cudaGraphSetConditional(k.outer_cond, leave ? 1u : 0u);
         }
     }
 }
@@ -1637,6 +1731,7 @@ __global__ void k_loop_arm(LoopK<T> k) {
     for (int i = t; i < k.p; i += n) k.cnt[i] = 0;
     for (size_t i = t; i < (size_t)k.p * kPages; i += n) k.pages[i] = 0;
     if (t < kCtrCount) k.ctr[t] = 0;
+    if (t < 2) k.todo[t] = make_ulonglong2(0, 0);
     if (t == 0) {
         *k.bar = 0u;
         *k.mg = 0u;
@@ -1692,6 +1787,7 @@ LoopK<T> loop_args(const IterBufs<T>& b, void* ws, int R, size_t* bytes) {
     k.part_a = reinterpret_cast<double*>(take(2 * (size_t)kNA * b.num_sms * sizeof(double)));
     k.part_i = reinterpret_cast<int*>(take(2 * (size_t)kNI * b.num_sms * sizeof(int)));
     k.ctr = reinterpret_cast<int*>(take(kCtrCount * sizeof(int)));
+    k.todo = reinterpret_cast<ulonglong2*>(take(2 * sizeof(ulonglong2)));
     if (bytes) *bytes = (size_t)(q - static_cast<uint8_t*>(ws));
     return k;
 }
