@@ -87,7 +87,7 @@ constexpr int kHeavyTerms = 32;          // rows with more terms are screened by
 constexpr int kQA = 3 * kWin;            // accumulated partials per window: quadratic form, ||D||^2, phi
 constexpr int kQI = 2 * kWin;            // counted partials per window: w+_ii <= 0, entries kept
 constexpr int kNA = 2 * kQA + 1;         // and ||Omega||^2
-constexpr int kNI = 2 * kQI + 3;         // and own entries emitted, NaN / Inf, full rows
+constexpr int kNI = 2 * kQI + 5;         // and entries emitted, NaN / Inf, full rows, Hits::halves, rows with neighbours
 
 constexpr unsigned kColMask = 0x0fffffffu;
 constexpr unsigned kFSupp = 0x80000000u;
@@ -316,6 +316,7 @@ struct Hits {
     T* w;
     int n;        // the same in every lane
     int emitted;  // per lane: entries with |W_ij| > lambda1 or in the support
+    int halves;   // pairs of rows with the diagonal alone where one of the two entries is
 
     __device__ __forceinline__ void flush(const LoopK<T>& k, const Csr<T>& csr, T lam1, T lam2, int lane) {
         __syncwarp();
@@ -327,9 +328,10 @@ struct Hits {
             const T wji = gather_w(k, csr, col, row);
             // row col's own screening meets the pair too where |W_ji| > lambda1
             const bool first_meets = row < col || fabs(wji) <= lam1;
-            // two rows with the diagonal alone count as a pair, as in the chain's list
             const bool both = __ldcg(k.rds + row) > T(0) && __ldcg(k.rds + col) > T(0);
-            emitted += both ? (first_meets ? 2 : 0) : 1;
+            const bool other = !(fabs(wji) <= lam1);
+            emitted += both ? (first_meets ? 1 + other : 0) : 1;
+            halves += both && first_meets && !other;
             if (first_meets) {
                 const T g = gradient_of(wij, wji, T(0), lam2, false);
                 if (!(fabs(g) <= lam1)) {
@@ -1009,7 +1011,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         const long long t_scr = tid == 0 && bid == 0 ? tail_clock_ns() : 0;
         // ---------------- screen
         if (bid == 0 && tid == 0) k.ctr[kCtrBig] = 0;
-        Hits<T> hits{sm.hit_i[warp], sm.hit_j[warp], sm.hit_w[warp], 0, 0};
+        Hits<T> hits{sm.hit_i[warp], sm.hit_j[warp], sm.hit_w[warp], 0, 0, 0};
         // the owned rows' support entries, then a share of the (row, block) tasks
         if (sm.sup < kSupFew || !leave_support(sm, k.ctr + kCtrFull))
             screen_support(k, om, i0, nr, sm.items, sm.item_r, sm.ni, s_rb, s_rc, sm.e0, sm.e1, lam2, hits.emitted);
@@ -1049,7 +1051,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         if (dense) break;
         ++attempts;
         const bool pool_full = sm.pool_full != 0;
-        int em = hits.emitted, bad = 0, full = 0;
+        int em = hits.emitted, bad = 0, full = 0, off = 0;
         A o2{};
         // the rows with candidates beside the diagonal, in row order (the sums below follow it)
         for (int r0 = 0; r0 < nr; r0 += kLT) {
@@ -1060,7 +1062,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
                 const bool pure = s_rc[r] < 0;
                 const T dv = s_dv[r];
                 s_om[r] = dv;
-                if (pure) ++em;
+                if (pure) ++em; else ++off;
                 if (c) k.cnt[i] = 0;
                 if (c > kMaxE - 2 || (pool_full && c > kSlots)) {
                     ++full;
@@ -1364,11 +1366,14 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
             }
             if (first) {
                 const int d = __reduce_add_sync(kFull, em), e = __reduce_add_sync(kFull, bad),
-                          f = __reduce_add_sync(kFull, full);
+                          f = __reduce_add_sync(kFull, full), hv = __reduce_add_sync(kFull, hits.halves),
+                          nf = __reduce_add_sync(kFull, off);
                 if (lane == 0) {
                     sm.red_i[warp][2 * kQI] = d;
                     sm.red_i[warp][2 * kQI + 1] = e;
                     sm.red_i[warp][2 * kQI + 2] = f;
+                    sm.red_i[warp][2 * kQI + 3] = hv;
+                    sm.red_i[warp][2 * kQI + 4] = nf;
                 }
             }
             __syncthreads();
@@ -1433,8 +1438,11 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
                 // lane x: step size h_base + x
                 int flags = 0, full_rows = 0;
                 if (first) {
-                    // the own entries emitted, against the handle's candidate capacity (as the
-                    // chain's emission list has it)
+                    // the entries emitted, against the handle's candidate capacity (as the chain's
+                    // list has them: up to p / 2 rows with neighbours, two rows with the
+                    // diagonal alone emit both entries or none)
+                    if (lane == 0 && 2 * sm.sum_i[2 * kQI + 4] <= k.p) sm.sum_i[2 * kQI] += sm.sum_i[2 * kQI + 3];
+                    __syncwarp();
                     if (sm.sum_i[2 * kQI] > k.em_cap) flags = kFlagEmOverflow;
                     else if (sm.sum_i[2 * kQI + 2] > 0) full_rows = 1;
                     else if (sm.sum_i[2 * kQI + 1] > 0) flags = kFlagNaN;
