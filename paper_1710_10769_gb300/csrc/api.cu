@@ -1942,27 +1942,54 @@ int hpc_get_s_entries(hpc_handle h, int64_t m, const int64_t* rows, const int64_
     return HPC_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+int adj_reserve(hpc_ctx* h, size_t bytes) {
+    if (bytes <= h->adj_bytes) return HPC_OK;
+    if (h->adj_buf) release(h, h->adj_buf);
+    h->adj_buf = nullptr;
+    h->adj_bytes = 0;
+    CUDA_TRY(hold(h, &h->adj_buf, bytes));
+    h->adj_bytes = bytes;
+    return HPC_OK;
+}
+
+template <typename T>
+int get_loop_candidates(hpc_ctx* h, int64_t* m_inout, int64_t* rows, int64_t* cols, double* omega, double* grad) {
+    const hpc::IterBufs<T> b = bufs<T>(h);
+    std::vector<int> at;
+    int64_t n = 0;
+    CUDA_TRY(hpc::loop_candidate_places<T>(b, at, &n, h->stream));
+    if (rows) {
+        if (n > *m_inout) return HPC_ERR_CAPACITY;
+        STATUS_TRY(adj_reserve(h, hpc::loop_candidate_bytes(h->p, n)));
+        std::vector<hpc::LoopCandidate> c((size_t)n);
+        CUDA_TRY(hpc::loop_candidates<T>(b, h->loop_ws, at, n, h->adj_buf, c.data(), h->stream));
+        for (int64_t t = 0; t < n; ++t) {
+            rows[t] = c[t].row;
+            cols[t] = c[t].col;
+            if (omega) omega[t] = c[t].om;
+            if (grad) grad[t] = c[t].g;
+        }
+    }
+    *m_inout = n;
+    return HPC_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 int hpc_get_candidates(hpc_handle h, int64_t* m_inout, int64_t* rows, int64_t* cols, double* omega, double* grad) {
     if (!h || !m_inout) return HPC_ERR_ARG;
     const int64_t p = h->p;
     STATUS_TRY(read_ctrl(h));
     if (h->loop_ws && h->h_ctrl->loop_attempts > 0 && !h->h_ctrl->loop_full) {
         // the last gradient pass ran in the one-launch loop
-        std::vector<hpc::LoopCandidate> c;
-        const int e = h->vdt == HPC_F64 ? hpc::loop_candidates<double>(bufs<double>(h), h->loop_ws, c, h->stream)
-                                        : hpc::loop_candidates<float>(bufs<float>(h), h->loop_ws, c, h->stream);
-        if (e != 0) { set_cuda_error((cudaError_t)e, "candidates", __LINE__); return HPC_ERR_CUDA; }
-        if (rows) {
-            if ((int64_t)c.size() > *m_inout) return HPC_ERR_CAPACITY;
-            for (size_t t = 0; t < c.size(); ++t) {
-                rows[t] = c[t].row;
-                cols[t] = c[t].col;
-                if (omega) omega[t] = c[t].om;
-                if (grad) grad[t] = c[t].g;
-            }
-        }
-        *m_inout = (int64_t)c.size();
-        return HPC_OK;
+        return h->vdt == HPC_F64 ? get_loop_candidates<double>(h, m_inout, rows, cols, omega, grad)
+                                 : get_loop_candidates<float>(h, m_inout, rows, cols, omega, grad);
     }
     std::vector<int> off(p + 1), len(p);
     CUDA_TRY(cudaMemcpyAsync(off.data(), h->bk_off, (p + 1) * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
@@ -2003,16 +2030,6 @@ int hpc_get_candidates(hpc_handle h, int64_t* m_inout, int64_t* rows, int64_t* c
 }  // extern "C"
 
 namespace {
-
-int adj_reserve(hpc_ctx* h, size_t bytes) {
-    if (bytes <= h->adj_bytes) return HPC_OK;
-    if (h->adj_buf) release(h, h->adj_buf);
-    h->adj_buf = nullptr;
-    h->adj_bytes = 0;
-    CUDA_TRY(hold(h, &h->adj_buf, bytes));
-    h->adj_bytes = bytes;
-    return HPC_OK;
-}
 
 template <typename T>
 hpc::Csr<T> cur_csr(hpc_ctx* h) { return {h->rp[h->cur], h->ci[h->cur], as<T>(h->cv[h->cur])}; }

@@ -245,13 +245,18 @@ template <typename T> cudaError_t launch_loop(const IterBufs<T>& b, void* ws, co
 // Blocks of that launch (0: the sizes do not fit it) and rows per block.
 template <typename T> int loop_grid(int p, int nbm, int num_sms, int* rows);
 template <typename T> size_t loop_workspace_bytes(int p, int nbm, int num_sms);
-// Candidates of the loop's last gradient pass, row by row, columns ascending (a CUDA error code).
+// Candidates of the loop's last gradient pass, row by row, columns ascending: each row's place and their
+// number n, then the entries, by way of loop_candidate_bytes(p, n) of device memory at tmp.
 struct LoopCandidate {
     int row, col;
     double om, g;
 };
 template <typename T>
-int loop_candidates(const IterBufs<T>& b, void* ws, std::vector<LoopCandidate>& out, cudaStream_t s);
+cudaError_t loop_candidate_places(const IterBufs<T>& b, std::vector<int>& at, int64_t* n, cudaStream_t s);
+size_t loop_candidate_bytes(int64_t p, int64_t n);
+template <typename T>
+cudaError_t loop_candidates(const IterBufs<T>& b, void* ws, const std::vector<int>& at, int64_t n, void* tmp,
+                            LoopCandidate* out, cudaStream_t s);
 constexpr int kLaunchesLoop = 2;         // k_loop_arm, k_loop
 
 // One cooperative launch of a one-block kernel that adds 1 to *out and sets cond to 0.

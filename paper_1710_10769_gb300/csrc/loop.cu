@@ -1749,6 +1749,21 @@ __global__ void k_loop_arm(LoopK<T> k) {
     }
 }
 
+// The candidates of the last pass, row by row, a warp per row: row i's from place at[i] on, n in all.
+template <typename T>
+__global__ void __launch_bounds__(256) k_loop_candidates(LoopK<T> k, const int* __restrict__ at, int64_t n,
+                                                         LoopCandidate* __restrict__ out) {
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= k.p) return;
+    const int L = max(1, k.len[i]), off = k.eoff[i];
+    if (off >= 0 && off + L > 2 * k.npool * kSlots) return;
+    const Ent<T>* e = off < 0 ? k.ents + (size_t)i * kSlots : k.big + off;
+    for (int q = threadIdx.x & 31; q < min(L, off < 0 ? kSlots : L) && at[i] + q < n; q += 32) {
+        const Ent<T> x = ld_ent(e + q);
+        out[at[i] + q] = LoopCandidate{i, (int)(x.cf & kColMask), (double)x.om, (double)x.g};
+    }
+}
+
 size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 template <typename T>
@@ -1838,23 +1853,34 @@ size_t loop_workspace_bytes(int p, int nbm, int num_sms) {
 }
 
 template <typename T>
-int loop_candidates(const IterBufs<T>& b, void* ws, std::vector<LoopCandidate>& out, cudaStream_t s) {
+cudaError_t loop_candidate_places(const IterBufs<T>& b, std::vector<int>& at, int64_t* n, cudaStream_t s) {
+    at.resize((size_t)b.p);
+    cudaError_t e = cudaMemcpyAsync(at.data(), b.bk.len, at.size() * sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    *n = 0;
+    for (int& a : at) {
+        const int L = std::max(1, a);
+        a = (int)*n;
+        *n += L;
+    }
+    return e;
+}
+
+size_t loop_candidate_bytes(int64_t p, int64_t n) {
+    return align256((size_t)p * sizeof(int)) + (size_t)n * sizeof(LoopCandidate);
+}
+
+template <typename T>
+cudaError_t loop_candidates(const IterBufs<T>& b, void* ws, const std::vector<int>& at, int64_t n, void* tmp,
+                            LoopCandidate* out, cudaStream_t s) {
     const LoopK<T> k = loop_args<T>(b, ws, 1, nullptr);
-    const size_t p = (size_t)b.p;
-    std::vector<int> L(p), off(p);
-    std::vector<Ent<T>> e(p * kSlots), big(2 * (size_t)k.npool * kSlots);
-    cudaError_t r = cudaMemcpyAsync(L.data(), k.len, p * sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (r == cudaSuccess) r = cudaMemcpyAsync(off.data(), k.eoff, p * sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (r == cudaSuccess) r = cudaMemcpyAsync(e.data(), k.ents, e.size() * sizeof(Ent<T>), cudaMemcpyDeviceToHost, s);
-    if (r == cudaSuccess) r = cudaMemcpyAsync(big.data(), k.big, big.size() * sizeof(Ent<T>), cudaMemcpyDeviceToHost, s);
-    if (r == cudaSuccess) r = cudaStreamSynchronize(s);
-    if (r != cudaSuccess) return (int)r;
-    for (size_t i = 0; i < p; ++i)
-        for (int q = 0; q < std::max(1, L[i]); ++q) {
-            const Ent<T>& x = off[i] < 0 ? e[i * kSlots + q] : big[(size_t)off[i] + q];
-            out.push_back(LoopCandidate{(int)i, (int)(x.cf & kColMask), (double)x.om, (double)x.g});
-        }
-    return 0;
+    LoopCandidate* d = reinterpret_cast<LoopCandidate*>(static_cast<uint8_t*>(tmp) + align256(at.size() * sizeof(int)));
+    cudaError_t e = cudaMemcpyAsync(tmp, at.data(), at.size() * sizeof(int), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return e;
+    k_loop_candidates<T><<<(unsigned)((b.p + 7) / 8), 256, 0, s>>>(k, static_cast<const int*>(tmp), n, d);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = cudaMemcpyAsync(out, d, (size_t)n * sizeof(LoopCandidate), cudaMemcpyDeviceToHost, s);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(s);
 }
 
 template <typename T>
@@ -1883,7 +1909,9 @@ cudaError_t launch_loop(const IterBufs<T>& b, void* ws, const LoopCond& lc, cuda
 #define HPC_LOOP_INSTANTIATE(T)                                                                              \
     template int loop_grid<T>(int, int, int, int*);                                                          \
     template size_t loop_workspace_bytes<T>(int, int, int);                                                  \
-    template int loop_candidates<T>(const IterBufs<T>&, void*, std::vector<LoopCandidate>&, cudaStream_t); \
+    template cudaError_t loop_candidate_places<T>(const IterBufs<T>&, std::vector<int>&, int64_t*, cudaStream_t); \
+    template cudaError_t loop_candidates<T>(const IterBufs<T>&, void*, const std::vector<int>&, int64_t, void*,   \
+                                            LoopCandidate*, cudaStream_t);                                   \
     template cudaError_t launch_loop<T>(const IterBufs<T>&, void*, const LoopCond&, cudaStream_t);
 
 HPC_LOOP_INSTANTIATE(float)
