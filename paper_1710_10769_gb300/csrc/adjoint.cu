@@ -642,8 +642,10 @@ k_support_sddmm(int p, Csr<T> om, const T* __restrict__ yt, const T* __restrict_
 // Measured on GB300, p = 16384, 28 672 entries: 88 iterations in 1.00 ms, 11.4 us each (three
 // kernels in a graph: about 15).
 //
-// Every wait is bounded (kCgWaitNs): after that CgState::timeout is raised and every block
-// leaves.  The cooperative launch keeps all blocks resident.
+// Every wait is bounded: after CgArgs::wait_ns CgState::timeout is raised and every block leaves.
+// The cooperative launch keeps all blocks resident.  A phase between two barriers gathers
+// sum n_i^2 <= nnz p entries of S, which at a few 10^9 a second on wide supports takes longer than
+// any fixed limit; the limit is 4 s and 0.1 ns for each of the nnz p.
 constexpr long long kCgWaitNs = 4000000000ll;
 constexpr int kCgT = 256;
 
@@ -662,6 +664,7 @@ struct CgArgs {
     double *x, *r, *p0, *p1, *Ap, *Tv;      // x, Ap, Tv: not RES
     double* part;                           // four arrays of kCgMaxBlocks partials
     CgState* st;
+    long long wait_ns;
 };
 
 // sum over the block of s, into *out by thread 0 (fixed order)
@@ -702,7 +705,7 @@ __device__ __forceinline__ CgSum cg_total(const double* part, double num) {
 }
 
 // Grid-wide barrier on a counter that only grows; false after a timeout.
-__device__ __forceinline__ bool cg_barrier(CgState* st, unsigned& target) {
+__device__ __forceinline__ bool cg_barrier(CgState* st, long long wait_ns, unsigned& target) {
     __shared__ int ok_s;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -719,7 +722,7 @@ __device__ __forceinline__ bool cg_barrier(CgState* st, unsigned& target) {
                 unsigned long long t;
                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
                 if (t0 == 0) t0 = (long long)t;
-                if (*static_cast<volatile int*>(&st->timeout) || (long long)t - t0 > kCgWaitNs) {
+                if (*static_cast<volatile int*>(&st->timeout) || (long long)t - t0 > wait_ns) {
                     atomicExch(&st->timeout, 1);
                     ok = 0;
                     break;
@@ -835,7 +838,7 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
         }
     }
     cg_block_sum(s, part[0] + blockIdx.x);
-    bool alive = cg_barrier(k.st, target);
+    bool alive = cg_barrier(k.st, k.wait_ns, target);
     double rr = alive ? cg_total<true>(part[0], 1.0).total : 0.0, beta = 0.0;       // the first direction is r itself
     const double rr0 = rr;
     int done = rr == 0.0 ? 1 : 0;
@@ -860,7 +863,7 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
                 k.Tv[e] = cg_row_dot(k, k.rinfo[a], a, k.om.ci[e], p_old, beta);
                 p_new[e] = fma(beta, p_old[e], k.r[e]);
             }
-            if (!(alive = cg_barrier(k.st, target))) break;
+            if (!(alive = cg_barrier(k.st, k.wait_ns, target))) break;
             for (int64_t e = e0; e < k.nnz; e += step) {
                 const int t = k.tr[e] >= 0 ? k.tr[e] : (int)e;     // a symmetric pattern always has (j, i)
                 const double w = (double)k.om.cv[e], v = p_new[e];
@@ -872,7 +875,7 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
             }
         }
         cg_block_sum(s, part[1] + blockIdx.x);
-        if (!(alive = cg_barrier(k.st, target))) break;
+        if (!(alive = cg_barrier(k.st, k.wait_ns, target))) break;
         const CgSum pap = cg_total<false>(part[1], rr);
         ++it;
         if (!(pap.total > 0.0)) { done = 2; break; }               // H not positive definite along p
@@ -895,7 +898,7 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
             }
         }
         cg_block_sum(s, part[0] + blockIdx.x);
-        if (!(alive = cg_barrier(k.st, target))) break;
+        if (!(alive = cg_barrier(k.st, k.wait_ns, target))) break;
         const CgSum v = cg_total<true>(part[0], rr);
         beta = rr > 0.0 ? v.ratio : 0.0;
         rr = v.total;
@@ -916,7 +919,7 @@ __global__ void __launch_bounds__(kCgT) k_cg(CgArgs<T> k) {
     }
     cg_block_sum(s1, part[2] + blockIdx.x);
     cg_block_sum(s2, part[3] + blockIdx.x);
-    if (alive) alive = cg_barrier(k.st, target);
+    if (alive) alive = cg_barrier(k.st, k.wait_ns, target);
     if (blockIdx.x == 0 && alive) {
         s1 = cg_total<true>(part[2], 1.0).total;
         __syncthreads();
@@ -1139,11 +1142,11 @@ size_t cg_vector_doubles(int64_t nnz) { return 6 * (size_t)nnz + 4 * kCgMaxBlock
 
 // CG on H_A v = b and its two inner products; vec: cg_vector_doubles(nnz), st: zeroed here.
 template <typename T>
-cudaError_t launch_cg(int64_t nnz, const int* row, Csr<T> om, const int4* rinfo, const int* tr, const T* S, int64_t lds,
+cudaError_t launch_cg(int p, int64_t nnz, const int* row, Csr<T> om, const int4* rinfo, const int* tr, const T* S, int64_t lds,
                       double lam2, double tol, int64_t max_iter, const double* b, const double* sgn, const double* om_d,
                       double* vec, CgState* st, int num_sms, cudaStream_t s) {
     CgArgs<T> k{nnz, row, om, rinfo, tr, S, lds, lam2, tol * tol, max_iter, b, sgn, om_d, nullptr, nullptr, nullptr,
-                nullptr, nullptr, nullptr, nullptr, st};
+                nullptr, nullptr, nullptr, nullptr, st, kCgWaitNs + (long long)(0.1 * (double)nnz * (double)p)};
     double** v[6] = {&k.x, &k.r, &k.p0, &k.p1, &k.Ap, &k.Tv};
     for (int q = 0; q < 6; ++q) *v[q] = vec + (size_t)q * nnz;
     k.part = vec + 6 * (size_t)nnz;
@@ -1185,7 +1188,7 @@ cudaError_t launch_cg(int64_t nnz, const int* row, Csr<T> om, const int4* rinfo,
                                        cudaStream_t);                                                           \
     template void launch_support_heldout<T>(int64_t, const int*, Csr<T>, const int*, const double*, double*,     \
                                             cudaStream_t);                                                      \
-    template cudaError_t launch_cg<T>(int64_t, const int*, Csr<T>, const int4*, const int*, const T*, int64_t,  \
+    template cudaError_t launch_cg<T>(int, int64_t, const int*, Csr<T>, const int4*, const int*, const T*, int64_t,  \
                                       double, double, int64_t, const double*, const double*, const double*,     \
                                       double*, CgState*, int, cudaStream_t);                                    \
     template void launch_support_vectors<T>(int, int64_t, Csr<T>, double*, double*, cudaStream_t);          \

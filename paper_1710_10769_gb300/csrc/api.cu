@@ -2189,7 +2189,7 @@ int hypergrad_t(hpc_ctx* h, const void* Xval, int xdt, int64_t nval, double cg_t
     hpc::launch_support_xy<T>(p, om, h->rinfo, as<T>(h->rdv), xtv, ldv, nval, Tv, s);
     hpc::launch_support_heldout<T>(nnz, rowid, om, tr, Tv, bvec, s);
     // CG on H_A v = b, then dL_val/dlambda1 = -<v, sgn_off>, dL_val/dlambda2 = -<v, Omega_A>
-    CUDA_TRY(hpc::launch_cg<T>(nnz, rowid, om, h->rinfo, tr, static_cast<const T*>(h->S), h->ld, h->lam2, cg_tol, cg_max,
+    CUDA_TRY(hpc::launch_cg<T>(p, nnz, rowid, om, h->rinfo, tr, static_cast<const T*>(h->S), h->ld, h->lam2, cg_tol, cg_max,
                                bvec, sgn, om_d, vec, cg, h->num_sms, s));
     hpc::CgState st;
     CUDA_TRY(cudaMemcpyAsync(&st, cg, sizeof st, cudaMemcpyDeviceToHost, s));

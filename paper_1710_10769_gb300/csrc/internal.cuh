@@ -348,7 +348,7 @@ struct CgState {
 constexpr int kCgMaxBlocks = 2048;
 size_t cg_vector_doubles(int64_t nnz);
 template <typename T>
-cudaError_t launch_cg(int64_t nnz, const int* row, Csr<T> om, const int4* rinfo, const int* tr, const T* S, int64_t lds,
+cudaError_t launch_cg(int p, int64_t nnz, const int* row, Csr<T> om, const int4* rinfo, const int* tr, const T* S, int64_t lds,
                       double lam2, double tol, int64_t max_iter, const double* b, const double* sgn, const double* om_d,
                       double* vec, CgState* st, int num_sms, cudaStream_t s);
 template <typename T>

@@ -824,14 +824,14 @@ __device__ __forceinline__ float warp_sum_up(float x) {
 // its block, where the chain spreads a row over the grid and keeps more loads in flight; the chain
 // pays 70 to 100 us for its launches and has no memory in its bounds.  Measured on GB300:
 //   screening  the loop 0.18 to 0.3 us per 1000 terms (a term: 128 FP32 columns of one neighbour's
-//              row of S), the chain 0.1 us per 1000 of all blocks of the rows with
-//              neighbours where the iterate is dense: level at half of them;
-//   support    W_ij and W_ji by gathers, 1.3 us per 1000 of sum n_i^2 over the rows of the
-//              block that has most, as 6 terms each;
+//              row of S), the chain 0.1 us per 1000 terms of all blocks of the neighbours,
+//              nbm (nnz - p), where the iterate is dense: level at half of them;
+//   support    W_ij and W_ji by gathers, up to 1.3 us per 1000 of sum n_i^2 over the rows of
+//              the block that has most, as 6 terms each: a quarter of the chain's terms;
 //   search     1 us per pair of 32-entry chunks of a block's rows: level at about 400.
 // A pass that loses may be worth it (bounds that start anew keep more blocks than they do a pass
 // later, if the rows are short), so the losses add up to a debt, and the loop leaves when that
-// passes half a full pass.  Without bounds there is nothing to wait for.
+// passes half of the chain's terms.  Without bounds there is nothing to wait for.
 // us of the chain and of the loop per iteration, without the rule: p = 8192, n = 1000, lambda1 = 0.07
 // (130 entries a row) 8200, 18300; p = 2000, 90 entries a row 640, 1080; a hub row of 700
 // entries at p = 700 430, 710.
@@ -846,11 +846,16 @@ __device__ __forceinline__ int row_units(int entries) {
     return c * (c + 1) / 2;
 }
 __device__ __forceinline__ int row_sup(int entries) { return min(entries, 1 << 13) * min(entries, 1 << 13) >> 6; }
-__device__ __forceinline__ unsigned sup_terms(int sup) { return 3u * (unsigned)sup >> 3; }
+__device__ __forceinline__ unsigned chain_terms(int nnz, int nbm, int p) {
+    return (unsigned)((unsigned long long)nbm * (unsigned)max(0, nnz - p) >> 10);
+}
 // One more pass that does `work` where both forms are level at `even`; whether to leave before it.
 __device__ __forceinline__ bool in_debt(unsigned& debt, unsigned work, unsigned even, unsigned credit) {
     debt = work > even ? debt + (work - even) : debt - min(debt, kWorkEven / 2);
     return debt > min(kDebtLeast + credit, kDebtMost);
+}
+__device__ __forceinline__ bool support_debt(unsigned& debt, int sup, int nnz, int nbm, int p) {
+    return in_debt(debt, 3u * (unsigned)sup >> 3, kSupEven + chain_terms(nnz, nbm, p) / 4, 0u);
 }
 // Whether to leave before a pass of many tasks (the same answer in the whole grid), and whether
 // this block leaves its support entries out, which ends the launch after the screening barrier.
@@ -858,17 +863,17 @@ __device__ __forceinline__ bool in_debt(unsigned& debt, unsigned work, unsigned 
 // arithmetic in line every pass took 2 us longer (47.8 -> 50.5 us at p = 400).
 template <typename T>
 __device__ __noinline__ bool leave_tasks(LoopSmem<T>& sm, unsigned long long terms64, int nnz, int nbm, int p) {
-    const unsigned whole = (unsigned)((unsigned long long)nbm * (unsigned)nnz >> 10);
+    const unsigned chain = chain_terms(nnz, nbm, p);
     if (threadIdx.x == 0)
-        sm.leave[1] = in_debt(sm.debt, (unsigned)(terms64 >> 4), kWorkEven + whole / 2,
-                              nnz / kShortMean < p ? whole / 2 : 0u);
+        sm.leave[1] = in_debt(sm.debt, (unsigned)(terms64 >> 4), kWorkEven + chain / 2,
+                              nnz / kShortMean < p ? chain / 2 : 0u);
     __syncthreads();
     return sm.leave[1] != 0;
 }
 template <typename T>
-__device__ __noinline__ bool leave_support(LoopSmem<T>& sm, int* full) {
+__device__ __noinline__ bool leave_support(LoopSmem<T>& sm, int* full, int nnz, int nbm, int p) {
     if (threadIdx.x == 0) {
-        sm.leave[0] = in_debt(sm.sup_debt, sup_terms(sm.sup), kSupEven, 0u);
+        sm.leave[0] = support_debt(sm.sup_debt, sm.sup, nnz, nbm, p);
         if (sm.leave[0]) atomicOr(full, kFullDense);
     }
     __syncthreads();
@@ -978,7 +983,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         unsigned d = 0u;
         sm.debt = ctrl->loop_debt;
         sm.sup_debt = 0u;
-        if (in_debt(d, sup_terms(sm.sup), kSupEven, 0u)) atomicOr(k.ctr + kCtrFull, kFullDense);
+        if (support_debt(d, sm.sup, nnz_now, k.nbm, k.p)) atomicOr(k.ctr + kCtrFull, kFullDense);
     }
     bool alive = loop_barrier(k.bar, target, ctrl, &sm.ok);
     const float mg = __uint_as_float(__ldcg(k.mg));
@@ -1013,7 +1018,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         if (bid == 0 && tid == 0) k.ctr[kCtrBig] = 0;
         Hits<T> hits{sm.hit_i[warp], sm.hit_j[warp], sm.hit_w[warp], 0, 0, 0};
         // the owned rows' support entries, then a share of the (row, block) tasks
-        if (sm.sup < kSupFew || !leave_support(sm, k.ctr + kCtrFull))
+        if (sm.sup < kSupFew || !leave_support(sm, k.ctr + kCtrFull, nnz_now, k.nbm, k.p))
             screen_support(k, om, i0, nr, sm.items, sm.item_r, sm.ni, s_rb, s_rc, sm.e0, sm.e1, lam2, hits.emitted);
         {
             const ulonglong2 todo = k.bnd ? __ldcg(k.todo + par) : make_ulonglong2(0, 0);
