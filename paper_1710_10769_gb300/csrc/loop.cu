@@ -1826,11 +1826,7 @@ LoopK<T> loop_args(const IterBufs<T>& b, void* ws, int R, size_t* bytes) {
 // block, at most one block per SM.  0 blocks: the sizes do not fit the loop.
 template <typename T>
 int loop_grid(int p, int nbm, int num_sms, int* rows) {
-    // Up to 16 rows per block, half of the SMs do in FP32 (p = 1001, 40 iterations: 126 blocks 1.41 ms, 72
-    // 1.38; FP64, p = 900: 2.3, 2.5), and two problems run side by side (a solve at p = 1000 on
-    // each of 16 streams: 9.8 -> 5.2 ms).
-    const int most = sizeof(T) == 4 && (p + 15) / 16 <= num_sms / 2 ? num_sms / 2 : num_sms;
-    const int nb = std::max(1, std::min(most, (p + 7) / 8));
+    const int nb = std::max(1, std::min(num_sms, (p + 7) / 8));
     const int R = (p + nb - 1) / nb;
     if (rows) *rows = R;
     if (R > kMaxR || (long long)p * nbm > 0x7fffffffll ||
