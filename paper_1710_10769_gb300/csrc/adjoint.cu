@@ -222,8 +222,9 @@ __device__ __forceinline__ void pair_of(long long t, int nt, int& bi, int& bj) {
 // entries to S, one row after the other, the rows with neighbours were a chain of three
 // latencies each, about nine of them per warp where half of the rows have neighbours.
 // Measured on GB300, p = 16384, 28 672 entries (half of the rows with neighbours): 770 -> 572 us.
-// A tile pair whose rows have more than kGradList entries takes the rows one by one, a warp
-// each (offdiag_row, support_terms_row).
+// Rows with more than kGradList entries in all come in one list after another (their support terms
+// a warp per row).  With a warp per row for such tile pairs, hub rows took longer: 4000 entries
+// at p = 4096 4.8 ms, 3.9 now, 8000 at p = 16384 11.3, 8.4.
 constexpr int kGradList = 512;
 constexpr int kAhead = 4;
 
@@ -235,7 +236,8 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
     __shared__ T a[TL][TL + 1];      // W[I, J], then G[I, J]
     __shared__ T b[TL][TL + 1];      // W[J, I], then G[J, I]
     __shared__ T dvs[2 * TL];        // w_ii of the rows of I, then of J
-    __shared__ int off[2 * TL + 1];  // first list entry of each row
+    __shared__ int off[2 * TL + 1];  // first entry of each row, all rows' entries in one sequence
+    __shared__ int2 rbd[2 * TL];     // its CSR position, that of its diagonal (-1: none)
     __shared__ int lk[kGradList];    // list: column k, w_ik, the entry's row (0 .. 2 TL - 1)
     __shared__ T lw[kGradList];
     __shared__ unsigned char lr[kGradList];
@@ -271,6 +273,7 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
             cnt = info.y - info.x - (info.z >= 0 ? 1 : 0);
         }
         dvs[threadIdx.x] = dv;
+        rbd[threadIdx.x] = make_int2(info.x, info.z);
         incl = cnt;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -286,22 +289,30 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
         if (w < warp) incl += wsum[w];
         total += wsum[w];
     }
-    const bool listed = total <= kGradList;
     if (threadIdx.x < 2 * TL) {
-        int at = incl - cnt;
-        off[threadIdx.x] = at;
+        off[threadIdx.x] = incl - cnt;
         if (threadIdx.x == 2 * TL - 1) off[2 * TL] = total;
-        if (listed)
-            for (int q = info.x; q < info.y; ++q) {
-                if (q == info.z) continue;
-                lk[at] = om.ci[q];
-                lw[at] = om.cv[q];
-                lr[at] = (unsigned char)threadIdx.x;
-                ++at;
-            }
     }
     __syncthreads();
-    // the group's cursor over the entries of its rows (grp, grp + 256 / PR, ..)
+    // entries w0 .. of the sequence into the list, a thread each
+    int w0 = 0, w1 = min(total, kGradList);
+    auto fill = [&]() {
+        for (int e = w0 + (int)threadIdx.x; e < w1; e += 256) {
+            int lo = 0, hi = 2 * TL - 1;             // the last row that starts at or before e
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (off[mid] <= e) lo = mid; else hi = mid - 1;
+            }
+            int q = rbd[lo].x + e - off[lo];
+            if (rbd[lo].y >= 0 && q >= rbd[lo].y) ++q;
+            lk[e - w0] = om.ci[q];
+            lw[e - w0] = om.cv[q];
+            lr[e - w0] = (unsigned char)lo;
+        }
+    };
+    fill();
+    __syncthreads();
+    // the group's cursor over the listed entries of its rows (grp, grp + 256 / PR, ..)
     const int grp = threadIdx.x / PR, gl = (threadIdx.x % PR) * VW;
     constexpr int NG = 256 / PR;
     int r = grp - NG, t = 0, end = 0;
@@ -309,10 +320,10 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
         while (t == end) {
             r += NG;
             if (r >= 2 * TL) return -1;
-            t = off[r];
-            end = off[r + 1];
+            t = max(off[r], w0);
+            end = max(t, min(off[r + 1], w1));
         }
-        return t++;
+        return t++ - w0;
     };
     auto fetch = [&](int e) -> typename V16::type {
         const T* src = S + (int64_t)lk[e] * lds + (lr[e] < TL ? J0 : I0) + gl;
@@ -325,13 +336,14 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
     };
     int ent[kAhead];
     typename V16::type sv4[kAhead];
-    if (listed) {
+    auto ahead = [&]() {
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
             ent[u] = r < 2 * TL ? next() : -1;
             if (ent[u] >= 0) sv4[u] = fetch(ent[u]);
         }
-    }
+    };
+    ahead();
     // 1. diagonal terms of both tiles from one read of S[I, J]
     if (vload) {
 #pragma unroll
@@ -355,8 +367,8 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
         }
     }
     __syncthreads();
-    // 2. off-diagonal terms of the rows that have them
-    if (listed) {
+    // 2. off-diagonal terms of the rows that have them, a list after another
+    for (;;) {
         while (ent[0] >= 0) {
 #pragma unroll
             for (int u = 0; u < kAhead; ++u) {
@@ -369,19 +381,19 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
 #pragma unroll
                 for (int x = 0; x < VW; ++x) w[x] = fmaT(wk, sv[x], w[x]);
             }
-#pragma unroll
-            for (int u = 0; u < kAhead; ++u) {
-                ent[u] = r < 2 * TL ? next() : -1;
-                if (ent[u] >= 0) sv4[u] = fetch(ent[u]);
-            }
+            ahead();
         }
-    } else {
-        for (int row = warp; row < 2 * TL; row += kW) {
-            if (off[row] == off[row + 1]) continue;
-            const int i = row < TL ? I0 + row : J0 + row - TL;
-            offdiag_row<T, TL>(p, om, rinfo[i], S, lds, row < TL ? J0 : I0, row < TL ? &a[row][0] : &b[row - TL][0]);
-        }
+        if (w1 == total) break;
+        __syncthreads();
+        w0 = w1;
+        w1 = min(total, w0 + kGradList);
+        fill();
+        __syncthreads();
+        r = grp - NG;
+        t = end = 0;
+        ahead();
     }
+    const bool listed = total <= kGradList;
     __syncthreads();
     // 3. symmetrise: G[I, J] and its transpose (a + b = b + a)
 #pragma unroll 4
@@ -408,6 +420,137 @@ k_dense_grad_pair(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __r
             support_terms_row<T, TL>(om, row < TL ? I0 + row : J0 + row - TL, row < TL ? J0 : I0, lam2,
                                      row < TL ? &a[row][0] : &b[row - TL][0]);
         }
+    }
+    __syncthreads();
+    const bool scaled = scale != T(1);
+    if ((vec & 1) && full) {
+        for (int idx = threadIdx.x; idx < TL * PR; idx += 256) {
+            const int y = idx / PR, x = (idx % PR) * VW;
+            T va[VW], vb[VW];
+#pragma unroll
+            for (int k = 0; k < VW; ++k) {
+                va[k] = scaled ? a[y][x + k] * scale : a[y][x + k];
+                vb[k] = scaled ? b[y][x + k] * scale : b[y][x + k];
+            }
+            *reinterpret_cast<typename V16::type*>(G + (int64_t)(I0 + y) * ldg + J0 + x) = V16::make(va);
+            if (!dtile) *reinterpret_cast<typename V16::type*>(G + (int64_t)(J0 + y) * ldg + I0 + x) = V16::make(vb);
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int idx = threadIdx.x + 256 * e, y = idx / TL, x = idx % TL;
+            if (I0 + y < p && J0 + x < p) {
+                const T v = a[y][x];
+                G[(int64_t)(I0 + y) * ldg + J0 + x] = scaled ? v * scale : v;
+            }
+            if (!dtile && J0 + y < p && I0 + x < p) {
+                const T v = b[y][x];
+                G[(int64_t)(J0 + y) * ldg + I0 + x] = scaled ? v * scale : v;
+            }
+        }
+    }
+}
+
+// The same for wide rows: a warp per row with neighbours, without a list.  With many entries in
+// every row the warps have enough of them in flight by themselves, the list's rounds only cost
+// (kGradList entries are a few rows' then), and the room in shared memory is a sixth block per SM.
+// The line, four neighbours per row (FP64: eight), is where a tile pair's rows fill one list.
+// Measured on GB300, ms, list rounds and this: p = 16384, 20 entries a row 5.53, 5.68; p = 4096, 20 a
+// row 0.45, 0.41; 200 a row 7.05, 2.69.
+template <typename T, int TL>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3)
+k_dense_grad_rows(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __restrict__ rdv,
+                  const T* __restrict__ S, int64_t lds, T* __restrict__ G, int64_t ldg, T lam2, T scale, int nt,
+                  int vec /* bit 0: 16-byte G stores; bit 1: 16-byte S loads */) {
+    __shared__ T a[TL][TL + 1];      // W[I, J], then G[I, J]
+    __shared__ T b[TL][TL + 1];      // W[J, I], then G[J, I]
+    __shared__ T dvs[2][TL];         // w_ii of the rows of I and of J
+    __shared__ int imp[2][TL];       // rows of I and of J with off-diagonal entries
+    __shared__ int nimp[2];
+    constexpr int E = TL * TL / 256;
+    int bi, bj;
+    pair_of(blockIdx.x, nt, bi, bj);
+    const int I0 = bi * TL, J0 = bj * TL;
+    const bool dtile = bi == bj;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x < 2) nimp[threadIdx.x] = 0;
+    __syncthreads();
+    if (threadIdx.x < 2 * TL) {
+        const int side = threadIdx.x / TL, yl = threadIdx.x % TL;
+        const int i = (side ? J0 : I0) + yl;
+        T dv = T(0);
+        bool impure = false;
+        if (i < p) {
+            dv = rdv[i];
+            impure = rinfo[i].w == 0;
+        }
+        dvs[side][yl] = dv;
+        if (impure) imp[side][atomicAdd(&nimp[side], 1)] = yl;
+    }
+    __syncthreads();
+    // 1. diagonal terms of both tiles from one read of S[I, J]
+    constexpr int VW = 16 / (int)sizeof(T), PR = TL / VW, EV = TL * PR / 256;   // 16-byte vectors
+    using V16 = Vec16<T>;
+    const bool full = I0 + TL <= p && J0 + TL <= p;
+    if ((vec & 2) && full) {
+        typename V16::type u[EV];
+#pragma unroll
+        for (int e = 0; e < EV; ++e) {           // all the tile's loads in flight before any use
+            const int idx = threadIdx.x + 256 * e, y = idx / PR, x = (idx % PR) * VW;
+            u[e] = *reinterpret_cast<const typename V16::type*>(S + (int64_t)(I0 + y) * lds + J0 + x);
+        }
+#pragma unroll
+        for (int e = 0; e < EV; ++e) {
+            const int idx = threadIdx.x + 256 * e, y = idx / PR, x = (idx % PR) * VW;
+            T sv[VW];
+            V16::unpack(u[e], sv);
+#pragma unroll
+            for (int k = 0; k < VW; ++k) {
+                a[y][x + k] = mulT(dvs[0][y], sv[k]);
+                b[x + k][y] = mulT(dvs[1][x + k], sv[k]);
+            }
+        }
+    } else {
+#pragma unroll 4
+        for (int e = 0; e < E; ++e) {
+            const int idx = threadIdx.x + 256 * e, y = idx / TL, x = idx % TL;
+            const T sv = (I0 + y < p && J0 + x < p) ? S[(int64_t)(I0 + y) * lds + J0 + x] : T(0);
+            a[y][x] = mulT(dvs[0][y], sv);
+            b[x][y] = mulT(dvs[1][x], sv);
+        }
+    }
+    __syncthreads();
+    // 2. off-diagonal terms of the rows that have them
+    const int n0 = nimp[0], n1 = nimp[1];
+    for (int r = warp; r < n0 + n1; r += kW) {
+        const int side = r < n0 ? 0 : 1;
+        const int yl = side ? imp[1][r - n0] : imp[0][r];
+        const int i = (side ? J0 : I0) + yl;
+        offdiag_row<T, TL>(p, om, rinfo[i], S, lds, side ? I0 : J0, side ? &b[yl][0] : &a[yl][0]);
+    }
+    __syncthreads();
+    // 3. symmetrise: G[I, J] in place; G[J, I] is its transpose (a + b = b + a)
+#pragma unroll 4
+    for (int e = 0; e < E; ++e) {
+        const int idx = threadIdx.x + 256 * e, y = idx / TL, x = idx % TL;
+        a[y][x] = T(0.5) * (a[y][x] + b[x][y]);
+    }
+    __syncthreads();
+    if (!dtile) {
+#pragma unroll 4
+        for (int e = 0; e < E; ++e) {
+            const int idx = threadIdx.x + 256 * e, y = idx / TL, x = idx % TL;
+            b[y][x] = a[x][y];
+        }
+        __syncthreads();
+        for (int r = warp; r < n0 + n1; r += kW) {
+            const int side = r < n0 ? 0 : 1;
+            const int yl = side ? imp[1][r - n0] : imp[0][r];
+            support_terms_row<T, TL>(om, (side ? J0 : I0) + yl, side ? I0 : J0, lam2, side ? &b[yl][0] : &a[yl][0]);
+        }
+    } else {
+        // the diagonal tile: every row has its diagonal entry here
+        for (int y = warp; y < TL && I0 + y < p; y += kW) support_terms_row<T, TL>(om, I0 + y, I0, lam2, &a[y][0]);
     }
     __syncthreads();
     const bool scaled = scale != T(1);
@@ -532,6 +675,8 @@ k_support_xy(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __restri
     const int4 info = rinfo[i];
     const T dv = rdv[i];
     for (int64_t m0 = 0; m0 < n; m0 += kXyCols) {
+        // vectors of a thread that hold samples (FP64 products of padding would be the time)
+        const int nu = (int)min((int64_t)U, (n - m0 + kXyT * VW - 1) / (kXyT * VW));
         auto load = [&](int64_t row, typename V16::type (&v)[U]) {
             const T zero[VW] = {};
 #pragma unroll
@@ -546,6 +691,7 @@ k_support_xy(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __restri
             load(i, v);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
+                if (u >= nu) break;
                 V16::unpack(v[u], y[u]);
 #pragma unroll
                 for (int x = 0; x < VW; ++x) y[u][x] = mulT(dv, y[u][x]);
@@ -558,6 +704,7 @@ k_support_xy(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __restri
             load(om.ci[q], v);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
+                if (u >= nu) break;
                 T xv[VW];
                 V16::unpack(v[u], xv);
 #pragma unroll
@@ -572,6 +719,7 @@ k_support_xy(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __restri
                 T s[VW] = {};
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
+                    if (u >= nu) break;
                     T xv[VW];
                     V16::unpack(v[u], xv);
 #pragma unroll
@@ -586,8 +734,8 @@ k_support_xy(int p, Csr<T> om, const int4* __restrict__ rinfo, const T* __restri
             for (int e = warp; e < ne; e += kXyT / 32) {
                 double r = ((double)part[e][lane] + (double)part[e][lane + 32]) +
                            ((double)part[e][lane + 64] + (double)part[e][lane + 96]);
-                r = warp_sum_d(r) / (double)n;
-                if (lane == 0) out[e0 + e] = m0 == 0 ? r : out[e0 + e] + r;
+                r = warp_sum_d(r);
+                if (lane == 0) out[e0 + e] = (m0 == 0 ? 0.0 : out[e0 + e]) + r / (double)n;
             }
             __syncthreads();
         }
@@ -1040,21 +1188,24 @@ static int entry_blocks(int64_t n) { return (int)std::min<int64_t>((n + 255) / 2
 template <typename T>
 void launch_smooth_parts(int p, int64_t nnz, Csr<T> om, const int4* rinfo, const T* rdv, const double* Tv, double* part,
                          double* out3, cudaStream_t s) {
-    const int nb = std::min((p + 255) / 256, 1024);
+    const int nb = entry_blocks(std::max<int64_t>(p, nnz));
     k_smooth_parts<T><<<nb, 256, 0, s>>>(p, nnz, om, rinfo, rdv, Tv, part);
     k_reduce_strided<<<1, 256, 0, s>>>(part, nb, 3, out3);
 }
 
 template <typename T>
-void launch_dense_grad(int p, Csr<T> om, const int4* rinfo, const T* rdv, const T* S, int64_t lds, T* G,
+void launch_dense_grad(int p, int64_t nnz, Csr<T> om, const int4* rinfo, const T* rdv, const T* S, int64_t lds, T* G,
                        int64_t ldg, T lam2, T scale, cudaStream_t s) {
     constexpr int TL = sizeof(T) == 4 ? 64 : 32;      // two tiles: 33 KB (FP32) / 17 KB (FP64) of shared memory
     const int nt = (p + TL - 1) / TL;
     // bit 0: 16-byte stores of G; bit 1: 16-byte loads of S
     const int vec = (((uintptr_t)G % 16 == 0 && (ldg * (int64_t)sizeof(T)) % 16 == 0) ? 1 : 0) |
                     (((uintptr_t)S % 16 == 0 && (lds * (int64_t)sizeof(T)) % 16 == 0) ? 2 : 0);
-    k_dense_grad_pair<T, TL><<<(unsigned)((int64_t)nt * (nt + 1) / 2), 256, 0, s>>>(p, om, rinfo, rdv, S, lds, G,
-                                                                                   ldg, lam2, scale, nt, vec);
+    const unsigned nb = (unsigned)((int64_t)nt * (nt + 1) / 2);
+    if ((nnz - p) * 2 * TL > (int64_t)kGradList * p)
+        k_dense_grad_rows<T, TL><<<nb, 256, 0, s>>>(p, om, rinfo, rdv, S, lds, G, ldg, lam2, scale, nt, vec);
+    else
+        k_dense_grad_pair<T, TL><<<nb, 256, 0, s>>>(p, om, rinfo, rdv, S, lds, G, ldg, lam2, scale, nt, vec);
 }
 
 template <typename T>
@@ -1173,7 +1324,7 @@ cudaError_t launch_cg(int p, int64_t nnz, const int* row, Csr<T> om, const int4*
 }
 
 #define HPC_ADJ_INSTANTIATE(T)                                                                                  \
-    template void launch_dense_grad<T>(int, Csr<T>, const int4*, const T*, const T*, int64_t, T*, int64_t, T, T, \
+    template void launch_dense_grad<T>(int, int64_t, Csr<T>, const int4*, const T*, const T*, int64_t, T*, int64_t, T, T, \
                                        cudaStream_t);                                                           \
     template void launch_spmm_dense<T>(int, Csr<T>, const int4*, const T*, const T*, int64_t, int64_t, T*,      \
                                        int64_t, cudaStream_t);                                                  \

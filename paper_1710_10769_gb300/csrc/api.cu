@@ -2067,7 +2067,7 @@ int backward_t(hpc_ctx* h, const void* X, int xdt, double grad_loss, void* dOmeg
     hpc::Csr<T> om = cur_csr<T>(h);
     hpc::launch_row_info<T>(p, om, h->rinfo, as<T>(h->rdv), h->stream);
     if (dOmega)
-        hpc::launch_dense_grad<T>(p, om, h->rinfo, as<T>(h->rdv), static_cast<const T*>(h->S), h->ld,
+        hpc::launch_dense_grad<T>(p, h->nnz, om, h->rinfo, as<T>(h->rdv), static_cast<const T*>(h->S), h->ld,
                                   static_cast<T*>(dOmega), ld_domega, (T)h->lam2, (T)grad_loss, h->stream);
     if (dX) {
         const size_t plane = align256((size_t)p * n * sizeof(T));

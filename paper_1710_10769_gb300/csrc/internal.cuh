@@ -305,7 +305,7 @@ cudaError_t launch_obs_pairs(int precision, const CUtensorMap* maps, const int2*
 
 // ---------------------------------------------------------------- differentiation (adjoint.cu)
 template <typename T>
-void launch_dense_grad(int p, Csr<T> om, const int4* rinfo, const T* rdv, const T* S, int64_t lds, T* G, int64_t ldg,
+void launch_dense_grad(int p, int64_t nnz, Csr<T> om, const int4* rinfo, const T* rdv, const T* S, int64_t lds, T* G, int64_t ldg,
                        T lam2, T scale, cudaStream_t s);
 template <typename T>
 void launch_spmm_dense(int p, Csr<T> om, const int4* rinfo, const T* rdv, const T* B, int64_t ldb, int64_t m, T* C,
