@@ -76,7 +76,7 @@ struct hpc_ctx {
     int cur = 0;
     int64_t csr_cap = 0;
     int64_t nnz = 0;
-    bool omega_sym = true;          // the iterate equals its transpose, entry by entry
+    bool sym_known = false;         // the device word csr_checks()->symmetric is the iterate's
     // screening output and candidate structure
     int64_t cap = 0;                // emission capacity
     int* em_row = nullptr;
@@ -265,20 +265,35 @@ int grow_csr(hpc_ctx* h, int64_t newcap) {
     return HPC_OK;
 }
 
-// Records whether the iterate is symmetric; the captured loop depends on it (use_loop).
-void set_symmetric(hpc_ctx* h, bool sym) {
-    if (sym != h->omega_sym) h->epoch += 1;
-    h->omega_sym = sym;
+// Device words behind the control block: hpc_set_omega's faults, and whether the current iterate is
+// symmetric (read by the iteration loop).
+hpc::CsrChecks* csr_checks(hpc_ctx* h) { return reinterpret_cast<hpc::CsrChecks*>(h->d_ctrl + 1); }
+
+// Before iterations: the symmetry of an iterate that hpc_set_omega brought, once (queued, not waited for).
+int know_symmetry(hpc_ctx* h) {
+    if (h->sym_known || h->variant != HPC_COV) return HPC_OK;
+    unsigned long long* sym = &csr_checks(h)->symmetric;
+    CUDA_TRY(cudaMemsetAsync(sym, 0xff, sizeof *sym, h->stream));
+    const int c = h->cur;
+    if (h->vdt == HPC_F64)
+        hpc::launch_csr_symmetric<double>({h->rp[c], h->ci[c], static_cast<double*>(h->cv[c])}, h->p, h->nnz, sym, h->stream);
+    else
+        hpc::launch_csr_symmetric<float>({h->rp[c], h->ci[c], static_cast<float*>(h->cv[c])}, h->p, h->nnz, sym, h->stream);
+    CUDA_TRY(cudaGetLastError());
+    h->sym_known = true;
+    return HPC_OK;
 }
 
 int set_identity(hpc_ctx* h) {
     if (h->vdt == HPC_F64)
-        hpc::launch_set_identity<double>({h->rp[h->cur], h->ci[h->cur], as<double>(h->cv[h->cur])}, (int)h->p, h->stream);
+        hpc::launch_set_identity<double>({h->rp[h->cur], h->ci[h->cur], as<double>(h->cv[h->cur])}, (int)h->p,
+                                         &csr_checks(h)->symmetric, h->stream);
     else
-        hpc::launch_set_identity<float>({h->rp[h->cur], h->ci[h->cur], as<float>(h->cv[h->cur])}, (int)h->p, h->stream);
+        hpc::launch_set_identity<float>({h->rp[h->cur], h->ci[h->cur], as<float>(h->cv[h->cur])}, (int)h->p,
+                                        &csr_checks(h)->symmetric, h->stream);
     CUDA_TRY(cudaGetLastError());
     h->nnz = h->p;
-    set_symmetric(h, true);
+    h->sym_known = true;
     return HPC_OK;
 }
 
@@ -303,6 +318,7 @@ hpc::IterBufs<T> bufs(hpc_ctx* h) {
     b.cnt2 = h->cnt2;
     b.scan_part = h->scan_part;
     b.bar = h->bar;
+    b.symmetric = &csr_checks(h)->symmetric;
     b.part_obj = h->part_obj;
     b.part_ls = h->part_ls;
     b.nblk = h->nblk;
@@ -543,6 +559,7 @@ int one_iteration(hpc_ctx* h, hpc_stats* st, bool use_stop, bool* done) {
 // Reset the counters of the control block and load the solve's parameters
 // (lambda, iteration limit, stopping rule) into it.
 int load_ctrl(hpc_ctx* h, int64_t k, bool use_stop) {
+    STATUS_TRY(know_symmetry(h));
     hpc::Ctrl& c = *h->h_ctrl;
     c.iter = 0;
     c.ls_trials = 0;
@@ -668,9 +685,7 @@ int tail_mode(const hpc_ctx* h) { return h->tune.fused_tail != 0 && tail_in_grap
 // Whether the handle's iterations run in the one-launch loop (loop.cu): the Cov
 // variant with the tail form left to the library (fused_tail 0), on a device that runs
 // cooperative kernels in graph loops, from kLoopMinRows rows on.  Allocates the loop's
-// workspace at the first call.  An iterate that is not symmetric (hpc_set_omega takes any) stays
-// with the chain, which removes the duplicates that it gives in a row's candidates; the loop's
-// buckets hold a column once.  It is the faster form at every size (us per iteration on
+// workspace at the first call.  It is the faster form at every size (us per iteration on
 // GB300, chain -> loop: 110 -> 37 at p = 64, 114 -> 38 at p = 256, 106 -> 35 at p = 512,
 // FP64 223 -> 66 at p = 384); below kLoopMinRows the chain stays all the same, because its
 // statistics are part of what callers of small problems check: hpc_stats.kernel_launches
@@ -682,7 +697,7 @@ constexpr int64_t kLoopMinRows = sizeof(T) == 8 ? 224 : 384;
 template <typename T>
 int use_loop(hpc_ctx* h, bool* yes) {
     *yes = false;
-    if (h->variant != HPC_COV || h->tune.fused_tail != 0 || h->chain_only || !h->omega_sym || h->p < kLoopMinRows<T> ||
+    if (h->variant != HPC_COV || h->tune.fused_tail != 0 || h->chain_only || h->p < kLoopMinRows<T> ||
         h->p >= (1ll << 28) || !tail_in_graph_supported(h))
         return HPC_OK;
     if (h->loop_ok < 0) {
@@ -1604,14 +1619,14 @@ int hpc_get_omega(hpc_handle h, int64_t* nnz_inout, int64_t* row_ptr, int32_t* c
 // streams that may still be writing the arrays, as the copies did.
 static int set_omega_device(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32_t* col, const void* val,
                             hpc_dtype vdt) {
-    hpc::CsrChecks* d_chk = reinterpret_cast<hpc::CsrChecks*>(h->d_ctrl + 1);
-    hpc::CsrChecks chk;
-    CUDA_TRY(cudaMemsetAsync(d_chk, 0xff, sizeof chk, cudaStreamLegacy));
-    hpc::launch_csr_check(row_ptr, col, val, vdt, h->vdt, h->p, nnz, d_chk, cudaStreamLegacy);
+    unsigned long long* d_key = &csr_checks(h)->key;
+    unsigned long long key = ~0ull;
+    CUDA_TRY(cudaMemsetAsync(d_key, 0xff, sizeof key, cudaStreamLegacy));
+    hpc::launch_csr_check(row_ptr, col, val, vdt, h->p, nnz, d_key, cudaStreamLegacy);
     CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaMemcpy(&chk, d_chk, sizeof chk, cudaMemcpyDeviceToHost));
-    if (chk.key != ~0ull) {
-        const unsigned fault = (unsigned)chk.key & 3u;
+    CUDA_TRY(cudaMemcpy(&key, d_key, sizeof key, cudaMemcpyDeviceToHost));
+    if (key != ~0ull) {
+        const unsigned fault = (unsigned)key & 3u;
         return fault == hpc::kCsrBadArg ? HPC_ERR_ARG : fault == hpc::kCsrBadDiag ? HPC_ERR_NONPOS_DIAG : HPC_ERR_NAN;
     }
     if (nnz > h->csr_cap) STATUS_TRY(grow_csr(h, 2 * nnz));
@@ -1625,44 +1640,24 @@ static int set_omega_device(hpc_handle h, int64_t nnz, const int64_t* row_ptr, c
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     h->nnz = nnz;
-    set_symmetric(h, chk.symmetric != 0);
+    h->sym_known = false;
     return HPC_OK;
 }
 
-int hpc_set_omega(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32_t* col, const void* val,
-                  hpc_dtype vdt, int on_device) {
-    if (!h || !row_ptr || !col || !val || nnz < h->p || (vdt != HPC_F32 && vdt != HPC_F64)) return HPC_ERR_ARG;
+static int set_omega_host(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32_t* col, const void* val,
+                          hpc_dtype vdt) {
     const int64_t p = h->p;
-    const size_t vs = dtype_size(vdt);
-    if (on_device && hpc::device_readable(row_ptr, (p + 1) * sizeof(int64_t), sizeof(int64_t)) &&
-        hpc::device_readable(col, nnz * sizeof(int32_t), sizeof(int32_t)) && hpc::device_readable(val, nnz * vs, vs))
-        return set_omega_device(h, nnz, row_ptr, col, val, vdt);
     std::vector<int64_t> rp(p + 1);
     std::vector<int32_t> ci(nnz);
     std::vector<double> v(nnz);
-    // other device addresses come by copies, which refuse what the device does not hold
-    const auto fetch = [&](void* dst, const void* src, size_t bytes) {
-        if (on_device) {
-            const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyDeviceToHost);
-            if (e != cudaSuccess) (void)cudaGetLastError();
-            return e;
-        }
-        std::memcpy(dst, src, bytes);
-        return cudaSuccess;
-    };
-    CUDA_TRY(fetch(rp.data(), row_ptr, (p + 1) * sizeof(int64_t)));
-    CUDA_TRY(fetch(ci.data(), col, nnz * sizeof(int32_t)));
-    if (vdt == HPC_F64) {
-        CUDA_TRY(fetch(v.data(), val, nnz * sizeof(double)));
-    } else {
-        std::vector<float> f(nnz);
-        CUDA_TRY(fetch(f.data(), val, nnz * sizeof(float)));
-        for (int64_t t = 0; t < nnz; ++t) v[t] = f[t];
-    }
+    std::memcpy(rp.data(), row_ptr, (p + 1) * sizeof(int64_t));
+    std::memcpy(ci.data(), col, nnz * sizeof(int32_t));
+    if (vdt == HPC_F64) std::memcpy(v.data(), val, nnz * sizeof(double));
+    else for (int64_t t = 0; t < nnz; ++t) v[t] = static_cast<const float*>(val)[t];
     // validate: row_ptr monotone, columns sorted and in range, positive diagonal present
     if (rp[0] != 0 || rp[p] != nnz) return HPC_ERR_ARG;
     for (int64_t i = 0; i < p; ++i) {
-        if (rp[i + 1] < rp[i]) return HPC_ERR_ARG;
+        if (rp[i + 1] < rp[i] || rp[i + 1] > nnz) return HPC_ERR_ARG;
         bool diag = false;
         for (int64_t t = rp[i]; t < rp[i + 1]; ++t) {
             if (ci[t] < 0 || ci[t] >= p) return HPC_ERR_ARG;
@@ -1691,16 +1686,28 @@ int hpc_set_omega(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32
         CUDA_TRY(cudaStreamSynchronize(h->stream));
     }
     h->nnz = nnz;
-    // the same comparison that device arrays get
-    hpc::CsrChecks* d_chk = reinterpret_cast<hpc::CsrChecks*>(h->d_ctrl + 1);
-    hpc::CsrChecks chk;
-    CUDA_TRY(cudaMemsetAsync(d_chk, 0xff, sizeof chk, h->stream));
-    hpc::launch_csr_symmetric(h->rp[c], h->ci[c], h->cv[c], h->vdt, p, nnz, d_chk, h->stream);
-    CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaMemcpyAsync(&chk, d_chk, sizeof chk, cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
-    set_symmetric(h, chk.symmetric != 0);
+    h->sym_known = false;
     return HPC_OK;
+}
+
+int hpc_set_omega(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32_t* col, const void* val,
+                  hpc_dtype vdt, int on_device) {
+    if (!h || !row_ptr || !col || !val || nnz < h->p || (vdt != HPC_F32 && vdt != HPC_F64)) return HPC_ERR_ARG;
+    if (!on_device) return set_omega_host(h, nnz, row_ptr, col, val, vdt);
+    const size_t b_rp = (h->p + 1) * sizeof(int64_t), b_ci = nnz * sizeof(int32_t), b_v = nnz * dtype_size(vdt);
+    if (hpc::device_readable(row_ptr, b_rp, sizeof(int64_t)) && hpc::device_readable(col, b_ci, sizeof(int32_t)) &&
+        hpc::device_readable(val, b_v, dtype_size(vdt)))
+        return set_omega_device(h, nnz, row_ptr, col, val, vdt);
+    // other addresses by copies, which refuse what the device does not hold
+    std::vector<int64_t> rp(h->p + 1);
+    std::vector<int32_t> ci(nnz);
+    std::vector<uint8_t> v(b_v);
+    cudaError_t e = cudaMemcpy(rp.data(), row_ptr, b_rp, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(ci.data(), col, b_ci, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(v.data(), val, b_v, cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    CUDA_TRY(e);
+    return set_omega_host(h, nnz, rp.data(), ci.data(), v.data(), vdt);
 }
 
 }  // extern "C"

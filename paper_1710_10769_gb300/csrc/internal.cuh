@@ -165,6 +165,7 @@ struct IterBufs {
     int64_t ldx;
     int64_t n;
     unsigned* bar;            // kBarWords: arrival counter of the fused tail's grid barriers
+    const unsigned long long* symmetric;      // CsrChecks::symmetric
 };
 
 // Device-side loop control (CUDA graph conditional nodes); use = 0 outside a graph.
@@ -196,23 +197,21 @@ template <typename T> void launch_grad_screen(const IterBufs<T>& b, cudaStream_t
 template <typename T> void launch_candidates(const IterBufs<T>& b, cudaStream_t s);
 template <typename T> void launch_ls_window(const IterBufs<T>& b, const LoopCond& lc, cudaStream_t s);
 template <typename T> void launch_accept(const IterBufs<T>& b, cudaStream_t s);
-template <typename T> void launch_set_identity(Csr<T> c, int p, cudaStream_t s);
+template <typename T> void launch_set_identity(Csr<T> c, int p, unsigned long long* symmetric, cudaStream_t s);
 template <typename T> void launch_csr_export(const int* rp, const int* ci, const T* cv, int p, int nnz,
                                              int64_t* rp64, int32_t* ci_out, void* val, int vdt,
                                              cudaStream_t s);
 enum : unsigned { kCsrBadArg = 1, kCsrBadDiag = 2, kCsrNotFinite = 3 };
-// Their outcome; all bits are set before a launch.
+// Outcomes of the checks of an iterate; all bits of a word are set before its check.
 struct CsrChecks {
     unsigned long long key;         // the first fault in row order
     unsigned long long symmetric;   // 0: some entry (i, j) has no equal entry (j, i)
 };
 static_assert(sizeof(Ctrl) % 8 == 0, "CsrChecks lies behind the control block");
-// The faults, and the symmetry of the entries as values of type out_dt.
-void launch_csr_check(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int out_dt, int64_t p, int64_t nnz,
-                      CsrChecks* out, cudaStream_t s);
-// The symmetry alone, of a handle's arrays.
-void launch_csr_symmetric(const int* rp, const int* ci, const void* v, int vdt, int64_t p, int64_t nnz, CsrChecks* out,
-                          cudaStream_t s);
+void launch_csr_check(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int64_t p, int64_t nnz,
+                      unsigned long long* key, cudaStream_t s);
+template <typename T>
+void launch_csr_symmetric(Csr<T> c, int64_t p, int64_t nnz, unsigned long long* symmetric, cudaStream_t s);
 template <typename T>
 void launch_csr_import(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int64_t p, int64_t nnz, Csr<T> out,
                        cudaStream_t s);

@@ -2296,7 +2296,8 @@ k_compact_write(int p, Buckets<T> bk, Csr<T> nx, int cap, const Ctrl* ctrl) {
 }
 
 template <typename T>
-__global__ void k_set_identity(Csr<T> c, int p) {
+__global__ void k_set_identity(Csr<T> c, int p, unsigned long long* symmetric) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *symmetric = ~0ull;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= p; i += gridDim.x * blockDim.x) {
         c.rp[i] = i;
         if (i < p) { c.ci[i] = i; c.cv[i] = T(1); }
@@ -2314,64 +2315,57 @@ __global__ void k_csr_export(const int* rp, const int* ci, const T* cv, int p, i
 
 // The checks of hpc_set_omega on a device CSR: the smallest key of a fault, row in the high half,
 // then the place in the row (0: its bounds; 1 + t: entry t; the largest: no diagonal), then the
-// fault, so that the fault reported is the first one in row order.  Rows whose bounds leave
-// 0 .. nnz are not read.  Thread per row.
+// fault, so that the fault reported is the first one in row order.  Nothing outside of 0 .. nnz is
+// read: rows whose bounds leave it are not, and of a row with more than p + 1 entries, which
+// has a fault among those, no more.  Warp per row (a thread per row took 0.9 ms for a row of 8000).
 template <typename V>
 __global__ void __launch_bounds__(256) k_csr_check(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                                    const V* __restrict__ v, int64_t p, int64_t nnz,
                                                    unsigned long long* key) {
-    const int64_t i = blockIdx.x * 256ll + threadIdx.x;
-    if (i >= p) return;
-    unsigned place = 0, fault = 0;
-    const int64_t a = rp[i], b = rp[i + 1];
-    if (i == 0 && (a != 0 || rp[p] != nnz)) {
-        fault = kCsrBadArg;
-    } else if (b < a || a < 0 || b > nnz) {
-        fault = kCsrBadArg;
-    } else {
-        bool diag = false;
-        int64_t last = -1;
-        for (int64_t t = a; t < b && !fault; ++t) {
-            const int64_t c = ci[t];
-            const V x = v[t];
-            place = 1u + (unsigned)min(t - a, (int64_t)0x1ffffffd);
-            if (c < 0 || c >= p || (t > a && c <= last)) fault = kCsrBadArg;
-            else if (c == i && !(x > V(0))) fault = kCsrBadDiag;
-            else if (!isfinite(x)) fault = kCsrNotFinite;
-            diag = diag || c == i;
-            last = c;
-        }
-        if (!fault && !diag) {
-            place = 0x1fffffffu;
-            fault = kCsrBadDiag;
-        }
-    }
-    if (fault) atomicMin(key, (unsigned long long)i << 32 | (unsigned long long)(place << 2 | fault));
-}
-
-// Whether every entry (i, j) has an equal entry (j, i), as values of type T: a warp per row, the
-// transpose by binary search in its column's row.  rp and ci may still hold faults: nothing
-// outside of 0 .. nnz is read, columns outside of 0 .. p - 1 are left out.
-template <typename T, typename I, typename V>
-__global__ void __launch_bounds__(256) k_csr_symmetric(const I* __restrict__ rp, const int32_t* __restrict__ ci,
-                                                       const V* __restrict__ v, int64_t p, int64_t nnz,
-                                                       unsigned long long* symmetric) {
     const int lane = threadIdx.x & 31;
     const int64_t i = blockIdx.x * 8ll + (threadIdx.x >> 5);
     if (i >= p) return;
-    const int64_t a = max((int64_t)0, (int64_t)rp[i]), b = min(nnz, (int64_t)rp[i + 1]);
-    if (b - a > p) return;                  // a fault: k_csr_check's finding
+    auto report = [&](unsigned place, unsigned fault) {
+        atomicMin(key, (unsigned long long)i << 32 | (unsigned long long)(place << 2 | fault));
+    };
+    const int64_t a = rp[i], b = rp[i + 1];
+    if ((i == 0 && (a != 0 || rp[p] != nnz)) || b < a || a < 0 || b > nnz) {
+        if (lane == 0) report(0u, kCsrBadArg);
+        return;
+    }
+    bool diag = false;
+    for (int64_t t = a + lane; t < min(b, a + p + 1); t += 32) {
+        const int64_t c = ci[t];
+        const V x = v[t];
+        unsigned fault = 0;
+        if (c < 0 || c >= p || (t > a && c <= ci[t - 1])) fault = kCsrBadArg;
+        else if (c == i && !(x > V(0))) fault = kCsrBadDiag;
+        else if (!isfinite(x)) fault = kCsrNotFinite;
+        if (fault) report(1u + (unsigned)min(t - a, (int64_t)0x1ffffffd), fault);
+        diag |= c == i;
+    }
+    if (!__any_sync(kFull, diag) && lane == 0) report(0x1fffffffu, kCsrBadDiag);
+}
+
+// Whether every entry (i, j) has an equal entry (j, i): a thread per entry, its row and its transpose by
+// binary searches.
+template <typename T>
+__global__ void __launch_bounds__(256) k_csr_symmetric(Csr<T> c, int p, int64_t nnz, unsigned long long* symmetric) {
     bool bad = false;
-    for (int64_t q = a + lane; q < b; q += 32) {
-        const int64_t j = ci[q];
-        if (j < 0 || j >= p) continue;
-        int64_t lo = max((int64_t)0, (int64_t)rp[j]), hi = min(nnz, (int64_t)rp[j + 1]);
-        const int64_t end = hi;
-        while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (ci[mid] < i) lo = mid + 1; else hi = mid;
+    for (int64_t q = blockIdx.x * 256ll + threadIdx.x; q < nnz; q += gridDim.x * 256ll) {
+        const int j = c.ci[q];
+        int i = 0, last = p - 1;                 // the last row that starts at or before q
+        while (i < last) {
+            const int mid = (int)(((long long)i + last + 1) >> 1);
+            if (c.rp[mid] <= q) i = mid; else last = mid - 1;
         }
-        bad |= !(lo < end && ci[lo] == i && (T)v[lo] == (T)v[q]);
+        int lo = c.rp[j], hi = c.rp[j + 1];
+        const int end = hi;
+        while (lo < hi) {
+            const int mid = (int)(((long long)lo + hi) >> 1);
+            if (c.ci[mid] < i) lo = mid + 1; else hi = mid;
+        }
+        bad |= !(lo < end && c.ci[lo] == i && c.cv[lo] == c.cv[q]);
     }
     if (bad) *symmetric = 0;
 }
@@ -2979,8 +2973,8 @@ void launch_point_end(const IterBufs<T>& b, PathOut out, cudaGraphConditionalHan
 }
 
 template <typename T>
-void launch_set_identity(Csr<T> c, int p, cudaStream_t s) {
-    k_set_identity<T><<<64, 256, 0, s>>>(c, p);
+void launch_set_identity(Csr<T> c, int p, unsigned long long* symmetric, cudaStream_t s) {
+    k_set_identity<T><<<64, 256, 0, s>>>(c, p, symmetric);
 }
 
 template <typename T>
@@ -2992,28 +2986,16 @@ void launch_csr_export(const int* rp, const int* ci, const T* cv, int p, int nnz
         k_csr_export<T, float><<<256, 256, 0, s>>>(rp, ci, cv, p, nnz, rp64, co, static_cast<float*>(val));
 }
 
-template <typename V>
-static void csr_check(const int64_t* rp, const int32_t* ci, const V* v, int out_dt, int64_t p, int64_t nnz,
-                      CsrChecks* out, cudaStream_t s) {
-    k_csr_check<V><<<(unsigned)((p + 255) / 256), 256, 0, s>>>(rp, ci, v, p, nnz, &out->key);
+void launch_csr_check(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int64_t p, int64_t nnz,
+                      unsigned long long* key, cudaStream_t s) {
     const unsigned nb = (unsigned)((p + 7) / 8);
-    if (out_dt == HPC_F64) k_csr_symmetric<double><<<nb, 256, 0, s>>>(rp, ci, v, p, nnz, &out->symmetric);
-    else k_csr_symmetric<float><<<nb, 256, 0, s>>>(rp, ci, v, p, nnz, &out->symmetric);
+    if (vdt == HPC_F64) k_csr_check<double><<<nb, 256, 0, s>>>(rp, ci, static_cast<const double*>(v), p, nnz, key);
+    else k_csr_check<float><<<nb, 256, 0, s>>>(rp, ci, static_cast<const float*>(v), p, nnz, key);
 }
 
-void launch_csr_check(const int64_t* rp, const int32_t* ci, const void* v, int vdt, int out_dt, int64_t p, int64_t nnz,
-                      CsrChecks* out, cudaStream_t s) {
-    if (vdt == HPC_F64) csr_check(rp, ci, static_cast<const double*>(v), out_dt, p, nnz, out, s);
-    else csr_check(rp, ci, static_cast<const float*>(v), out_dt, p, nnz, out, s);
-}
-
-void launch_csr_symmetric(const int* rp, const int* ci, const void* v, int vdt, int64_t p, int64_t nnz, CsrChecks* out,
-                          cudaStream_t s) {
-    const unsigned nb = (unsigned)((p + 7) / 8);
-    if (vdt == HPC_F64)
-        k_csr_symmetric<double><<<nb, 256, 0, s>>>(rp, ci, static_cast<const double*>(v), p, nnz, &out->symmetric);
-    else
-        k_csr_symmetric<float><<<nb, 256, 0, s>>>(rp, ci, static_cast<const float*>(v), p, nnz, &out->symmetric);
+template <typename T>
+void launch_csr_symmetric(Csr<T> c, int64_t p, int64_t nnz, unsigned long long* symmetric, cudaStream_t s) {
+    k_csr_symmetric<T><<<(unsigned)std::min<int64_t>((nnz + 255) / 256, 4096), 256, 0, s>>>(c, (int)p, nnz, symmetric);
 }
 
 template <typename T>
@@ -3041,12 +3023,13 @@ void launch_gather_s(const void* S, int is_f64, int64_t ld, int64_t m, const int
     template void launch_accept<T>(const IterBufs<T>&, cudaStream_t);                              \
     template cudaError_t launch_tail<T>(const IterBufs<T>&, bool, cudaStream_t);                     \
     template int tail_grid<T>(const IterBufs<T>&, bool);                                             \
-    template void launch_set_identity<T>(Csr<T>, int, cudaStream_t);                               \
+    template void launch_set_identity<T>(Csr<T>, int, unsigned long long*, cudaStream_t);          \
     template void launch_row_info<T>(int, Csr<T>, int4*, T*, cudaStream_t);                        \
     template void launch_rowblock_max<T>(const T*, int64_t, int, int, unsigned short*, cudaStream_t); \
     template int screen_plan<T>(int, int, std::vector<long long>&);                                 \
     template void launch_csr_import<T>(const int64_t*, const int32_t*, const void*, int, int64_t, int64_t, Csr<T>, \
                                        cudaStream_t);                                              \
+    template void launch_csr_symmetric<T>(Csr<T>, int64_t, int64_t, unsigned long long*, cudaStream_t);        \
     template void launch_csr_export<T>(const int*, const int*, const T*, int, int, int64_t*, int32_t*, \
                                        void*, int, cudaStream_t);
 

@@ -56,7 +56,9 @@
 // that the chain does faster (dense iterates and hub rows, see in_debt) ends the launch with
 // Ctrl::loop_full set and the iterate unchanged; the chain of kernels then runs the next
 // iterations (one at first, twice as many after every further end of this kind) before the loop
-// tries again.  No phase of a launch is long, then, which the bounded waits need.
+// tries again.  An iterate that is not symmetric (hpc_set_omega takes any) is the chain's
+// altogether: a column could come twice into a row's bucket, and the chain removes such duplicates.
+// No phase of a launch is long, then, which the bounded waits need.
 //
 // Measured on GB300 (us per iteration, the chain of kernels -> this loop): 140 -> 46 at
 // p = 65536 (n = 32768), 120 -> 43 at p = 16384, 98 -> 30 at p = 1001, 220 -> 50 in FP64 at
@@ -163,6 +165,7 @@ struct LoopK {
     const unsigned short* m1;    // block maxima (null: no bounds)
     const unsigned short* m1g;   // group maxima (null: none)
     int nbm, ngl;
+    const unsigned long long* symmetric;     // 0: the iterate is not
     int use_cond;
     cudaGraphConditionalHandle chain_cond;   // set to 1 where the chain has to run next
     cudaGraphConditionalHandle outer_cond;   // the loop over both: ends here unless the chain runs
@@ -929,6 +932,20 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
     int last_h = 0;
     if (tid == 0) { sm.flags = 0; sm.full = 0; sm.accept = -1; sm.converged = 0; sm.n2 = 0.0; sm.nlong = 0; sm.nhuge = 0; sm.ni = 0; sm.npl = 0; sm.sup = 0; sm.units = 0; }
     __syncthreads();
+
+    if (*k.symmetric == 0ull) {
+        // all of the solve is the chain's
+        if (bid == 0 && tid == 0) {
+            ctrl->loop_launches += 1;
+            ctrl->loop_full = 1;
+            ctrl->chain_left = 0x7fffffff;
+            if (k.use_cond) {
+                cudaGraphSetConditional(k.chain_cond, 1u);
+                cudaGraphSetConditional(k.outer_cond, 1u);
+            }
+        }
+        return;
+    }
 
     // ---------------- set-up of the owned rows from the current iterate
     for (int r = tid; r < nr; r += kLT) {
@@ -1794,6 +1811,7 @@ LoopK<T> loop_args(const IterBufs<T>& b, void* ws, int R, size_t* bytes) {
     k.m1g = b.m1 ? b.m1g : nullptr;
     k.nbm = b.nbm;
     k.ngl = b.ngl;
+    k.symmetric = b.symmetric;
     uint8_t* q = static_cast<uint8_t*>(ws);
     auto take = [&](size_t n) { uint8_t* r = q; q += align256(n); return r; };
     const size_t p = (size_t)b.p;
