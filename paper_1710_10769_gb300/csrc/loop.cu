@@ -831,18 +831,18 @@ __device__ __forceinline__ float warp_sum_up(float x) {
 //              nbm (nnz - p), where the iterate is dense: level at half of them;
 //   support    W_ij and W_ji by gathers, up to 1.3 us per 1000 of sum n_i^2 over the rows of
 //              the block that has most, as 6 terms each: a quarter of the chain's terms;
-//   search     1 us per pair of 32-entry chunks of a block's rows: level at about 400.
+//   search     1 us per pair of 32-entry chunks of a block's rows: level at about 500.
 // A pass that loses may be worth it (bounds that start anew keep more blocks than they do a pass
 // later, if the rows are short), so the losses add up to a debt, and the loop leaves when that
-// passes half of the chain's terms.  Without bounds there is nothing to wait for.
+// passes what a pass over all blocks loses.  Without bounds there is nothing to wait for.
 // us of the chain and of the loop per iteration, without the rule: p = 8192, n = 1000, lambda1 = 0.07
 // (130 entries a row) 8200, 18300; p = 2000, 90 entries a row 640, 1080; a hub row of 700
 // entries at p = 700 430, 710.
 // Terms are counted by 1024 here.
 constexpr unsigned kWorkEven = 512, kWorkBlind = 1370, kSupEven = 340;
-constexpr unsigned kDebtLeast = 256, kDebtMost = 32768;
+constexpr unsigned kDebtLeast = 256, kDebtMost = 1u << 16;
 constexpr int kShortMean = 32;
-constexpr int kUnitsMax = 400;
+constexpr int kUnitsMax = 512;
 constexpr int kTasksFew = 1 << 16, kHeavyFew = 256, kSupFew = 900;
 __device__ __forceinline__ int row_units(int entries) {
     const int c = (entries + 31) >> 5;
@@ -854,7 +854,7 @@ __device__ __forceinline__ unsigned chain_terms(int nnz, int nbm, int p) {
 }
 // One more pass that does `work` where both forms are level at `even`; whether to leave before it.
 __device__ __forceinline__ bool in_debt(unsigned& debt, unsigned work, unsigned even, unsigned credit) {
-    debt = work > even ? debt + (work - even) : debt - min(debt, kWorkEven / 2);
+    debt = work > even ? debt + (work - even) : debt - min(debt, even - work);
     return debt > min(kDebtLeast + credit, kDebtMost);
 }
 __device__ __forceinline__ bool support_debt(unsigned& debt, int sup, int nnz, int nbm, int p) {
@@ -866,10 +866,10 @@ __device__ __forceinline__ bool support_debt(unsigned& debt, int sup, int nnz, i
 // arithmetic in line every pass took 2 us longer (47.8 -> 50.5 us at p = 400).
 template <typename T>
 __device__ __noinline__ bool leave_tasks(LoopSmem<T>& sm, unsigned long long terms64, int nnz, int nbm, int p) {
-    const unsigned chain = chain_terms(nnz, nbm, p);
+    const unsigned chain = chain_terms(nnz, nbm, p), all = chain_terms(nnz, nbm, 0);
     if (threadIdx.x == 0)
         sm.leave[1] = in_debt(sm.debt, (unsigned)(terms64 >> 4), kWorkEven + chain / 2,
-                              nnz / kShortMean < p ? chain / 2 : 0u);
+                              nnz / kShortMean < p ? all - chain / 2 : 0u);
     __syncthreads();
     return sm.leave[1] != 0;
 }
@@ -1023,6 +1023,11 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         }
         alive = loop_barrier(k.bar, target, ctrl, &sm.ok);
     }
+    if (alive && k.bnd && !dense) {
+        const ulonglong2 todo = __ldcg(k.todo + par);
+        if ((int)todo.x > kTasksFew || (int)todo.y > kHeavyFew)
+            dense = leave_tasks(sm, (todo.x >> 32) + (todo.y >> 32), nnz_now, k.nbm, k.p);
+    }
     bool run = alive && iter < iter_limit;
 
     while (run) {
@@ -1041,7 +1046,8 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
             const ulonglong2 todo = k.bnd ? __ldcg(k.todo + par) : make_ulonglong2(0, 0);
             const int nt = (int)todo.x, nh = (int)todo.y;
             // the same in every block: the pass is left to the chain before its tasks
-            if (nt > kTasksFew || nh > kHeavyFew) dense = leave_tasks(sm, (todo.x >> 32) + (todo.y >> 32), nnz_now, k.nbm, k.p);
+            if (attempts > 0 && (nt > kTasksFew || nh > kHeavyFew))
+                dense = leave_tasks(sm, (todo.x >> 32) + (todo.y >> 32), nnz_now, k.nbm, k.p);
             if (dense) break;
             const bool all = !k.bnd || nt > k.ntask_cap - nh || nt < 0 || nh < 0;
             const int* list = k.tasks + (size_t)par * k.ntask_cap;
@@ -1805,6 +1811,7 @@ LoopK<T> loop_args(const IterBufs<T>& b, void* ws, int R, size_t* bytes) {
     k.rds = b.rdv;
     k.bar = b.bar;
     k.ctrl = b.ctrl;
+    k.symmetric = b.symmetric;
     k.eps = b.eps;
     k.max_halvings = b.max_halvings;
     k.m1 = b.m1;
