@@ -89,7 +89,7 @@ constexpr int kHeavyTerms = 32;          // rows with more terms are screened by
 constexpr int kQA = 3 * kWin;            // accumulated partials per window: quadratic form, ||D||^2, phi
 constexpr int kQI = 2 * kWin;            // counted partials per window: w+_ii <= 0, entries kept
 constexpr int kNA = 2 * kQA + 1;         // and ||Omega||^2
-constexpr int kNI = 2 * kQI + 5;         // and entries emitted, NaN / Inf, full rows, Hits::halves, rows with neighbours
+constexpr int kNI = 2 * kQI + 5;         // and entries emitted, NaN / Inf, full rows, LoopSmem::halves, off
 
 constexpr unsigned kColMask = 0x0fffffffu;
 constexpr unsigned kFSupp = 0x80000000u;
@@ -192,6 +192,8 @@ struct LoopSmem {
     int sup;                            // sum of n_i^2 / 64 over the owned rows of n_i entries
     unsigned debt, sup_debt;            // in_debt's; one thread's
     int leave[2];                       // outcomes of leave_support and leave_tasks
+    int halves;                         // pairs of rows with the diagonal alone that have one entry above lambda1
+    int off;                            // owned rows with neighbours
     int units;                          // pairs of 32-entry chunks of the rows with more than 32 candidates
     // the decision, the same in every block
     int flags, accept, nnz, nnz_pre, more, converged, full;
@@ -319,7 +321,7 @@ struct Hits {
     T* w;
     int n;        // the same in every lane
     int emitted;  // per lane: entries with |W_ij| > lambda1 or in the support
-    int halves;   // pairs of rows with the diagonal alone where one of the two entries is
+    int* halves;  // LoopSmem's
 
     __device__ __forceinline__ void flush(const LoopK<T>& k, const Csr<T>& csr, T lam1, T lam2, int lane) {
         __syncwarp();
@@ -334,7 +336,7 @@ struct Hits {
             const bool both = __ldcg(k.rds + row) > T(0) && __ldcg(k.rds + col) > T(0);
             const bool other = !(fabs(wji) <= lam1);
             emitted += both ? (first_meets ? 1 + other : 0) : 1;
-            halves += both && first_meets && !other;
+            if (both && first_meets && !other) atomicAdd(halves, 1);
             if (first_meets) {
                 const T g = gradient_of(wij, wji, T(0), lam2, false);
                 if (!(fabs(g) <= lam1)) {
@@ -930,7 +932,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
     int pbuf = 0;                      // partial buffer
     int buf = 0;                       // CSR buffer of the current iterate: 0 cur, 1 next
     int last_h = 0;
-    if (tid == 0) { sm.flags = 0; sm.full = 0; sm.accept = -1; sm.converged = 0; sm.n2 = 0.0; sm.nlong = 0; sm.nhuge = 0; sm.ni = 0; sm.npl = 0; sm.sup = 0; sm.units = 0; }
+    if (tid == 0) { sm.flags = 0; sm.full = 0; sm.accept = -1; sm.converged = 0; sm.n2 = 0.0; sm.nlong = 0; sm.nhuge = 0; sm.ni = 0; sm.npl = 0; sm.sup = 0; sm.units = 0; sm.halves = 0; sm.off = 0; }
     __syncthreads();
 
     if (*k.symmetric == 0ull) {
@@ -969,6 +971,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         s_mv[r] = 0;
         if (!pure) {
             s_list[atomicAdd(&sm.nlong, 1)] = r;
+            atomicAdd(&sm.off, 1);
             atomicAdd(&sm.sup, row_sup(re - rb));
             const int at = atomicAdd(&sm.ni, re - rb);
             for (int q = rb; q < re; ++q)
@@ -1038,7 +1041,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         const long long t_scr = tid == 0 && bid == 0 ? tail_clock_ns() : 0;
         // ---------------- screen
         if (bid == 0 && tid == 0) k.ctr[kCtrBig] = 0;
-        Hits<T> hits{sm.hit_i[warp], sm.hit_j[warp], sm.hit_w[warp], 0, 0, 0};
+        Hits<T> hits{sm.hit_i[warp], sm.hit_j[warp], sm.hit_w[warp], 0, 0, &sm.halves};
         // the owned rows' support entries, then a share of the (row, block) tasks
         if (sm.sup < kSupFew || !leave_support(sm, k.ctr + kCtrFull, nnz_now, k.nbm, k.p))
             screen_support(k, om, i0, nr, sm.items, sm.item_r, sm.ni, s_rb, s_rc, sm.e0, sm.e1, lam2, hits.emitted);
@@ -1079,7 +1082,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         if (dense) break;
         ++attempts;
         const bool pool_full = sm.pool_full != 0;
-        int em = hits.emitted, bad = 0, full = 0, off = 0;
+        int em = hits.emitted, bad = 0, full = 0;
         A o2{};
         // the rows with candidates beside the diagonal, in row order (the sums below follow it)
         for (int r0 = 0; r0 < nr; r0 += kLT) {
@@ -1090,7 +1093,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
                 const bool pure = s_rc[r] < 0;
                 const T dv = s_dv[r];
                 s_om[r] = dv;
-                if (pure) ++em; else ++off;
+                if (pure) ++em;
                 if (c) k.cnt[i] = 0;
                 if (c > kMaxE - 2 || (pool_full && c > kSlots)) {
                     ++full;
@@ -1394,14 +1397,13 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
             }
             if (first) {
                 const int d = __reduce_add_sync(kFull, em), e = __reduce_add_sync(kFull, bad),
-                          f = __reduce_add_sync(kFull, full), hv = __reduce_add_sync(kFull, hits.halves),
-                          nf = __reduce_add_sync(kFull, off);
+                          f = __reduce_add_sync(kFull, full);
                 if (lane == 0) {
                     sm.red_i[warp][2 * kQI] = d;
                     sm.red_i[warp][2 * kQI + 1] = e;
                     sm.red_i[warp][2 * kQI + 2] = f;
-                    sm.red_i[warp][2 * kQI + 3] = hv;
-                    sm.red_i[warp][2 * kQI + 4] = nf;
+                    sm.red_i[warp][2 * kQI + 3] = warp == 0 ? sm.halves : 0;
+                    sm.red_i[warp][2 * kQI + 4] = warp == 0 ? sm.off : 0;
                 }
             }
             __syncthreads();
@@ -1522,7 +1524,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         // ---------------- accept: the owned rows of Omega+
         const T tau = tau_pow2<T>(h), tl1 = tau * lam1;
         const int par2 = par ^ 1;
-        if (tid == 0) { sm.ni = 0; sm.npl = 0; sm.sup = 0; sm.units = 0; }
+        if (tid == 0) { sm.ni = 0; sm.npl = 0; sm.sup = 0; sm.units = 0; sm.halves = 0; sm.off = 0; }
         __syncthreads();
         if (bid == 0 && tid == 0) { k.ctr[kCtrPage] = 0; k.ctr[kCtrFull] = 0; }
         // entries per row (s_rc of a long row becomes its entry count)
@@ -1617,6 +1619,7 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
                 if (lane == 0) {
                     at = atomicAdd(&sm.ni, o - rb);
                     atomicAdd(&sm.sup, row_sup(o - rb));
+                    atomicAdd(&sm.off, 1);
                 }
                 at = __shfl_sync(kFull, at, 0);
                 for (int q = lane; q < o - rb; q += 32)
