@@ -187,7 +187,9 @@ int hpc_load_x(hpc_handle h, const void* X, hpc_dtype xdt, int x_on_host);
  *    the Gram of the next hpc_load_x. Device X needs no copy.
  *  - That next hpc_load_x (of another X) then queues the staged X's panel
  *    preparation (the tensor-core Gram's transpose) on the second stream, behind
- *    its own Gram, so the preparation overlaps the solve.
+ *    its own Gram, so that it runs while the host goes on: before the solve's
+ *    iterations, or after them, or, where they run as a chain of kernels, under
+ *    them (hpc_tuning.fused_tail).
  *  - A later hpc_load_x of the staged X (same pointer and type) uses the prepared
  *    panels, or the staged copy if no Gram came in between.
  *  - Pipeline over data sets X_0, X_1, ...: hpc_prefetch_x(X_{k+1}),
@@ -218,7 +220,10 @@ int hpc_get_omega(hpc_handle h, int64_t* nnz_inout, int64_t* row_ptr, int32_t* c
 
 /* Set the iterate (warm start / resume) from a symmetric CSR with a positive
  * diagonal present in every row, columns ascending.  HPC_ERR_NONPOS_DIAG if a
- * diagonal entry is missing or <= 0; HPC_ERR_ARG if not sorted or out of range. */
+ * diagonal entry is missing or <= 0; HPC_ERR_ARG if not sorted or out of range.
+ * Symmetry is not required here; iterations from a CSR that has none run in the
+ * chain of kernels, which fail (HPC_ERR_CUDA) where an entry of the support has no
+ * partner in the candidate structure. */
 int hpc_set_omega(hpc_handle h, int64_t nnz, const int64_t* row_ptr, const int32_t* col,
                   const void* val, hpc_dtype vdt, int on_device);
 
@@ -480,8 +485,14 @@ typedef struct {
                                   decision only at an exact tie).  Where only the tail
                                   differs the two forms take the same time to within a
                                   few percent.  A cooperative kernel waits until its
-                                  whole grid is resident.  Not touched by the
-                                  autotuner.  hpc_solve_batch's single graph launch
+                                  whole grid is resident: it queues behind kernels of
+                                  other streams (hpc_prefetch_x's panel preparation
+                                  runs before or after a solve's iterations then, not
+                                  under them), and solves on several streams run one
+                                  after the other where the grid needs more than half
+                                  of the SMs.  Not touched by the autotuner, whose
+                                  ls_window, ls_blocks_per_sm and rows_ctas_per_sm
+                                  are the chain's.  hpc_solve_batch's single graph launch
                                   runs its problems' loops concurrently, always on the
                                   chain; handles solved from its worker threads keep
                                   their own setting (0)                            */

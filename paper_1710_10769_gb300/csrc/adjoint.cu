@@ -787,7 +787,7 @@ k_support_sddmm(int p, Csr<T> om, const T* __restrict__ yt, const T* __restrict_
 //        twice the gathers, which no thread waits for longer than for its own.
 //   else a grid-stride loop with T in memory and a third barrier: where the gathers are the
 //        time, they are not made twice.
-// Measured on GB300, p = 16384, 28 672 entries: 88 iterations in 1.00 ms, 11.4 us each (three
+// Measured on GB300, p = 16384, 28 672 entries: 87 iterations in 1.00 ms, 11.5 us each (three
 // kernels in a graph: about 15).
 //
 // Every wait is bounded: after CgArgs::wait_ns CgState::timeout is raised and every block leaves.

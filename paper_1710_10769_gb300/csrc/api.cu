@@ -2373,7 +2373,8 @@ int autotune_t(hpc_ctx* h, const void* X, int xdt, int on_host, int64_t iters, h
         // (the tail's form is not tuned here: the one-launch tail is a cooperative kernel,
         // which waits for the whole grid to be resident, so it queues behind work on
         // other streams, such as hpc_prefetch_x's transpose, that an iteration-only
-        // timing does not see)
+        // timing does not see.  Cov handles whose iterations run in the one-launch loop use
+        // the knobs below where the loop leaves iterations to the chain, and in batches)
         const Knob knobs[] = {{1, {2, 4, 8, 16}}, {3, {1, 2, 3, 4}}, {2, {1, 2, 3}}};
         h->chain_only = true;       // the knobs are the chain's
         for (const Knob& k : knobs) {

@@ -61,9 +61,11 @@
 // No phase of a launch is long, then, which the bounded waits need.
 //
 // Measured on GB300 (us per iteration, the chain of kernels -> this loop): 140 -> 46 at
-// p = 65536 (n = 32768), 120 -> 43 at p = 16384, 98 -> 30 at p = 1001, 220 -> 50 in FP64 at
-// p = 500; the 32-point path at p = 8192 from 169 to 54 ms.  What is left is the latency of
-// the steps' dependent loads and of the three barriers (about 2 us each).
+// p = 65536 (n = 32768), 120 -> 41 at p = 16384, 98 -> 29 at p = 1001, 220 -> 47 in FP64 at
+// p = 500; the 32-point path at p = 8192 from 163 to 52 ms.  Of the 41 us at p = 16384 the screening
+// takes 10, the build 4, the search with its decision 16, the accept 11; at the path's
+// smallest lambda1 the screening takes 200 of 310.  What is left is the latency of the steps'
+// dependent loads and of the three barriers (about 2 us each).
 //
 // Every wait is bounded (kBarrierWaitNs), after which kFlagTimeout is raised and every
 // block leaves.  The cooperative launch keeps all blocks resident (one per SM).
