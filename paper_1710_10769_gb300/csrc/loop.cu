@@ -128,7 +128,7 @@ __device__ __forceinline__ void st_ent(Ent<double>* q, unsigned cf, double om, d
 }
 
 enum : int { kFullPool = 1, kFullDense = 2 };      // bits of kCtrFull
-enum : int { kCtrPage, kCtrBig, kCtrFull, kCtrCount = 4 };
+enum : int { kCtrPage, kCtrBig, kCtrFull, kCtrStart, kCtrCount };
 
 template <typename T>
 struct LoopK {
@@ -157,7 +157,9 @@ struct LoopK {
     unsigned* mg;        // bits of max |S_ij|, i != j (rounded up)
     ulonglong2* todo;    // 2: tasks in the list, and of long rows: their number, and from bit 32 on their
                          // terms in units of 64
-    int* ctr;            // counters: pages, entries of big, full rows
+    int* ctr;            // counters: pages, entries of big, full rows (kCtrFull's bits), and whether the first
+                         // pass is too dense (a word of its own: without bounds no barrier lies between
+                         // the blocks' reads of it and the first pass's votes)
     double* part_a;      // 2 x kNA x grid
     int* part_i;         // 2 x kNI x grid
     unsigned* bar;
@@ -834,7 +836,8 @@ __device__ __forceinline__ float warp_sum_up(float x) {
 //              row of S), the chain 0.1 us per 1000 terms of all blocks of the neighbours,
 //              nbm (nnz - p), where the iterate is dense: level at half of them;
 //   support    W_ij and W_ji by gathers, up to 1.3 us per 1000 of sum n_i^2 over the rows of
-//              the block that has most, as 6 terms each: a quarter of the chain's terms;
+//              the block that has most, as 6 terms each: a quarter of the chain's terms, at most
+//              0.9 ms (a band of 2000 entries a row takes seconds: its blocks are few for the chain);
 //   search     1 us per pair of 32-entry chunks of a block's rows: level at about 500.
 // A pass that loses may be worth it (bounds that start anew keep more blocks than they do a pass
 // later, if the rows are short), so the losses add up to a debt, and the loop leaves when that
@@ -843,7 +846,7 @@ __device__ __forceinline__ float warp_sum_up(float x) {
 // (130 entries a row) 8200, 18300; p = 2000, 90 entries a row 640, 1080; a hub row of 700
 // entries at p = 700 430, 710.
 // Terms are counted by 1024 here.
-constexpr unsigned kWorkEven = 512, kWorkBlind = 1370, kSupEven = 340;
+constexpr unsigned kWorkEven = 512, kWorkBlind = 1370, kSupEven = 340, kSupMost = 4096;
 constexpr unsigned kDebtLeast = 256, kDebtMost = 1u << 16;
 constexpr int kShortMean = 32;
 constexpr int kUnitsMax = 512;
@@ -852,7 +855,7 @@ __device__ __forceinline__ int row_units(int entries) {
     const int c = (entries + 31) >> 5;
     return c * (c + 1) / 2;
 }
-__device__ __forceinline__ int row_sup(int entries) { return min(entries, 1 << 13) * min(entries, 1 << 13) >> 6; }
+__device__ __forceinline__ int row_sup(int entries) { return min(entries, 1 << 11) * min(entries, 1 << 11) >> 6; }
 __device__ __forceinline__ unsigned chain_terms(int nnz, int nbm, int p) {
     return (unsigned)((unsigned long long)nbm * (unsigned)max(0, nnz - p) >> 10);
 }
@@ -862,7 +865,7 @@ __device__ __forceinline__ bool in_debt(unsigned& debt, unsigned work, unsigned 
     return debt > min(kDebtLeast + credit, kDebtMost);
 }
 __device__ __forceinline__ bool support_debt(unsigned& debt, int sup, int nnz, int nbm, int p) {
-    return in_debt(debt, 3u * (unsigned)sup >> 3, kSupEven + chain_terms(nnz, nbm, p) / 4, 0u);
+    return in_debt(debt, 3u * (unsigned)sup >> 3, min(kSupEven + chain_terms(nnz, nbm, p) / 4, kSupMost), 0u);
 }
 // Whether to leave before a pass of many tasks (the same answer in the whole grid), and whether
 // this block leaves its support entries out, which ends the launch after the screening barrier.
@@ -1005,11 +1008,11 @@ __global__ void __launch_bounds__(kLT, 1) k_loop(LoopK<T> k) {
         unsigned d = 0u;
         sm.debt = ctrl->loop_debt;
         sm.sup_debt = 0u;
-        if (support_debt(d, sm.sup, nnz_now, k.nbm, k.p)) atomicOr(k.ctr + kCtrFull, kFullDense);
+        if (support_debt(d, sm.sup, nnz_now, k.nbm, k.p)) atomicOr(k.ctr + kCtrStart, 1);
     }
     bool alive = loop_barrier(k.bar, target, ctrl, &sm.ok);
     const float mg = __uint_as_float(__ldcg(k.mg));
-    bool dense = alive && (__ldcg(k.ctr + kCtrFull) & kFullDense) != 0;
+    bool dense = alive && __ldcg(k.ctr + kCtrStart) != 0;
     if (alive && k.bnd && !dense) {
         // the tasks of the rows of the diagonal alone; the bounds of the others, from their
         // weights
